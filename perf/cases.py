@@ -251,7 +251,9 @@ def run(s):
                              workspace=s["workspace"])
         out = ssd.ssd_verify_combine(s["stats"], c["V_llm"] * c["ranks"], s["tok_off"], s["ids"],
                                      c["tau_slm"], out=s["out"])
-        return dict({k: out[k] for k in results}, stats=s["stats"][0])
+        # a rank's (maximum, sum) pair stands for one log-sum-exp and is as good relative to any
+        # other logit of the row: what it is for comes back in row_lse and token_logp
+        return {k: out[k] for k in results}
     d = ssd.ssd_ctc_draft(s["ctc"], s["frame_off"], 0, c["cap"], out=s["draft"])
     g = ssd.ssd_entropy_gate_from_maxima(d["utt_max_entropy"], d["utt_status"], c["tau_ctc"],
                                          out=s["gate"])
@@ -268,6 +270,56 @@ def run(s):
                          v["all_accepted"], out=s["final"])
     return dict(draft={k: t for k, t in d.items() if k != "workspace"}, gate=g,
                 verify={k: v[k] for k in results}, final=f)
+
+
+def _log_sum_exp(x, entropy=False):
+    """Per row of x, in 64 bits and a gigabyte at a time: log-sum-exp and, if asked for, entropy."""
+    lse = torch.empty((x.shape[0],), dtype=torch.float64, device=x.device)
+    ent = torch.empty_like(lse) if entropy else None
+    step = max(1, (1 << 27) // x.shape[1])
+    for r in range(0, x.shape[0], step):
+        c = x[r:r + step].double()
+        top = c.amax(1)
+        c -= top[:, None]
+        e = c.exp()
+        total = e.sum(1)
+        lse[r:r + step] = top + total.log()
+        if entropy:
+            ent[r:r + step] = total.log() - (c * e).sum(1) / total
+    return lse, ent
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits, and None in the place of whole numbers."""
+    s = prepare(case, seed)
+    x = s["logits"]
+    lse, _ = _log_sum_exp(x)
+    if case["kind"] == "greedy":
+        return dict(next_token=None, next_logp=x.amax(1).double() - lse, row_lse=lse, row_status=None)
+    ids = s["ids"].long()
+    whole = dict.fromkeys(("accepted_len", "all_accepted", "utt_status"))
+    if case["kind"] == "shard":
+        here = ids < case["V_llm"]
+        mine = x.gather(1, torch.where(here, ids, 0)[:, None])[:, 0].double()
+        mine = torch.where(here, mine, -math.inf)
+        others = s["stats"][1:].double()
+        lse = torch.logsumexp(torch.cat([lse[None], others[..., 0] + others[..., 1].log()]), 0)
+        logit = torch.maximum(mine, others[..., 2].amax(0))
+        return dict(whole, token_logp=logit - lse, row_lse=lse)
+    lengths = s["frame_off"].diff()
+    frame_lse, entropy = _log_sum_exp(s["ctc"], entropy=True)
+    utterance = torch.repeat_interleave(torch.arange(len(lengths), device=x.device), lengths)
+    most = torch.zeros((len(lengths),), dtype=torch.float64, device=x.device)
+    most.scatter_reduce_(0, utterance, entropy, "amax")
+    draft = dict(dict.fromkeys(k for k in s["draft"] if k != "workspace"),
+                 frame_entropy=entropy, frame_lse=frame_lse, utt_max_entropy=most)
+    verify = dict(whole)
+    if not case["early_exit"]:
+        read = torch.repeat_interleave(most >= case["tau_ctc"], s["tok_off"].diff())
+        logp = x.gather(1, ids[:, None])[:, 0].double() - lse
+        verify.update(token_logp=torch.where(read, logp, 0.0), row_lse=torch.where(read, lse, 0.0))
+    return dict(draft=draft, gate=dict(gate_accept=None, max_entropy=most), verify=verify,
+                final=dict.fromkeys(s["final"]))
 
 
 def work(case):
