@@ -396,12 +396,13 @@ int32_t ssd_verify_combine(const float *stats_all, int32_t R, int64_t V_total,
  * whole element can (odd vocabulary sizes, column slices).  These functions replay on the host
  * the very address arithmetic those kernels use (one shared header) for a matrix that would
  * start at base_addr, over all of its tiles (ssd_ctc_draft) or rows, column spans and stage
- * parts (ssd_verify, whose streaming kernel ssd_greedy_step shares), and report
+ * parts (ssd_verify, whose streaming kernels ssd_greedy_step shares), and report
  *   lo, hi   the lowest address that would be read and one past the highest
  *   faults   how many tiles / rows break a rule: a read outside the matrix (outside the row,
  *            for ssd_verify), a bulk copy off a 16-byte boundary or larger than its stage, or
  *            reads that do not cover the tile's / row's bytes exactly once
- *   kernel   2: the bulk-copy kernel would run; 1: the plain-load kernel, which indexes
+ *   kernel   2: a kernel of wide reads would run (bulk copies, or 32-byte loads whose units
+ *            are held to the row in the same way); 1: the plain-load kernel, which indexes
  *            elements one by one (lo, hi are then the matrix's own extent)
  * so a caller -- the tests do -- can assert faults == 0, lo >= base_addr and
  * hi <= base_addr + ((rows - 1) * ld + V) * element size for any shape and misalignment.

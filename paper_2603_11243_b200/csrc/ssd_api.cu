@@ -12,6 +12,7 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
 int g_sm_count[kMaxDevices];                                   // 0: not asked yet
 std::map<std::pair<const void *, int>, size_t> g_smem_set;     // (kernel, device) -> bytes set
+std::map<std::pair<const void *, int>, int> g_carveout_set;    // (kernel, device) -> percent
 thread_local int t_replay = 0;
 }  // namespace
 
@@ -44,6 +45,21 @@ cudaError_t ensure_dynamic_smem(const void *kernel, size_t bytes) {
     return e;
 }
 
+cudaError_t ensure_l1(const void *kernel, size_t smem) {
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    // what two CTAs take (1 KB each is the system's, 1 KB for static arrays), in percent of the
+    // 228 KB that can be shared memory
+    const int percent = (int)((2 * (smem + 2048) * 100 + 228 * 1024 - 1) / (228 * 1024));
+    std::lock_guard<std::mutex> lock(g_mutex);
+    int &have = g_carveout_set[std::make_pair(kernel, dev)];
+    if (percent <= have) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
+    if (e == cudaSuccess) have = percent;
+    return e;
+}
+
 static thread_local int32_t t_last_cuda_error = 0;
 void record_cuda_error(cudaError_t e) { t_last_cuda_error = (int32_t)e; }
 static thread_local uint64_t t_launches = 0;
@@ -57,10 +73,10 @@ using namespace ssd;
 // GPU) the plan is the one for the 148-SM part the kernels are tuned for, and a launch that
 // follows fails with SSD_ERR_CUDA.
 static int plan_for_query(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts *opts,
-                          VerifyPlan *plan) {
-    if (device_sm_count() > 0) return plan_verify(B, M, V, dtype, opts, plan);
+                          VerifyPlan *plan, const RowsAt &at) {
+    if (device_sm_count() > 0) return plan_verify(B, M, V, dtype, opts, at, plan);
     PlanReplay replay;
-    return plan_verify(B, M, V, dtype, opts, plan);
+    return plan_verify(B, M, V, dtype, opts, at, plan);
 }
 
 extern "C" {
@@ -98,7 +114,7 @@ size_t ssd_verify_workspace_bytes(int32_t B, int64_t M, int32_t V, ssd_dtype dty
                                   const ssd_launch_opts *opts) {
     if (B < 0 || M < 0 || V < 1 || (dtype != SSD_F32 && dtype != SSD_BF16)) return 0;
     VerifyPlan plan;
-    if (plan_for_query(B, M, V, dtype, opts, &plan) != SSD_OK) return 0;
+    if (plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{nullptr, V, false}) != SSD_OK) return 0;
     return plan.workspace_bytes;
 }
 
@@ -170,7 +186,7 @@ int32_t ssd_verify(const void *logits, ssd_dtype dtype, int32_t V, int64_t ld,
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V, dtype, opts, &plan);
+    int rc = plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{logits, ld, false});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < plan.workspace_bytes ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))
@@ -192,7 +208,7 @@ int32_t ssd_verify_shard(const void *logits, ssd_dtype dtype, int32_t V_local, i
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V_local, dtype, opts, &plan);
+    int rc = plan_for_query(B, M, V_local, dtype, opts, &plan, RowsAt{logits, ld, false});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < plan.workspace_bytes ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))
@@ -252,7 +268,7 @@ size_t ssd_verify_early_exit_workspace_bytes(int32_t B, int64_t M, int32_t V, ss
                                              const ssd_launch_opts *opts) {
     if (B < 0 || M < 0 || V < 1 || (dtype != SSD_F32 && dtype != SSD_BF16)) return 0;
     VerifyPlan plan;
-    if (plan_for_query(B, M, V, dtype, opts, &plan) != SSD_OK) return 0;
+    if (plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{nullptr, V, false}) != SSD_OK) return 0;
     return verify_ee_workspace_bytes(B, plan);
 }
 
@@ -272,7 +288,7 @@ int32_t ssd_verify_early_exit(const void *logits, ssd_dtype dtype, int32_t V, in
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V, dtype, opts, &plan);
+    int rc = plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{logits, ld, false});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < verify_ee_workspace_bytes(B, plan) ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))
@@ -298,7 +314,7 @@ size_t ssd_greedy_step_workspace_bytes(int64_t R, int32_t V, ssd_dtype dtype,
                                        const ssd_launch_opts *opts) {
     if (R < 0 || V < 1 || (dtype != SSD_F32 && dtype != SSD_BF16)) return 0;
     VerifyPlan plan;
-    if (plan_for_query(0, R, V, dtype, opts, &plan) != SSD_OK) return 0;
+    if (plan_for_query(0, R, V, dtype, opts, &plan, RowsAt{nullptr, V, true}) != SSD_OK) return 0;
     return greedy_workspace_bytes(R, plan);
 }
 
@@ -312,7 +328,7 @@ int32_t ssd_greedy_step(const void *logits, ssd_dtype dtype, int32_t V, int64_t 
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(0, R, V, dtype, opts, &plan);
+    int rc = plan_for_query(0, R, V, dtype, opts, &plan, RowsAt{logits, ld, true});
     if (rc != SSD_OK) return rc;
     if (plan.kernel != 2) return SSD_ERR_ARG;
     if (R > 0 && (!workspace || workspace_bytes < greedy_workspace_bytes(R, plan) ||

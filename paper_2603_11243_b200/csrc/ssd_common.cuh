@@ -39,6 +39,14 @@ __device__ __forceinline__ void pdl_enter() {
     pdl_wait();
 }
 
+// Asks for the L1-heavy split of an SM's memory, once per kernel and device (again only if a
+// launch needs more shared memory than any before it).  Without a wish a kernel keeps the split
+// it finds, and one that is scheduled behind a bulk-copy kernel finds 28 KB of L1: the direct
+// loads of verify_rows_direct, whose data in flight lie in L1, then ran at 0.8 of their speed on
+// those SMs.  Every kernel without a ring asks, since the split can only change on an idle SM.
+constexpr size_t kSmallSmem = 16 * 1024;
+cudaError_t ensure_l1(const void *kernel, size_t smem);
+
 void count_launch();     // one more kernel launched by this host thread (ssd_launch_count)
 
 template <typename... KArgs, typename... Args>
@@ -55,6 +63,10 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     count_launch();
+    if (smem <= kSmallSmem) {
+        const cudaError_t e = ensure_l1(reinterpret_cast<const void *>(kernel), smem);
+        if (e != cudaSuccess) return e;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
@@ -247,6 +259,11 @@ __device__ __forceinline__ uint32_t bf16x2_max_nan(uint32_t a, uint32_t b) {
     asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
+__device__ __forceinline__ uint32_t bf16x2_min_nan(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("min.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
 __device__ __forceinline__ float fmax_nan(float a, float b) {
     float d;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
@@ -279,6 +296,28 @@ __device__ __forceinline__ float2 exp2_fma_pair(float2 t) {
     float2 y;
     y.x = __int_as_float(__float_as_int(r.x) * (1 << 23) + __float_as_int(p.x));
     y.y = __int_as_float(__float_as_int(r.y) * (1 << 23) + __float_as_int(p.y));
+    return y;
+}
+
+// 2^t for a pair on the FMA pipe, for t already known to be >= -126 (the caller clamps the
+// logits from below) and not checked from above (the caller clamps them, or tests its largest
+// exponent once per row): nearest integer n by the 1.5*2^23 trick, a degree-5 polynomial for 2^f
+// on f = t - n in [-1/2, 1/2] (least maximum relative error, by Remez's exchange; 2.1e-7 in fp32,
+// as good as ex2.approx), n added into the exponent field.
+__device__ __forceinline__ float2 exp2_fma_pair_inrange(float2 t) {
+    const float kMagic = 12582912.f;
+    const float2 r = fadd2(t, make_float2(kMagic, kMagic));
+    const float2 n = fadd2(r, make_float2(-kMagic, -kMagic));
+    const float2 f = ffma2(n, make_float2(-1.f, -1.f), t);
+    float2 q = make_float2(0.0013276472454890609f, 0.0013276472454890609f);
+    q = ffma2(q, f, make_float2(0.0096755409613251686f, 0.0096755409613251686f));
+    q = ffma2(q, f, make_float2(0.055507130920886993f, 0.055507130920886993f));
+    q = ffma2(q, f, make_float2(0.24022120237350464f, 0.24022120237350464f));
+    q = ffma2(q, f, make_float2(0.69314694404602051f, 0.69314694404602051f));
+    q = ffma2(q, f, make_float2(1.0f, 1.0f));
+    float2 y;
+    y.x = __int_as_float(__float_as_int(r.x) * (1 << 23) + __float_as_int(q.x));
+    y.y = __int_as_float(__float_as_int(r.y) * (1 << 23) + __float_as_int(q.y));
     return y;
 }
 
@@ -410,12 +449,22 @@ struct VerifyPlan {
     int fma_exp;       // pairs per chunk whose exponential runs on the FMA pipe (bf16 only)
     int partials;      // partial (max, sum) pairs per row = split * warps
     int finish_inside; // rows are finalised inside the streaming kernel (no closing kernel)
+    int direct;        // rows are streamed by the direct-load kernel
+    int spans;         // direct-load kernel: column spans per row, one warp and one pair each
+    int span_blocks;   // direct-load kernel: blocks per span
+    int direct_ctas;
     size_t smem_bytes;
     size_t fin_smem_bytes;
     size_t workspace_bytes;
 };
+// Where the rows of a call lie and what they are read for; scratch sizes do not depend on it.
+struct RowsAt {
+    const void *base;
+    int64_t ld;
+    bool greedy;
+};
 int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts *opts,
-                VerifyPlan *plan);
+                const RowsAt &at, VerifyPlan *plan);
 int launch_verify_shard(const void *logits, ssd_dtype dtype, int V_local, int64_t ld, int64_t M,
                         int64_t col0, const int64_t *tok_off, const int32_t *draft_ids, int B,
                         const uint8_t *skip, void *workspace, float *shard_stats,

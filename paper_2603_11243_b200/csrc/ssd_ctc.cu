@@ -231,26 +231,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-// 2^t for a pair on the FMA pipe, for t already known to be >= -126 (the caller clamps the
-// logits from below) and not checked from above (the caller tests its largest exponent once
-// per row): nearest integer n by the 1.5*2^23 trick, a degree-4 polynomial for 2^f on
-// f = t - n in [-1/2, 1/2] (relative error 3.6e-6), n added into the exponent field.
-__device__ __forceinline__ float2 exp2_fma_pair_inrange(float2 t) {
-    const float kMagic = 12582912.f;
-    const float2 r = fadd2(t, make_float2(kMagic, kMagic));
-    const float2 n = fadd2(r, make_float2(-kMagic, -kMagic));
-    const float2 f = ffma2(n, make_float2(-1.f, -1.f), t);
-    float2 q = make_float2(0.00966636836528778f, 0.00966636836528778f);
-    q = ffma2(q, f, make_float2(0.055921975523233414f, 0.055921975523233414f));
-    q = ffma2(q, f, make_float2(0.2402234971523285f, 0.2402234971523285f));
-    q = ffma2(q, f, make_float2(0.6931210160255432f, 0.6931210160255432f));
-    q = ffma2(q, f, make_float2(1.0f, 1.0f));
-    float2 y;
-    y.x = __int_as_float(__float_as_int(r.x) * (1 << 23) + __float_as_int(q.x));
-    y.y = __int_as_float(__float_as_int(r.y) * (1 << 23) + __float_as_int(q.y));
-    return y;
-}
-
 // S += 2^t, A += t*2^t over one chunk (t = x*log2e + nrh) and the running maximum with the
 // chunk it was first met in.  With kF, that many of a bf16 chunk's four pairs take the FMA-pipe
 // exponential; `floor2` is then a packed pair of a bf16 value below which those logits are

@@ -1,0 +1,384 @@
+// verify_rows_direct: the streaming kernel of ssd_verify, ssd_verify_shard and ssd_greedy_step
+// for bf16 logits (use_direct in ssd_verify.cu says where it runs and what it measured against
+// the ring of verify_rows_tma).
+//
+// A warp works on one span of columns of one row at a time and reads it with 32-byte loads
+// straight into registers: no shared memory, no barriers, no hand-over between warps.  What
+// bounds it on long batches is the 1 kW power cap (a kernel that only reads takes 611 us for 4.4
+// GB there, the ring 710, this one 665), so what counts is instructions per logit: 4.8 against
+// 6.0 of the ring.  148 x 32 warps keep up to two blocks of 1 KB each in flight, the block loop
+// holds nothing but the loads, the sums and a counter, and everything that happens once per span
+// (reference, range check, merge of the lanes) is done once for the warp instead of once per
+// thread.  More in flight was slower throughout (two units a lane and block: +3 %; 48 warps: +18
+// %; bulk prefetch to L2: +3 % and more), and so were blocks interleaved among warps.
+#pragma once
+
+#include "ssd_common.cuh"
+#include "ssd_ranges.cuh"
+#include "ssd_stream.cuh"
+
+namespace ssd {
+namespace direct {
+
+using ranges::kDirectBlockBytes;
+
+constexpr int kThreads = 512, kWarps = kThreads / 32, kCtasPerSm = 2;
+constexpr float kSpanSumLimit = 1.0e27f;   // below every value a clamped exponential can take
+
+struct DirectParams {
+    const char *logits;
+    int V;
+    int64_t row_pitch;
+    int row_bytes;
+    int64_t M;
+    int spans, span_blocks;   // column spans per row, blocks per span (see plan_spans)
+    const int64_t *tok_off;
+    int B;
+    const uint8_t *skip;
+    int table;             // count the rows to read per utterance in shared memory first
+    void *partials;        // [M, spans] float2 (reference, sum), or float4 with the arg max
+};
+
+// One lane's 32-byte piece of a block.
+struct Unit {
+    uint32_t r[8];
+};
+__device__ __forceinline__ Unit load_unit(const char *p) {
+    Unit v;
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v.r[0]), "=r"(v.r[1]), "=r"(v.r[2]), "=r"(v.r[3]), "=r"(v.r[4]),
+                   "=r"(v.r[5]), "=r"(v.r[6]), "=r"(v.r[7])
+                 : "l"(p));
+    return v;
+}
+
+template <typename T> __device__ __forceinline__ float unit_max(const Unit &v) {
+    const uint4 a = make_uint4(v.r[0], v.r[1], v.r[2], v.r[3]);
+    const uint4 b = make_uint4(v.r[4], v.r[5], v.r[6], v.r[7]);
+    if (Elem<T>::kBytes == 4) return fmaxf(chunk_max<float>(a), chunk_max<float>(b));
+    const uint32_t h = bf16x2_max(bf16x2_max(bf16x2_max(a.x, a.y), bf16x2_max(a.z, a.w)),
+                                  bf16x2_max(bf16x2_max(b.x, b.y), bf16x2_max(b.z, b.w)));
+    return fmaxf(bf16_lo(h), bf16_hi(h));
+}
+
+// What a span's exponentials are taken relative to: one logit m of the warp's first block, as
+// nmh = -fl(m * log2e), and for the FMA-pipe exponential a floor and a ceiling around m as
+// packed bf16 pairs.  They are rounded towards m, so that with |m| < 4096 (a bf16 step of at
+// most 16) both stay within [69, 85] of it: the floor's exponential is below 2^-99, the
+// ceiling's between 2^99 and 2^123, which the span's range check sees.
+struct Reference {
+    float m, nmh;
+    uint32_t floor2 = 0, ceil2 = 0;
+    template <typename T> __device__ __forceinline__ void set(float to) {
+        m = to;
+        nmh = -(to * kLog2e);
+        if (Elem<T>::kBytes == 2) {
+            uint32_t lo = __float_as_uint(to - 85.f), hi = __float_as_uint(to + 85.f);
+            lo += (lo & 0x80000000u) ? 0u : 0xffffu;
+            hi += (hi & 0x80000000u) ? 0xffffu : 0u;
+            floor2 = (lo >> 16) * 0x10001u;
+            ceil2 = (hi >> 16) * 0x10001u;
+        }
+    }
+};
+
+// kF of a bf16 unit's eight pairs take the FMA-pipe exponential.  The unit's terms are summed
+// apart and join the lane's sums once: a span with one logit far above the rest leaves large
+// values in a sum, and a thousand small terms added to that one by one would each lose the same
+// fraction of an ulp.
+template <typename T, int kF>
+__device__ __forceinline__ void add_unit(const Unit &v, const Reference &ref, float2 &Sa, float2 &Sb) {
+    const float2 sc = make_float2(kLog2e, kLog2e), nm = make_float2(ref.nmh, ref.nmh);
+    float2 ta, tb;
+    if (Elem<T>::kBytes == 4) {
+        float2 e[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            e[k] = stream::exp2_pair(make_float2(__uint_as_float(v.r[2 * k]), __uint_as_float(v.r[2 * k + 1])), sc, nm);
+        ta = fadd2(e[0], e[2]);
+        tb = fadd2(e[1], e[3]);
+    } else {
+        float2 e[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if ((kF >= 1 && k == 0) || (kF >= 2 && k == 4)) {
+                const uint32_t w = bf16x2_min_nan(bf16x2_max_nan(v.r[k], ref.floor2), ref.ceil2);
+                e[k] = exp2_fma_pair_inrange(ffma2(make_float2(bf16_lo(w), bf16_hi(w)), sc, nm));
+            } else {
+                e[k] = stream::exp2_pair(make_float2(bf16_lo(v.r[k]), bf16_hi(v.r[k])), sc, nm);
+            }
+        }
+        ta = fadd2(fadd2(e[0], e[2]), fadd2(e[4], e[6]));
+        tb = fadd2(fadd2(e[1], e[3]), fadd2(e[5], e[7]));
+    }
+    Sa = fadd2(Sa, ta);
+    Sb = fadd2(Sb, tb);
+}
+
+// A span whose sums left fp32's range, or whose first block holds no finite logit to refer to
+// (masked logits, NaN, +inf, a magnitude beyond 4096): two passes over its elements.
+struct SpanResult {
+    float m, S, vmax;
+    int vidx;
+};
+template <typename T>
+__device__ __noinline__ SpanResult span_exact(const DirectParams &p, int64_t row, int sp, int lane) {
+    constexpr int ES = Elem<T>::kBytes;
+    const char *x = p.logits + row * p.row_pitch;
+    const ranges::RowUnits ru = ranges::row_units(reinterpret_cast<uintptr_t>(x), p.row_bytes);
+    const ranges::UnitSpan us = ranges::unit_span(ru, p.spans, sp, p.span_blocks);
+    const int n = (us.hi - us.lo) / ES, first = us.lo / ES;
+    x += us.lo;
+    SpanResult r;
+    r.vmax = -INFINITY;
+    r.vidx = INT_MAX;
+    for (int i = lane; i < n; i += 32) {
+        const float v = Elem<T>::load(x + (size_t)i * ES);
+        if (v > r.vmax) { r.vmax = v; r.vidx = first + i; }
+    }
+    const float vm = warp_max(r.vmax);
+    r.vidx = __reduce_min_sync(0xffffffffu, r.vmax == vm ? r.vidx : INT_MAX);
+    r.vmax = r.m = vm;
+    float S = 0.f;
+    if (vm > -INFINITY) {
+        // (x - vm) * log2e, not x * log2e - vm * log2e: a mask of the type's lowest value would
+        // leave fp32's range there
+        for (int i = lane; i < n; i += 32) S += ex2((Elem<T>::load(x + (size_t)i * ES) - vm) * kLog2e);
+        S = warp_sum(S);
+    } else {
+        // only -inf adds nothing; NaN has to show
+        for (int i = lane; i < n; i += 32) {
+            const float v = Elem<T>::load(x + (size_t)i * ES);
+            if (v != v) S = v;
+        }
+        S = warp_sum(S);
+    }
+    r.S = S;
+    return r;
+}
+
+inline int row_blocks(int64_t row_bytes) {
+    const int64_t nb = (row_bytes + kDirectBlockBytes - 1) / kDirectBlockBytes;
+    return nb > 0 ? (int)nb : 1;
+}
+
+// Where a warp is in the rows it has to read.  With `skip`, the rows of utterances that are not
+// read are left out of the count (act: rows to read before utterance b), so that the others are
+// dealt out evenly whatever is skipped; with more utterances or rows than the table takes
+// (table_fits), skipped rows are passed over one by one.
+struct Cursor {
+    int a;             // index among the rows to read
+    int sp, b;
+    int shift;         // row - a, for the rows of utterance b
+    int row;
+    bool valid;
+};
+
+template <typename T, int kF, bool kArg>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const DirectParams p) {
+    constexpr int ES = Elem<T>::kBytes;
+    extern __shared__ int32_t act[];
+    __shared__ int32_t warp_tot[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool table = p.table != 0;
+    pdl_launch_dependents();
+    pdl_wait();
+    int rows = (int)p.M;
+    if (table) {
+        const int per = (p.B + kThreads - 1) / kThreads, b0 = (int)threadIdx.x * per;
+        int32_t mine = 0;
+        for (int b = b0; b < min(p.B, b0 + per); ++b) {
+            const int64_t i0 = p.tok_off[b], i1 = p.tok_off[b + 1];
+            act[b] = mine;
+            if (!(i0 < 0 || i1 < i0 || i1 > p.M || p.skip[b])) mine += (int32_t)(i1 - i0);
+        }
+        int32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) warp_tot[warp] = incl;
+        __syncthreads();
+        int32_t before = incl - mine, total = 0;
+        for (int w = 0; w < kWarps; ++w) {
+            const int32_t t = warp_tot[w];
+            if (w < warp) before += t;
+            total += t;
+        }
+        rows = total;
+        for (int b = b0; b < min(p.B, b0 + per); ++b) act[b] += before;
+        if (threadIdx.x == 0) act[p.B] = total;
+        __syncthreads();
+    }
+
+    // item k of warp w is number w + k * (warps of the grid) of the rows * spans items, counted
+    // so that neighbours go to different CTAs
+    const unsigned gw = blockIdx.x + gridDim.x * warp, GW = gridDim.x * kWarps;
+    const int da = (int)(GW / (unsigned)p.spans), ds = (int)(GW % (unsigned)p.spans);
+    Cursor cur;
+    cur.a = (int)(gw / (unsigned)p.spans);
+    cur.sp = (int)(gw % (unsigned)p.spans);
+    cur.b = -1;
+    cur.shift = 0;
+    int b_end = 0;                       // rows to read up to and with utterance b
+    auto step = [&]() {
+        cur.a += da; cur.sp += ds;
+        if (cur.sp >= p.spans) { cur.sp -= p.spans; ++cur.a; }
+    };
+    auto settle = [&]() {
+        if (table) {
+            cur.valid = cur.a < rows;
+            if (cur.valid && cur.a >= b_end) {
+                do b_end = act[++cur.b + 1]; while (b_end <= cur.a);
+                cur.shift = (int)p.tok_off[cur.b] - act[cur.b];
+            }
+            cur.row = cur.a + cur.shift;
+            return;
+        }
+        for (;;) {
+            cur.valid = cur.a < rows;
+            cur.row = cur.a;
+            if (!cur.valid || !p.skip) return;
+            const int b = utterance_of_row(p.tok_off, p.B, cur.row);
+            if (b < 0 || !p.skip[b]) return;
+            step();
+        }
+    };
+    settle();
+    if (!cur.valid) return;
+
+    // the span the cursor stands on: this lane's address in its first block, blocks, bytes of
+    // the last block from this lane's unit on, the element this lane has of the row's two edges
+    const char *at;
+    int blocks, rest, edge_idx = 0, unit_elem = 0;
+    float edge;
+    auto open = [&]() {
+        const char *x = p.logits + (int64_t)cur.row * p.row_pitch;
+        const ranges::RowUnits ru = ranges::row_units(reinterpret_cast<uintptr_t>(x), p.row_bytes);
+        const ranges::UnitSpan us = ranges::unit_span(ru, p.spans, cur.sp, p.span_blocks);
+        const int bytes = us.uhi - us.ulo;
+        at = x + us.ulo + lane * 32;
+        blocks = (bytes + kDirectBlockBytes - 1) / kDirectBlockBytes;
+        if (blocks < 1) blocks = 1;
+        rest = bytes - (blocks - 1) * kDirectBlockBytes - lane * 32;
+        const int e = lane < 16 ? us.lo + lane * ES : us.uhi + (lane - 16) * ES;
+        edge = -INFINITY;
+        if (e < (lane < 16 ? us.ulo : us.hi)) edge = Elem<T>::load(x + e);
+        if (kArg) {
+            edge_idx = e / ES;
+            unit_elem = us.ulo / ES + lane * (32 / ES);
+        }
+    };
+    auto load_next = [&](Unit &d) { d = load_unit(at); at += kDirectBlockBytes; };
+    auto load_last = [&](Unit &d) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) d.r[k] = Elem<T>::kNegInfBits;
+        if (rest > 0) d = load_unit(at);
+    };
+
+    Unit u, v;
+    open();
+    if (blocks > 1) load_next(u); else load_last(u);
+    for (;;) {
+        Reference ref;
+        const int64_t slot = (int64_t)cur.row * p.spans + cur.sp;
+        const float my_edge = edge;
+        const int my_edge_idx = edge_idx, my_unit_elem = unit_elem;
+        float vmax = -INFINITY, Sw = 0.f;
+        int vblk = 0;
+        float2 Sa = make_float2(0.f, 0.f), Sb = Sa;
+        ref.set<T>(warp_max(fmaxf(unit_max<T>(u), my_edge)));
+        bool fast = fabsf(ref.m) < 4096.f;
+        int k = fast ? blocks - 1 : 0;      // blocks that follow the one in u
+        auto add = [&](const Unit &d, int blk) {
+            if (kArg) {
+                const float m = unit_max<T>(d);
+                if (m > vmax) { vmax = m; vblk = blk; }
+            }
+            add_unit<T, kF>(d, ref, Sa, Sb);
+        };
+#pragma unroll 1
+        for (; k > 2; k -= 2) {
+            load_next(v);
+            add(u, blocks - 1 - k);
+            load_next(u);
+            add(v, blocks - k);
+        }
+        if (k == 2) {
+            load_next(v);
+            add(u, blocks - 3);
+            load_last(u);
+            add(v, blocks - 2);
+        } else if (k == 1) {
+            load_last(v);
+            add(u, blocks - 2);
+            u = v;
+        }
+        const int last = blocks - 1;
+        // the next span's first block is on its way before this span is finished
+        step();
+        settle();
+        if (cur.valid) {
+            open();
+            if (blocks > 1) load_next(v); else load_last(v);
+        }
+        if (fast) {
+            add(u, last);
+            Sw = warp_sum((Sa.x + Sa.y) + (Sb.x + Sb.y) + ex2(fmaf(my_edge, kLog2e, ref.nmh)));
+            fast = Sw < kSpanSumLimit;
+            Sw *= ex2(-fmaf(ref.m, kLog2e, ref.nmh));   // every exponent carried m*log2e + nmh
+        }
+        SpanResult out;
+        if (fast) {
+            out.m = ref.m;
+            out.S = Sw;
+            if (kArg) {
+                // a lane's maximum is known to a unit: its first element stands for it, and the
+                // closing kernel looks the position up
+                out.vmax = warp_max(fmaxf(vmax, my_edge));
+                int idx = INT_MAX;
+                if (my_edge == out.vmax && my_edge > -INFINITY) idx = my_edge_idx;
+                if (vmax == out.vmax && vmax > -INFINITY)
+                    idx = min(idx, my_unit_elem + vblk * (kDirectBlockBytes / ES));
+                out.vidx = __reduce_min_sync(0xffffffffu, idx);
+            }
+        } else {
+            out = span_exact<T>(p, slot / p.spans, (int)(slot % p.spans), lane);
+        }
+        if (lane == 0) {
+            if (kArg) reinterpret_cast<float4 *>(p.partials)[slot] =
+                make_float4(out.m, out.S, out.vmax, __int_as_float(out.vidx));
+            else reinterpret_cast<float2 *>(p.partials)[slot] = make_float2(out.m, out.S);
+        }
+        if (!cur.valid) return;
+        u = v;
+    }
+}
+
+inline bool table_fits(int B, int64_t M) {
+    // a malformed list of offsets may name a row more than once: B * M bounds the count
+    return B + 1 <= stream::kOffCacheMax && (B + 1) * M < (1ll << 31);
+}
+
+// Column spans per row.  All warps of the grid get the same number of spans (plus or minus one),
+// so the time goes with the number of rounds times the blocks of a span, and a span costs about
+// three blocks' worth of instructions of its own (reference, merge, the next span's addresses).
+// (A finer cut of the rows that do not fill a round, so that every warp gets the same bytes, was
+// slower throughout: 22.4 against 21.1 us on 250 rows of 304 KB, 95 against 93.5 on 5,568 of 98.)
+inline void plan_spans(int64_t M, int64_t row_bytes, int warps, int most, int *spans, int *span_blocks) {
+    const int64_t nb = row_blocks(row_bytes);
+    int64_t best = 0;
+    for (int rounds = 1; rounds <= 16; ++rounds) {
+        int64_t ns = M > 0 ? (int64_t)rounds * warps / M : 1;
+        ns = ns < 1 ? 1 : ns > most ? most : ns;
+        const int64_t bps = (nb + ns - 1) / ns;
+        ns = (nb + bps - 1) / bps;
+        const int64_t cost = (M * ns + warps - 1) / warps * (bps + 3);
+        if (best == 0 || cost < best) { best = cost; *span_blocks = (int)bps; *spans = (int)ns; }
+        if (M > 0 && (int64_t)rounds * warps / M >= most) break;
+    }
+}
+
+}  // namespace direct
+}  // namespace ssd

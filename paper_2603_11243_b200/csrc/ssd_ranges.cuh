@@ -127,5 +127,37 @@ SSD_HD PartReads part_reads(const RowGeom &g, int pc0, int pc1) {
     return r;
 }
 
+// ---- verification / greedy step by direct loads: a row is 32-byte units and two edges --------
+// Units are the 32-byte-aligned pieces that lie wholly inside the row; what is left at its two
+// ends is less than a unit each and is read element by element.  A row without a whole unit
+// inside may be all head.  Everything is in bytes from the row's start (rows under 1 GB).
+constexpr int kDirectBlockBytes = 1024;      // what a warp reads at a time: a unit per lane
+struct RowUnits {
+    int head, units, row;      // head [0, head), units [head, head + units), tail up to row
+};
+SSD_HD RowUnits row_units(uintptr_t row_start, int row_bytes) {
+    RowUnits r;
+    r.row = row_bytes;
+    r.head = (int)(0u - (uint32_t)row_start) & 31;
+    if (r.head > row_bytes) r.head = row_bytes;
+    r.units = (row_bytes - r.head) & ~31;
+    return r;
+}
+
+// Span sp of ns: the units of blocks [sp * per_span, (sp + 1) * per_span) that the row has,
+// [ulo, uhi), with the head for the first span and the tail for the last one: [lo, hi).
+struct UnitSpan {
+    int lo, ulo, uhi, hi;
+};
+SSD_HD UnitSpan unit_span(const RowUnits &r, int ns, int sp, int per_span) {
+    UnitSpan s;
+    const int from = sp * (per_span * kDirectBlockBytes), to = from + per_span * kDirectBlockBytes;
+    s.ulo = r.head + (from < r.units ? from : r.units);
+    s.uhi = r.head + (to < r.units ? to : r.units);
+    s.lo = sp == 0 ? 0 : s.ulo;
+    s.hi = sp == ns - 1 ? r.row : s.uhi;
+    return s;
+}
+
 }  // namespace ranges
 }  // namespace ssd

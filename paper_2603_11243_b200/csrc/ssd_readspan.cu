@@ -1,4 +1,4 @@
-// Host-side replay of the bulk-copy kernels' address arithmetic (ssd_ranges.cuh): for a logits
+// Host-side replay of the streaming kernels' address arithmetic (ssd_ranges.cuh): for a logits
 // matrix that would start at a given address, which bytes would be read, do the reads of every
 // tile / row part cover its bytes exactly, and do they stay inside the matrix and the stage.
 // Nothing is dereferenced and no GPU is needed; the tests sweep shapes and misalignments.
@@ -95,12 +95,31 @@ int32_t ssd_verify_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, int
     if (base_addr % es) return SSD_ERR_ALIGN;
     PlanReplay replay;
     VerifyPlan plan;
-    const int rc = plan_verify(B, M, V, dtype, opts, &plan);
+    const int rc = plan_verify(B, M, V, dtype, opts,
+                               RowsAt{reinterpret_cast<const void *>((uintptr_t)base_addr), ld, false}, &plan);
     if (rc != SSD_OK) return rc;
     const int64_t row_pitch = ld * es, row_bytes = (int64_t)V * es;
     const uintptr_t base = (uintptr_t)base_addr;
     Span sp;
-    if (plan.kernel == 2) {
+    if (plan.direct) {
+        for (int64_t row = 0; row < M; ++row) {
+            const uintptr_t g0 = base + (uintptr_t)(row * row_pitch);
+            const ranges::RowUnits r = ranges::row_units(g0, (int)row_bytes);
+            bool ok = r.units == 0 || (g0 + (uintptr_t)r.head) % 32 == 0;
+            ok = ok && r.head >= 0 && r.head < 32 && r.units % 32 == 0;
+            ok = ok && r.row - r.head - r.units >= 0 && r.row - r.head - r.units < 32;
+            int at = 0;                // the spans must tile the row in order
+            for (int s = 0; s < plan.spans; ++s) {
+                const ranges::UnitSpan c = ranges::unit_span(r, plan.spans, s, plan.span_blocks);
+                ok = ok && c.lo == at && c.ulo >= c.lo && c.uhi >= c.ulo && c.hi >= c.uhi;
+                ok = ok && c.ulo - c.lo < 32 && c.hi - c.uhi < 32 && (c.uhi - c.ulo) % 32 == 0;
+                sp.add(g0 + (uintptr_t)c.lo, g0 + (uintptr_t)c.hi);
+                at = c.hi;
+            }
+            ok = ok && at == r.row;
+            if (!ok) ++sp.faults;
+        }
+    } else if (plan.kernel == 2) {
         const int max_chunks = plan.stage_bytes >> 4;
         for (int64_t row = 0; row < M; ++row) {
             const ranges::RowGeom g = ranges::row_geom(base, row, row_pitch, row_bytes);

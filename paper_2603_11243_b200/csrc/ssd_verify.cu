@@ -12,16 +12,19 @@
 //                      2^((x-m)*log2e) relative to a reference logit m of its own and checks
 //                      once per stage that the sum stayed in range (see Online), so the common
 //                      case is one exponential and no comparison per logit.
+//   verify_rows_direct (ssd_direct.cuh) a warp per column span of a row, 32-byte loads into
+//                      registers; what runs by default where it is faster (see use_direct).
 //   verify_rows_plain  one CTA per item with scalar global loads; any alignment.  Fallback.
 //
-// The same streaming kernel with a running arg max serves the greedy decoding step (Eq. 6),
+// The same streaming kernels with a running arg max serve the greedy decoding step (Eq. 6),
 // and with a closing kernel that leaves (maximum, sum, draft logit) per row instead of the
-// decision it serves an LLM head whose columns are split over several ranks (ssd_verify_shard,
+// decision they serve an LLM head whose columns are split over several ranks (ssd_verify_shard,
 // ssd_verify_combine).
 #include <limits.h>
 #include <math.h>
 
 #include "ssd_common.cuh"
+#include "ssd_direct.cuh"
 #include "ssd_ranges.cuh"
 #include "ssd_stream.cuh"
 
@@ -226,28 +229,42 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
 }
 
 
-// Merge of a row's P (reference, sum) pairs into (maximum, sum relative to it).
-__device__ __forceinline__ float2 merge_partials(const float2 *pp, int P) {
+// Merge of a row's P (reference, sum) pairs into (maximum, sum relative to it) by the G lanes of
+// a group, lane `sub` of which takes pairs sub, sub + G, ...  All 32 lanes of the warp call it.
+template <int G> __device__ __forceinline__ float2 merge_partials(const float2 *pp, int P, int sub) {
     float Mx = kNegInit, S = 0.f;
-    if ((P & 1) == 0 && P <= 16) {
-        const float4 *p4 = reinterpret_cast<const float4 *>(pp);
-        float4 v[8];
+    if (P <= 4 * G) {
+        float2 v[4];                      // all of a lane's pairs are fetched together
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            v[q] = q < P / 2 ? p4[q] : make_float4(kNegInit, 0.f, kNegInit, 0.f);
+        for (int j = 0; j < 4; ++j) {
+            v[j] = make_float2(kNegInit, 0.f);
+            if (sub + j * G < P) v[j] = pp[sub + j * G];
+        }
+        Mx = fmaxf(fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)), kNegInit);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) Mx = fmaxf(Mx, fmaxf(v[q].x, v[q].z));
+        for (int o = G / 2; o > 0; o >>= 1) Mx = fmaxf(Mx, __shfl_xor_sync(0xffffffffu, Mx, o));
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            S += v[q].y * ex2((v[q].x - Mx) * kLog2e) + v[q].w * ex2((v[q].z - Mx) * kLog2e);
+        for (int j = 0; j < 4; ++j) S += v[j].y * ex2((v[j].x - Mx) * kLog2e);
     } else {
-        for (int q = 0; q < P; ++q) Mx = fmaxf(Mx, pp[q].x);
-        for (int q = 0; q < P; ++q) {
+        for (int q = sub; q < P; q += G) Mx = fmaxf(Mx, pp[q].x);
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) Mx = fmaxf(Mx, __shfl_xor_sync(0xffffffffu, Mx, o));
+        for (int q = sub; q < P; q += G) {
             const float2 v = pp[q];
             S += v.y * ex2((v.x - Mx) * kLog2e);
         }
     }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
     return make_float2(Mx, S);
+}
+
+// Lanes that share a row's pairs: four pairs a lane, so that their loads are one round trip.
+// (A thread that walked 36 pairs of a row by itself, twice, took 10 us for a draft of 250 tokens.)
+inline int merge_lanes(int P) {
+    int G = 1;
+    while (G < 32 && 4 * G < P) G *= 2;
+    return G;
 }
 
 // Eq. 5 for one row, given its maximum Mx, ln of its sum of exponentials relative to Mx and the
@@ -605,7 +622,7 @@ __global__ void __launch_bounds__(256) verify_rows_plain(const VerifyParams p) {
 
 constexpr int kFinishThreads = 1024;   // one sweep for drafts of up to 1024 tokens
 
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
     const char *__restrict__ logits, int V, int64_t ld, int64_t M,
     const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
@@ -643,20 +660,28 @@ __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
     __syncthreads();
     unsigned myflags = 0;
     int myfirst = K;
-    for (int i = tid; i < K; i += blockDim.x) {
-        const int64_t r = i0 + i;
-        const int id = draft_ids[r];
-        const bool id_ok = id >= 0 && id < V;
-        // the row's partials and the draft token's logit are fetched together
+    const int sub = tid % G;
+    for (int base = 0; base < K; base += kFinishThreads / G) {
+        const int i = base + tid / G;
+        const bool mine = i < K;
+        const int64_t r = i0 + (mine ? i : 0);
+        // the row's pairs and the draft token's logit are fetched together
         float x = 0.f;
-        if (id_ok) x = Elem<T>::load(logits + (r * ld + id) * ES);
-        const float2 ms = merge_partials(partials + r * P, P);
-        const RowDecision d = decide_row(x, ms.x, logf(ms.y), id_ok, log_tau, reject_none, reject_all);
-        myflags |= d.flags;
-        token_logp[r] = d.logp;
-        if (row_lse) row_lse[r] = d.lse;
-        const bool reject = d.reject;
-        if (reject && i < myfirst) myfirst = i;
+        bool id_ok = false;
+        if (mine && sub == 0) {
+            const int id = draft_ids[r];
+            id_ok = id >= 0 && id < V;
+            if (id_ok) x = Elem<T>::load(logits + (r * ld + id) * ES);
+        }
+        const float2 ms = merge_partials<G>(partials + r * P, P, sub);
+        if (mine && sub == 0) {
+            const RowDecision d = decide_row(x, ms.x, logf(ms.y), id_ok, log_tau, reject_none, reject_all);
+            myflags |= d.flags;
+            token_logp[r] = d.logp;
+            if (row_lse) row_lse[r] = d.lse;
+            const bool reject = d.reject;
+            if (reject && i < myfirst) myfirst = i;
+        }
     }
     if (myfirst < K) atomicMin(&first_reject, myfirst);
     if (myflags) atomicOr(&flags, myflags);
@@ -674,7 +699,7 @@ constexpr uint32_t kStatsInternal = 0x7fc0dead;   // in place of a row's maximum
 // triple (maximum of the local columns, sum of exponentials relative to it, logit of the draft
 // token if its column is local, else -inf).  Rows of skipped or malformed utterances are left
 // untouched; the combining kernel does not read them.
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
     const char *__restrict__ logits, int V_local, int64_t ld, int64_t M, int64_t col0,
     const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
@@ -688,15 +713,21 @@ __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
     const bool skipped = skip != nullptr && skip[b] != 0;
     if (i0 < 0 || i1 < i0 || i1 > M || skipped) return;
     const bool internal = err == epoch;
-    for (int64_t r = i0 + tid; r < i1; r += blockDim.x) {
-        const int64_t local = (int64_t)draft_ids[r] - col0;
-        const bool owned = local >= 0 && local < V_local;
+    const int sub = tid % G;
+    for (int64_t base = i0; base < i1; base += kFinishThreads / G) {
+        const bool mine = base + tid / G < i1;
+        const int64_t r = mine ? base + tid / G : base;
         float x = -INFINITY;
-        if (owned) x = Elem<T>::load(logits + (r * ld + local) * ES);
-        const float2 ms = merge_partials(partials + r * P, P);
-        stats[3 * r + 0] = internal ? __uint_as_float(kStatsInternal) : ms.x;
-        stats[3 * r + 1] = ms.y;
-        stats[3 * r + 2] = x;
+        if (mine && sub == 0) {
+            const int64_t local = (int64_t)draft_ids[r] - col0;
+            if (local >= 0 && local < V_local) x = Elem<T>::load(logits + (r * ld + local) * ES);
+        }
+        const float2 ms = merge_partials<G>(partials + r * P, P, sub);
+        if (mine && sub == 0) {
+            stats[3 * r + 0] = internal ? __uint_as_float(kStatsInternal) : ms.x;
+            stats[3 * r + 1] = ms.y;
+            stats[3 * r + 2] = x;
+        }
     }
 }
 
@@ -765,11 +796,13 @@ __global__ void __launch_bounds__(kFinishThreads) combine_kernel(
     }
 }
 
-// Greedy step: merges the partials of a row, one warp per row.  A partial is
-// (reference, sum, largest logit, index of its first occurrence).
+// Greedy step: merges the partials of a row, one warp per row.  A partial is (reference, sum,
+// largest logit, an index at or up to one 32-byte unit before its first occurrence): the unit is
+// looked through here, once per row, instead of once per column span in the streaming kernel.
 constexpr int kGreedyWarps = 8;
+template <typename T>
 __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
-    int V, int64_t R, const float4 *__restrict__ partials, int P, int32_t *__restrict__ next_token,
+    const char *__restrict__ logits, int V, int64_t ld, int64_t R, const float4 *__restrict__ partials, int P, int32_t *__restrict__ next_token,
     float *__restrict__ next_logp, float *__restrict__ row_lse, uint32_t *__restrict__ row_status,
     const unsigned long long *err_word, unsigned long long epoch) {
     pdl_enter();
@@ -794,6 +827,13 @@ __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
     }
     S = warp_sum(S);
     vi = __reduce_min_sync(0xffffffffu, vi);
+    if (vi >= 0 && vi < V) {
+        const int64_t e = (int64_t)vi + lane;
+        const bool hit = lane < 32 / Elem<T>::kBytes && e < V &&
+                         Elem<T>::load(logits + (r * ld + e) * Elem<T>::kBytes) == vm;
+        const unsigned hits = __ballot_sync(0xffffffffu, hit);
+        if (hits) vi += __ffs(hits) - 1;
+    }
     if (lane == 0) {
         const float lnS = logf(S);
         const float lse = Mx + lnS;
@@ -810,10 +850,36 @@ __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
 
 unsigned long long next_epoch();
 
+// Whether rows are streamed by the direct-load kernel (it needs no more scratch than the pairs of
+// the bulk-copy one).  Not where an option speaks about that one's ring.  Measured, ring against
+// direct loads, us on one B200, passes back to back:
+//   bf16, rows under 96 KB: direct (5,568 rows of 24 KB: 44.3 / 32.6; 20,000 of 48 KB: 197 / 160;
+//     20,000 of 64 KB: 234 / 206).  The ring hands a stage of a whole row from warp to warp.
+//   bf16, rows off a 16-byte boundary: direct (5,000 of 98 KB: 97.4 / 88.2; 20,000 of 64 KB:
+//     272 / 211).  The ring's producer waits for the ragged ends of every row.
+//   bf16, few rows (column spans in the ring): direct (300 of 98 KB: 15.0 / 12.0; 400 of 304 KB:
+//     31.1 / 28.6)
+//   bf16, aligned rows of 96 KB and more: the ring while the power cap does not bite (1,500 of
+//     98 KB: 31.9 / 33.7; 8,000: 136 / 141), direct beyond (12,000: 200 / 200; 16,000: 265 / 245;
+//     22,000 of 200 KB: 708 / 664): it spends a fifth fewer instructions on a logit.
+//   fp32: the ring (16,000 of 192 KB: 437 / 455; 1,000: 36.1 / 38.8), which has more bytes in
+//     flight and half the logits per byte; the greedy step on few rows: direct (200 of 196 KB:
+//     14.0 / 12.3; 300 of 608 KB: 36.4 / 35.8; 500 of 196 KB: 21.9 / 23.3)
+// The greedy step on bf16 rows: direct (1,024 of 304 KB: 59.5 / 55.1; 24 of 98 KB: 14.0 / 12.6).
+static int use_direct(int64_t M, int64_t row_bytes, ssd_dtype dtype, int kernel, int sms,
+                      const ssd_launch_opts *o, const RowsAt &at) {
+    if (kernel != 2 || row_bytes >= (1ll << 30) || M >= (1ll << 30)) return 0;
+    if (o && (o->kernel || o->warps || o->stages || o->stage_bytes || o->fma_exp || o->finish)) return 0;
+    const bool few = M < 4ll * sms;
+    if (dtype == SSD_F32) return at.greedy && M <= 2ll * sms;
+    if (at.greedy || few || row_bytes < 96 * 1024 || M * row_bytes >= 1200ll << 20) return 1;
+    return (reinterpret_cast<uintptr_t>(at.base) | (uintptr_t)(at.ld * 2)) % 16 != 0;
+}
+
 // Workspace: [0,256) header (error word, finished-CTA counter), two words per utterance, then
 // M * partials float2.
 int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts *o,
-                VerifyPlan *plan) {
+                const RowsAt &at, VerifyPlan *plan) {
     const int es = dtype == SSD_F32 ? 4 : 2;
     VerifyPlan pl{};
     pl.kernel = (o && o->kernel) ? o->kernel : 2;
@@ -875,6 +941,17 @@ int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts 
     pl.fma_exp = (o && o->fma_exp) ? (o->fma_exp < 0 ? 0 : o->fma_exp) : (dtype == SSD_BF16 ? 1 : 0);
     if (pl.fma_exp > 3) return SSD_ERR_ARG;
     pl.partials = split * pl.warps;
+    pl.direct = use_direct(M, row_bytes, dtype, pl.kernel, sms, o, at);
+    if (pl.direct) {
+        pl.direct_ctas = (o && o->ctas > 0) ? o->ctas : direct::kCtasPerSm * sms;
+        if (o && o->split > 0) {
+            pl.spans = split;
+            pl.span_blocks = (direct::row_blocks(row_bytes) + split - 1) / split;
+        } else {
+            direct::plan_spans(M, row_bytes, pl.direct_ctas * direct::kWarps,
+                               pl.partials < 64 ? pl.partials : 64, &pl.spans, &pl.span_blocks);
+        }
+    }
     // header | two words per utterance | partials
     pl.workspace_bytes = 256 + (((size_t)(B > 0 ? B : 0) * 16 + 255) & ~(size_t)255) +
                          (size_t)M * pl.partials * sizeof(float2);
@@ -902,7 +979,49 @@ static size_t partials_offset(int B) {
     return 256 + (((size_t)(B > 0 ? B : 0) * 16 + 255) & ~(size_t)255);
 }
 
-// Launches the streaming kernel that leaves plan.partials (reference, sum) pairs per row in the
+// Pairs per row that the streaming kernel of a plan leaves.
+static int pairs_per_row(const VerifyPlan &plan) { return plan.direct ? plan.spans : plan.partials; }
+
+// fp32 logits come here with the arg max only (see use_direct).
+template <bool kArg>
+static cudaError_t launch_direct(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_t M,
+                                 const int64_t *tok_off, int B, const uint8_t *skip, void *partials,
+                                 const VerifyPlan &plan, cudaStream_t stream) {
+    const int es = dtype == SSD_F32 ? 4 : 2;
+    direct::DirectParams p{};
+    p.logits = static_cast<const char *>(logits);
+    p.V = V; p.row_pitch = ld * es; p.row_bytes = V * es; p.M = M;
+    p.spans = plan.spans; p.span_blocks = plan.span_blocks;
+    p.tok_off = tok_off; p.B = B; p.skip = skip; p.partials = partials;
+    p.table = skip && direct::table_fits(B, M);
+    const int64_t items = M * plan.spans;
+    const int64_t ctas = items < plan.direct_ctas ? items : plan.direct_ctas;
+    const size_t smem = p.table ? (size_t)(B + 1) * sizeof(int32_t) : 0;
+    // one pair in eight on the FMA pipe is the best split under the power cap (22,000 rows of
+    // 200 KB: none 694 us, one 674, two 683); with the arg max none is (1,024 of 304 KB: 55.1
+    // against 55.9)
+    auto kern = direct::verify_rows_direct<bf16_t, kArg ? 0 : 1, kArg>;
+    if (kArg && dtype == SSD_F32) kern = direct::verify_rows_direct<float, 0, true>;
+    return launch_pdl(kern, (unsigned)ctas, (unsigned)direct::kThreads, smem, stream, p);
+}
+
+// The closing kernel for P pairs per row.
+template <template <int> class Pick> static auto pick_lanes(int P) -> decltype(Pick<1>::kernel()) {
+    switch (merge_lanes(P)) {
+        case 1: return Pick<1>::kernel();
+        case 2: return Pick<2>::kernel();
+        case 4: return Pick<4>::kernel();
+        case 8: return Pick<8>::kernel();
+        case 16: return Pick<16>::kernel();
+        default: return Pick<32>::kernel();
+    }
+}
+template <typename T> struct FinishKernels {
+    template <int G> struct Verify { static auto kernel() { return &verify_finish_kernel<T, G>; } };
+    template <int G> struct Shard { static auto kernel() { return &shard_finish_kernel<T, G>; } };
+};
+
+// Launches the streaming kernel that leaves pairs_per_row (reference, sum) pairs per row in the
 // workspace (nothing for rows of skipped utterances).
 static int launch_verify_rows(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_t M,
                               const int64_t *tok_off, int B, const uint8_t *skip, void *workspace,
@@ -923,7 +1042,10 @@ static int launch_verify_rows(const void *logits, ssd_dtype dtype, int V, int64_
         e = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_begin), L.stream);
         if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     }
-    if (plan.kernel == 2) {
+    if (plan.direct) {
+        e = launch_direct<false>(logits, dtype, V, ld, M, tok_off, B, skip, p.partials, plan, L.stream);
+        if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
+    } else if (plan.kernel == 2) {
         void (*kern)(const VerifyParams) = verify_rows_tma<float, 0, false>;
         if (dtype == SSD_BF16)
             kern = plan.fma_exp == 1 ? verify_rows_tma<bf16_t, 1, false>
@@ -1024,11 +1146,13 @@ int launch_verify(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_
     const int rc = launch_verify_rows(logits, dtype, V, ld, M, tok_off, B, skip, workspace, epoch,
                                       plan, L);
     if (rc != SSD_OK) return rc;
+    const int P = pairs_per_row(plan);
     e = launch_pdl(
-        dtype == SSD_F32 ? verify_finish_kernel<float> : verify_finish_kernel<bf16_t>,
+        dtype == SSD_F32 ? pick_lanes<FinishKernels<float>::Verify>(P)
+                         : pick_lanes<FinishKernels<bf16_t>::Verify>(P),
         (unsigned)B, (unsigned)kFinishThreads, 0, L.stream,
         static_cast<const char *>(logits), V, ld, M, tok_off, draft_ids, B, th.log_tau,
-        th.reject_none, th.reject_all, skip, static_cast<const float2 *>(partials), plan.partials,
+        th.reject_none, th.reject_all, skip, static_cast<const float2 *>(partials), P,
         token_logp, row_lse, accepted_len, all_accepted, utt_status,
         static_cast<const unsigned long long *>(err_word), epoch);
     if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
@@ -1050,11 +1174,13 @@ int launch_verify_shard(const void *logits, ssd_dtype dtype, int V_local, int64_
     const int rc = launch_verify_rows(logits, dtype, V_local, ld, M, tok_off, B, skip, workspace,
                                       epoch, plan, L);
     if (rc != SSD_OK) return rc;
+    const int P = pairs_per_row(plan);
     cudaError_t e = launch_pdl(
-        dtype == SSD_F32 ? shard_finish_kernel<float> : shard_finish_kernel<bf16_t>,
+        dtype == SSD_F32 ? pick_lanes<FinishKernels<float>::Shard>(P)
+                         : pick_lanes<FinishKernels<bf16_t>::Shard>(P),
         (unsigned)B, (unsigned)kFinishThreads, 0, L.stream,
         static_cast<const char *>(logits), V_local, ld, M, col0, tok_off, draft_ids, B, skip,
-        static_cast<const float2 *>(partials), plan.partials, shard_stats,
+        static_cast<const float2 *>(partials), P, shard_stats,
         static_cast<const unsigned long long *>(err_word), epoch);
     if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     e = cudaGetLastError();
@@ -1105,21 +1231,26 @@ int launch_greedy(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_
         e = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_begin), L.stream);
         if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     }
-    void (*kern)(const VerifyParams) = verify_rows_tma<float, 0, true>;
-    if (dtype == SSD_BF16)
-        kern = plan.fma_exp >= 1 ? verify_rows_tma<bf16_t, 1, true> : verify_rows_tma<bf16_t, 0, true>;
-    e = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), plan.smem_bytes);
-    if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
-    e = launch_pdl(kern, (unsigned)ctas, (unsigned)((plan.warps + 1) * 32), plan.smem_bytes,
-                   L.stream, p);
+    if (plan.direct) {
+        e = launch_direct<true>(logits, dtype, V, ld, R, nullptr, 0, nullptr, partials, plan, L.stream);
+    } else {
+        void (*kern)(const VerifyParams) = verify_rows_tma<float, 0, true>;
+        if (dtype == SSD_BF16)
+            kern = plan.fma_exp >= 1 ? verify_rows_tma<bf16_t, 1, true> : verify_rows_tma<bf16_t, 0, true>;
+        e = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), plan.smem_bytes);
+        if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
+        e = launch_pdl(kern, (unsigned)ctas, (unsigned)((plan.warps + 1) * 32), plan.smem_bytes,
+                       L.stream, p);
+    }
     if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     if (o && o->ev_end) {
         e = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_end), L.stream);
         if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     }
-    e = launch_pdl(greedy_finish_kernel, (unsigned)((R + kGreedyWarps - 1) / kGreedyWarps),
-                   (unsigned)(kGreedyWarps * 32), 0, L.stream, V, R,
-                   static_cast<const float4 *>(partials), plan.partials, next_token, next_logp,
+    e = launch_pdl(dtype == SSD_F32 ? greedy_finish_kernel<float> : greedy_finish_kernel<bf16_t>,
+                   (unsigned)((R + kGreedyWarps - 1) / kGreedyWarps),
+                   (unsigned)(kGreedyWarps * 32), 0, L.stream, p.logits, V, ld, R,
+                   static_cast<const float4 *>(partials), pairs_per_row(plan), next_token, next_logp,
                    row_lse, row_status, static_cast<const unsigned long long *>(err_word), epoch);
     if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     e = cudaGetLastError();

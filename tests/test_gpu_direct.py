@@ -1,0 +1,135 @@
+"""The direct-load streaming kernel (what ssd_verify, ssd_verify_shard and ssd_greedy_step run by
+default on most bf16 calls) against the fp64 oracle and the plain-load kernel, at the sizes where
+its units, blocks, spans and tables have their edges."""
+import numpy as np
+import pytest
+import torch
+
+import helpers as H
+from oracle import ref
+from paper_2603_11243_b200 import binding as ssd
+
+pytestmark = pytest.mark.gpu
+
+# a unit is 16 bf16 logits, a block 512; sizes around both, and one of several spans
+SIZES = (1, 2, 15, 16, 17, 31, 33, 47, 511, 512, 513, 1024, 1039, 4097, 20011)
+
+
+def _rows(M, V, col0, seed, dtype=torch.bfloat16, scale=2.0):
+    g = torch.Generator()
+    g.manual_seed(seed)
+    wide = (torch.randn((M, V + 19), generator=g) * scale).to(dtype)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32)
+    return wide, wide[:, col0:col0 + V], ids
+
+
+def _offsets(lens):
+    return torch.tensor(np.concatenate([[0], np.cumsum(lens)]), dtype=torch.int64)
+
+
+def _verify(view, off, ids, dev, wide, col0, skip=None, opts=None):
+    x = wide.to(dev)[:, col0:col0 + view.shape[1]]
+    sk = None if skip is None else torch.as_tensor(skip, dtype=torch.uint8).to(dev)
+    out = ssd.ssd_verify(x, off.to(dev), ids.to(dev), 0.1, skip=sk, opts=opts)
+    torch.cuda.synchronize()
+    return out
+
+
+@pytest.mark.parametrize("col0", [0, 1, 7, 13])
+@pytest.mark.parametrize("V", SIZES)
+def test_verify_sizes_and_alignments(cuda_device, V, col0):
+    lens = [5, 0, 17, 1, 9]
+    wide, view, ids = _rows(sum(lens), V, col0, 7 * V + col0)
+    off = _offsets(lens)
+    skip = [0, 0, 1, 0, 0]
+    out = _verify(view, off, ids, cuda_device, wide, col0, skip)
+    orc = ref.verify(H.storage_numpy(view.contiguous()), V, off.numpy(), ids.numpy(),
+                     float(np.float32(0.1)), skip=np.array(skip, np.uint8))
+    H.compare_stage2(out, orc, off.numpy(), 0.1, skip=np.array(skip, np.uint8), require_all_margins=False)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", SIZES)
+def test_greedy_first_of_equals(cuda_device, V, dtype):
+    """The largest logit planted several times, next to unit and block edges: the first counts."""
+    wide, view, _ = _rows(23, V, 3, V, dtype)
+    rng = np.random.default_rng(V)
+    for r in range(23):
+        for c in {int(rng.integers(0, V)), V - 1, min(V - 1, 16 * int(rng.integers(0, 1 + V // 16)))}:
+            view[r, c] = 30.0
+    want = ref.greedy_step(H.storage_numpy(view.contiguous()), V)
+    got = ssd.ssd_greedy_step(wide.to(cuda_device)[:, 3:3 + V])
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(got["next_token"].cpu().numpy(), want["next_token"])
+    assert np.abs(got["row_lse"].cpu().numpy() - want["row_lse"]).max() <= H.FLOAT_TOL
+
+
+@pytest.mark.parametrize("V", [700, 5000])
+def test_rows_outside_the_fast_pass(cuda_device, V):
+    """Masked vocabularies, logits far from the reference in both directions, large magnitudes:
+    the same answers as the plain-load kernel; NaN and +inf are flagged by both."""
+    lens = [4] * 12
+    wide, view, ids = _rows(48, V, 5, V)
+    lowest = torch.finfo(torch.bfloat16).min
+    view[0:4, :600] = float("-inf")              # nothing finite in a span's first block
+    view[4:8, :] = float("-inf")
+    view[4:8, V // 2] = 1.5                      # one finite logit
+    view[8:12, :] = lowest
+    view[8:12, 3] = 0.0
+    view[12:16, V - 1] = 300.0                   # far above everything before it
+    view[16:20, 0] = 300.0                       # a first logit far above the rest
+    view[20:24] += 6000.0
+    view[24:28] -= 6000.0
+    view[28:32, V - 2] = float("nan")
+    view[32:36, 1] = float("inf")
+    view[36:40, :] = float("-inf")               # a row of nothing
+    for r in list(range(0, 28)) + list(range(40, 48)):
+        ids[r] = int(view[r].float().argmax())
+    off = _offsets(lens)
+    a = _verify(view, off, ids, cuda_device, wide, 5)
+    b = _verify(view, off, ids, cuda_device, wide, 5, opts=H.opts(kernel=1))
+    for k in ("accepted_len", "all_accepted", "utt_status"):
+        assert torch.equal(a[k], b[k]), k
+    assert (a["utt_status"].cpu().numpy()[[7, 8, 9]] == ssd.UTT_NONFINITE).all()
+    fine = [r for r in range(48) if not 28 <= r < 40]
+    for k in ("token_logp", "row_lse"):
+        x, y = a[k].cpu()[fine].double(), b[k].cpu()[fine].double()
+        # the two sum in different orders: a few units in the last place of values up to 6,000
+        assert bool(((x - y).abs() <= H.FLOAT_TOL + 4 * 2.0 ** -23 * y.abs()).all()), k
+    ga = ssd.ssd_greedy_step(wide.to(cuda_device)[:, 5:5 + V])
+    want = view.float().argmax(1).numpy()
+    rows = [r for r in range(48) if not 28 <= r < 40]
+    np.testing.assert_array_equal(ga["next_token"].cpu().numpy()[rows], want[rows])
+
+
+@pytest.mark.parametrize("B,split", [(1, 0), (2046, 0), (2047, 0), (2500, 0), (700, 3)])
+def test_skipped_utterances(cuda_device, B, split):
+    """The count of rows to read in shared memory, its largest size, and the way without it."""
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, 4, size=B)
+    skip = (rng.random(B) < 0.6).astype(np.uint8)
+    V = 1100
+    wide, view, ids = _rows(int(lens.sum()) or 1, V, 2, B)
+    off = _offsets(lens)
+    M = int(off[-1])
+    if M == 0:
+        wide, view, ids = wide[:0], view[:0], ids[:0]
+    o = H.opts(split=split) if split else None
+    a = _verify(view, off, ids, cuda_device, wide, 2, skip, o)
+    b = _verify(view, off, ids, cuda_device, wide, 2, skip, H.opts(kernel=1))
+    for k in ("accepted_len", "all_accepted", "utt_status"):
+        assert torch.equal(a[k], b[k]), k
+    rows = torch.from_numpy(np.repeat(skip == 0, lens))
+    diff = (a["token_logp"].cpu()[rows] - b["token_logp"].cpu()[rows]).abs()
+    assert diff.numel() == 0 or float(diff.max()) <= H.FLOAT_TOL
+
+
+def test_malformed_offsets(cuda_device):
+    """Offsets that run backwards: flagged, the sound utterances around them unharmed."""
+    wide, view, ids = _rows(30, 900, 0, 3)
+    off = torch.tensor([0, 10, 4, 20, 31, 30], dtype=torch.int64)
+    skip = [0, 0, 0, 0, 0]
+    a = _verify(view, off, ids, cuda_device, wide, 0, skip)
+    b = _verify(view, off, ids, cuda_device, wide, 0, skip, H.opts(kernel=1))
+    for k in ("accepted_len", "all_accepted", "utt_status"):
+        assert torch.equal(a[k], b[k]), k
