@@ -4,6 +4,10 @@ Every function here takes torch tensors that already live on the CUDA device, pa
 addresses to the C entry point of the same name and returns the output tensors; all
 computation happens in the library's CUDA kernels.  There is no CPU fallback: importing this
 module without a built libssd.so, or calling it with host tensors, raises.
+
+The calls of a decoding step, with result buffers given and no launch options, are marshalled by
+_ssd_call (csrc/ssd_call.cpp); whatever it does not take -- it answers None -- goes the general way
+through ctypes, which is also where wrong arguments are named.
 """
 import ctypes as C
 import os
@@ -38,6 +42,20 @@ class LaunchOpts(C.Structure):
 
 
 _lib = None
+_call = None
+
+
+def _native():
+    global _call
+    if _call is None:
+        lib()
+        try:
+            from . import _ssd_call
+        except ImportError as e:
+            raise ImportError("_ssd_call.so is not built: run `python -m paper_2603_11243_b200.build` "
+                              "(needs nvcc and a host compiler)") from e
+        _call = _ssd_call
+    return _call
 
 
 def lib():
@@ -181,6 +199,12 @@ def ssd_ctc_draft(logits: torch.Tensor, frame_off: torch.Tensor, blank_id: int,
                   max_draft_len: int, V: Optional[int] = None, out=None, want_logprob=False,
                   opts: Optional[LaunchOpts] = None) -> Dict[str, torch.Tensor]:
     """Stage 1 (Section 2.1, Eq. 2, Eq. 3): frame statistics and the collapsed draft."""
+    if out is not None and opts is None:
+        rc = (_call or _native()).ctc_draft(logits, frame_off, blank_id, max_draft_len, V, out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_ctc_draft")
     N, ld = _rows_ld(logits)
     V = logits.shape[1] if V is None else V
     B = frame_off.shape[0] - 1
@@ -241,6 +265,12 @@ def ssd_entropy_gate_from_maxima(utt_max_entropy: torch.Tensor, utt_status: torc
     """The entropy gate (Eq. 3) through ssd_entropy_gate's second form: from the utterance
     maxima and status words ssd_ctc_draft left behind (B values instead of N frame entropies).
     `out` needs gate_accept and max_entropy only."""
+    if out is not None:
+        rc = (_call or _native()).gate_from_maxima(utt_max_entropy, utt_status, tau_ctc, out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_entropy_gate")
     if out is None:
         B, dev = utt_max_entropy.shape[0], utt_max_entropy.device
         out = dict(gate_accept=torch.empty((B,), dtype=torch.uint8, device=dev),
@@ -264,6 +294,12 @@ def ssd_verify(logits: torch.Tensor, tok_off: torch.Tensor, draft_ids: torch.Ten
                tau_slm: float, skip: Optional[torch.Tensor] = None, V: Optional[int] = None,
                out=None, opts: Optional[LaunchOpts] = None) -> Dict[str, torch.Tensor]:
     """Stage 2 (Eq. 5, Section 2.3): draft-token log-likelihoods and the accepted prefix."""
+    if out is not None and opts is None:
+        rc = (_call or _native()).verify(logits, tok_off, draft_ids, tau_slm, skip, V, out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_verify")
     M, ld = _rows_ld(logits)
     V = logits.shape[1] if V is None else V
     B = tok_off.shape[0] - 1
@@ -321,6 +357,13 @@ def ssd_verify_shard(logits: torch.Tensor, col0: int, tok_off: torch.Tensor,
                      opts: Optional[LaunchOpts] = None) -> torch.Tensor:
     """Stage 2 over a vocabulary-parallel LLM head, this rank's part: `logits` holds columns
     [col0, col0 + V_local) of the whole vocabulary; returns [M, 3] (max, sum, draft logit)."""
+    if stats is not None and workspace is not None and opts is None:
+        rc = (_call or _native()).verify_shard(logits, col0, tok_off, draft_ids, skip, V_local, stats,
+                                               workspace)
+        if rc == OK:
+            return stats
+        if rc is not None:
+            raise SsdError(rc, "ssd_verify_shard")
     M, ld = _rows_ld(logits)
     V_local = logits.shape[1] if V_local is None else V_local
     B = tok_off.shape[0] - 1
@@ -347,6 +390,13 @@ def ssd_verify_combine(stats_all: torch.Tensor, V_total: int, tok_off: torch.Ten
                        skip: Optional[torch.Tensor] = None, out=None) -> Dict[str, torch.Tensor]:
     """After the all-gather of every rank's ssd_verify_shard result into stats_all [R, M, 3]:
     log-likelihoods (Eq. 5) and the accepted prefix, as ssd_verify returns them."""
+    if out is not None:
+        rc = (_call or _native()).verify_combine(stats_all, V_total, tok_off, draft_ids, tau_slm, skip,
+                                                 out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_verify_combine")
     if stats_all.dim() != 3 or stats_all.shape[2] != 3 or not stats_all.is_contiguous() \
             or stats_all.dtype != torch.float32:
         raise ValueError("stats_all must be a contiguous float32 tensor [R, M, 3]")
@@ -401,6 +451,12 @@ def ssd_verify_early_exit(logits: torch.Tensor, tok_off: torch.Tensor, draft_ids
                           opts: Optional[LaunchOpts] = None) -> Dict[str, torch.Tensor]:
     """Stage 2 with early exit (Section 2.3 needs only the first reject): same decisions as
     ssd_verify; token_logp only for the rows that were read."""
+    if out is not None and opts is None:
+        rc = (_call or _native()).verify_early_exit(logits, tok_off, draft_ids, tau_slm, skip, V, out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_verify_early_exit")
     if out is None:
         M = logits.shape[0]
         out = alloc_early_exit_outputs(M, tok_off.shape[0] - 1,
@@ -456,6 +512,12 @@ def ssd_assemble(tokens: torch.Tensor, tok_off: torch.Tensor, gate_accept: torch
                  accepted_len: torch.Tensor, all_accepted: torch.Tensor,
                  out=None) -> Dict[str, torch.Tensor]:
     """Eq. 7: final hypotheses and the ordered list of utterances left to the AR pass."""
+    if out is not None:
+        rc = (_call or _native()).assemble(tokens, tok_off, gate_accept, accepted_len, all_accepted, out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_assemble")
     B, M = tok_off.shape[0] - 1, tokens.shape[0]
     if tokens.dtype != torch.int32 or accepted_len.dtype != torch.int32:
         raise TypeError("tokens and accepted_len must be int32")
@@ -487,6 +549,12 @@ def ssd_greedy_step_workspace_bytes(R, V, dtype_code, opts=None) -> int:
 def ssd_greedy_step(logits: torch.Tensor, V: Optional[int] = None, out=None,
                     opts: Optional[LaunchOpts] = None) -> Dict[str, torch.Tensor]:
     """One greedy decoding step (Eq. 6) per row: most likely token and its log-likelihood."""
+    if out is not None and opts is None:
+        rc = (_call or _native()).greedy_step(logits, V, out)
+        if rc == OK:
+            return out
+        if rc is not None:
+            raise SsdError(rc, "ssd_greedy_step")
     R, ld = _rows_ld(logits)
     V = logits.shape[1] if V is None else V
     code = _dtype_code(logits)

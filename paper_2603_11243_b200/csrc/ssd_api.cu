@@ -1,8 +1,9 @@
 // The C ABI of libssd: argument validation and dispatch.  Every step of the path runs in the
 // kernels of ssd_ctc.cu and ssd_verify.cu; nothing here computes.
+#include <atomic>
 #include <map>
 #include <mutex>
-#include <utility>
+#include <tuple>
 
 #include "ssd_common.cuh"
 
@@ -10,9 +11,8 @@ namespace ssd {
 namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
-int g_sm_count[kMaxDevices];                                   // 0: not asked yet
-std::map<std::pair<const void *, int>, size_t> g_smem_set;     // (kernel, device) -> bytes set
-std::map<std::pair<const void *, int>, int> g_carveout_set;    // (kernel, device) -> percent
+std::atomic<int> g_sm_count[kMaxDevices];                               // 0: not asked yet
+std::map<std::tuple<const void *, int, int>, int> g_attributes;         // (kernel, device, attribute) -> value set
 thread_local int t_replay = 0;
 }  // namespace
 
@@ -23,41 +23,50 @@ int device_sm_count() {
     if (t_replay > 0) return 148;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-    std::lock_guard<std::mutex> lock(g_mutex);
-    if (g_sm_count[dev] == 0) {
-        int n = 0;
+    int n = g_sm_count[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
             return 0;
-        g_sm_count[dev] = n;
+        g_sm_count[dev].store(n, std::memory_order_relaxed);
     }
-    return g_sm_count[dev];
+    return n;
 }
 
-cudaError_t ensure_dynamic_smem(const void *kernel, size_t bytes) {
+namespace {
+// Raises an attribute of (kernel, device) to `value` where it is lower.  A launch asks every
+// time; what this thread has asked before is answered without the lock.
+struct Asked {
+    const void *kernel;
+    int dev, attr, value;
+};
+thread_local Asked t_asked[64];
+cudaError_t raise_attribute(const void *kernel, cudaFuncAttribute attr, int value) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    Asked &a = t_asked[((reinterpret_cast<uintptr_t>(kernel) >> 4) * 0x9e3779b97f4a7c15ull + attr) >> 58 & 63];
+    if (a.kernel == kernel && a.dev == dev && a.attr == (int)attr && value <= a.value) return cudaSuccess;
     std::lock_guard<std::mutex> lock(g_mutex);
-    size_t &have = g_smem_set[std::make_pair(kernel, dev)];
-    if (bytes <= have) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) have = bytes;
-    return e;
+    int &have = g_attributes[std::make_tuple(kernel, dev, (int)attr)];
+    if (value > have) {
+        e = cudaFuncSetAttribute(kernel, attr, value);
+        if (e != cudaSuccess) return e;
+        have = value;
+    }
+    a = Asked{kernel, dev, (int)attr, have};
+    return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t ensure_dynamic_smem(const void *kernel, size_t bytes) {
+    return raise_attribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 cudaError_t ensure_l1(const void *kernel, size_t smem) {
-    int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
     // what two CTAs take (1 KB each is the system's, 1 KB for static arrays), in percent of the
     // 228 KB that can be shared memory
-    const int percent = (int)((2 * (smem + 2048) * 100 + 228 * 1024 - 1) / (228 * 1024));
-    std::lock_guard<std::mutex> lock(g_mutex);
-    int &have = g_carveout_set[std::make_pair(kernel, dev)];
-    if (percent <= have) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
-    if (e == cudaSuccess) have = percent;
-    return e;
+    return raise_attribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           (int)((2 * (smem + 2048) * 100 + 228 * 1024 - 1) / (228 * 1024)));
 }
 
 static thread_local int32_t t_last_cuda_error = 0;

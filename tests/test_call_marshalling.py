@@ -1,0 +1,100 @@
+"""The native marshalling of the hot calls: what it does not take goes the general way and raises
+what that raises; what it takes computes what the general way computes."""
+import pytest
+import torch
+
+import helpers as H
+from paper_2603_11243_b200 import binding as ssd
+from paper_2603_11243_b200 import build as ssd_build
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    ssd_build.build()
+
+
+def _verify_inputs(device, M=6, V=40):
+    x = torch.zeros((M, V), dtype=torch.bfloat16, device=device)
+    off = torch.tensor([0, M], dtype=torch.int64, device=device)
+    ids = torch.zeros((M,), dtype=torch.int32, device=device)
+    out = ssd.alloc_verify_outputs(M, 1, device, 4096)
+    return x, off, ids, out
+
+
+def test_what_is_not_plainly_fine_is_declined():
+    call = ssd._native()
+    x, off, ids, out = _verify_inputs("cpu")
+    assert call.verify(x, off, ids, 0.1, None, None, out) is None               # host tensors
+    assert call.verify("logits", off, ids, 0.1, None, None, out) is None
+    assert call.verify(x, off, ids, 0.1, None, None) is None                    # an argument short
+    assert call.greedy_step(x.half(), None, out) is None
+    assert call.ctc_draft(x, off, 0, 1 << 40, None, out) is None
+    assert call.assemble(ids, off, ids, ids, ids, None) is None
+    assert call.verify_combine(x, 4, off, ids, "0.1", None, out) is None
+
+
+def test_errors_are_those_of_the_general_way():
+    x, off, ids, out = _verify_inputs("cpu")
+    with pytest.raises(ValueError):
+        ssd.ssd_verify(x, off, ids, 0.1, out=out)                               # no host path
+    with pytest.raises(TypeError):
+        ssd.ssd_verify(x, off.int(), ids, 0.1, out=out)
+    with pytest.raises(ValueError):
+        ssd.ssd_greedy_step(x.t(), out=out)
+    with pytest.raises(ValueError):
+        ssd.ssd_verify_combine(x, 4, off, ids, 0.1, out=out)
+    with pytest.raises(KeyError):
+        ssd.ssd_verify(x, off, ids, 0.1, out={})
+
+
+@pytest.mark.gpu
+def test_same_results_both_ways(cuda_device):
+    """opts given (all automatic) is the general way.  Padded rows, V below the row's width,
+    absent optional buffers, a stream of the caller's."""
+    dev = cuda_device
+    g = torch.Generator().manual_seed(5)
+    wide = torch.randn((37, 1203), generator=g).bfloat16().to(dev)
+    x = wide[:, 3:1200]
+    off = torch.tensor([0, 9, 9, 37], dtype=torch.int64, device=dev)
+    ids = torch.randint(0, 1000, (37,), generator=g, dtype=torch.int32).to(dev)
+    skip = torch.tensor([0, 0, 1], dtype=torch.uint8, device=dev)
+    side = torch.cuda.Stream(dev)
+    auto = H.opts()
+
+    def both(run):
+        with torch.cuda.stream(side):
+            a, b = run(None), run(auto)
+        side.synchronize()
+        for k in a:
+            if k != "workspace":
+                assert torch.equal(a[k].cpu(), b[k].cpu()), k
+
+    side.wait_stream(torch.cuda.current_stream())
+    for V in (None, 1000):
+        need = ssd.ssd_verify_workspace_bytes(3, 37, V or x.shape[1], ssd.BF16)
+
+        def zeroed(o, *drop):
+            for k in drop:
+                del o[k]
+            for t in o.values():
+                t.zero_()
+            return o
+
+        both(lambda o: ssd.ssd_verify(x, off, ids, 0.1, skip=skip, V=V, opts=o,
+                                      out=zeroed(ssd.alloc_verify_outputs(37, 3, dev, need), "row_lse")))
+        both(lambda o: ssd.ssd_verify_early_exit(
+            x, off, ids, 0.1, V=V, opts=o,
+            out=zeroed(ssd.alloc_early_exit_outputs(37, 3, V or x.shape[1], ssd.BF16, dev))))
+        both(lambda o: ssd.ssd_ctc_draft(x, off, 0, 20, V=V, opts=o,
+                                         out=zeroed(ssd.alloc_ctc_outputs(37, 3, dev), "draft_frames")))
+        both(lambda o: {"stats": ssd.ssd_verify_shard(
+            x, 5, off, ids, skip=skip, V_local=V, opts=o, stats=torch.zeros((37, 3), device=dev),
+            workspace=torch.zeros((max(need, 256),), dtype=torch.uint8, device=dev))})
+        ws = ssd.ssd_greedy_step_workspace_bytes(37, V or x.shape[1], ssd.BF16)
+        both(lambda o: ssd.ssd_greedy_step(x, V=V, opts=o, out=dict(
+            next_token=torch.zeros((37,), dtype=torch.int32, device=dev),
+            workspace=torch.zeros((ws,), dtype=torch.uint8, device=dev))))
+    out = ssd.alloc_verify_outputs(37, 3, dev, 16)
+    with pytest.raises(ssd.SsdError) as e:
+        ssd.ssd_verify(x, off, ids, 0.1, out=dict(out, workspace=out["workspace"][:16]))
+    assert e.value.code == ssd.ERR_WORKSPACE
