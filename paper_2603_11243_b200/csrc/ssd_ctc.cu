@@ -841,6 +841,17 @@ int plan_ctc(ssd_dtype dtype, int V, int64_t ld, int64_t N, int B, const ssd_lau
     // lanes per row: the smallest power of two for which one pass (32/G rows) is at most 16.5 KB
     int G = 2;
     while (G < 32 && (32 / G) * row_pitch > 16896) G *= 2;
+    // Few rows: more lanes per row, as long as one pass per warp is enough for all of them and a
+    // lane still walks four chunks.  A tile of 16 KB is 4 us of work for the one warp that has it,
+    // and with fewer tiles than warps that is the kernel's time (1,000 rows of 1,025 bf16 symbols:
+    // 9.8 us with 4 lanes per row on 125 warps, 7.1 with 32 on 1,000; 4,500 of 349: 9.4 with 2,
+    // 7.1 with 8, 7.3 with 16; 4,500 of 1,025: 10.3 with 4, 8.9 with 16, 12.4 with 32).
+    bool spread = false;
+    while (!(o && o->split > 0) && G < 32 &&
+           N * 2 * G <= 32ll * 16 * device_sm_count() && chunks_max >= 8 * G) {
+        G *= 2;
+        spread = true;
+    }
     if (o && o->split > 0) {
         G = o->split;
         if (G != 2 && G != 4 && G != 8 && G != 16 && G != 32) return SSD_ERR_ARG;
@@ -859,7 +870,7 @@ int plan_ctc(ssd_dtype dtype, int V, int64_t ld, int64_t N, int B, const ssd_lau
     int64_t stage_stride = 0;
     if (kernel != 1 && row_pitch <= 2 * row_bytes + 64 && row_pitch < (1 << 20)) {
         int64_t groups = 8192 / (rpw * row_pitch);
-        if (groups < 1) groups = 1;
+        if (groups < 1 || spread) groups = 1;
         if (o && o->stage_bytes > 0) groups = (o->stage_bytes + rpw - 1) / rpw;
         for (; groups >= 1 && warps == 0; groups = groups > 1 ? groups / 2 : 0) {
             R = (int)(groups * rpw);
