@@ -25,9 +25,12 @@ struct Launch {
 // the stream is still running, which takes the launch latency of the short per-utterance
 // kernels off the critical path.  A kernel first lets its own successor be scheduled, then
 // waits until every earlier grid has completed and its writes are visible; nothing before
-// pdl_enter() / pdl_wait() touches global memory.  The streaming kernels call the two halves
-// apart, with their shared-memory set-up in between, so that the set-up (and the cold
-// instruction fetches that come with it) overlaps the predecessor's tail.
+// pdl_enter() / pdl_wait() writes global memory, or reads it but for the closing kernels below.
+// The streaming kernels call the two halves apart, with their shared-memory set-up in front of
+// the wait, so that the set-up (and the cold instruction fetches that come with it) overlaps the
+// predecessor's tail, and let their successor be scheduled after it: the closing kernel of the
+// same call then begins when everything before the streaming kernel is complete, and fetches
+// (from L2, load_input) what the caller passed in while the streaming kernel still runs.
 __device__ __forceinline__ void pdl_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -344,6 +347,9 @@ template <typename T> struct Elem;
 template <> struct Elem<float> {
     static constexpr int kBytes = 4;
     static constexpr int kPerChunk = 4;  // elements in a 16-byte chunk
+    __device__ static __forceinline__ float load_l2(const void *p) {
+        return __ldcg(reinterpret_cast<const float *>(p));
+    }
     __device__ static __forceinline__ float load(const void *p) {
         return *reinterpret_cast<const float *>(p);
     }
@@ -354,10 +360,16 @@ template <> struct Elem<float> {
     }
     static constexpr uint32_t kNegInfBits = 0xff800000u;
 };
+// An input of the call, read before the streaming kernel of the same call is through.
+template <typename V> __device__ __forceinline__ V load_input(const V *p) { return __ldcg(p); }
+
 struct bf16_t { uint16_t bits; };
 template <> struct Elem<bf16_t> {
     static constexpr int kBytes = 2;
     static constexpr int kPerChunk = 8;
+    __device__ static __forceinline__ float load_l2(const void *p) {
+        return __uint_as_float(static_cast<uint32_t>(__ldcg(reinterpret_cast<const uint16_t *>(p))) << 16);
+    }
     __device__ static __forceinline__ float load(const void *p) {
         return __uint_as_float(static_cast<uint32_t>(*reinterpret_cast<const uint16_t *>(p)) << 16);
     }

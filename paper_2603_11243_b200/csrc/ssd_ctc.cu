@@ -474,7 +474,6 @@ template <typename T, int G, int kF>
 __global__ void __launch_bounds__(512, 1) ctc_rows_tma(const CtcParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int ES = Elem<T>::kBytes, EPC = Elem<T>::kPerChunk;
-    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int W = p.warps, R = p.rows_per_tile;
     const int64_t gw = (int64_t)blockIdx.x + (int64_t)gridDim.x * warp, GW = (int64_t)gridDim.x * W;
@@ -546,6 +545,7 @@ __global__ void __launch_bounds__(512, 1) ctc_rows_tma(const CtcParams p) {
         if (lane == 0) pend = tagged_begin(counter, epoch, pend_k);
     };
     pdl_wait();
+    pdl_launch_dependents();
     issue(t);
     if (dynamic) {
         // The tag of this launch's counter words: the host's call number plus the number of
@@ -618,7 +618,8 @@ __global__ void __launch_bounds__(512, 1) ctc_rows_tma(const CtcParams p) {
 template <typename T>
 __global__ void __launch_bounds__(256) ctc_rows_plain(const CtcParams p) {
     constexpr int ES = Elem<T>::kBytes;
-    pdl_enter();
+    pdl_wait();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t GW = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -687,12 +688,14 @@ __global__ void __launch_bounds__(kUttThreads) collapse_kernel(
     __shared__ int warp_tot[2][32];
     __shared__ MaxAt scratch[32];
     __shared__ unsigned flags_sh[32];
-    pdl_enter();
+    pdl_launch_dependents();
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nw = blockDim.x >> 5;
+    if (N == 0) pdl_wait();        // no streaming kernel of this call before this one
+    const int64_t t0 = load_input(frame_off + b), t1 = load_input(frame_off + b + 1);
+    pdl_wait();
     // the frame statistics kernel before this one is through, the next one has not begun
     if (launch_gen && b == 0 && tid == 0) *launch_gen = *launch_gen + 1;
-    const int64_t t0 = frame_off[b], t1 = frame_off[b + 1];
     if (t0 < 0 || t1 < t0 || t1 > N) {
         if (tid == 0) {
             draft_len[b] = 0; draft_full_len[b] = 0; utt_max_entropy[b] = 0.f;

@@ -181,8 +181,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     __shared__ int32_t warp_tot[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool table = p.table != 0;
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     int rows = (int)p.M;
     if (table) {
         const int per = (p.B + kThreads - 1) / kThreads, b0 = (int)threadIdx.x * per;

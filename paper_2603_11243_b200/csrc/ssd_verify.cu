@@ -58,7 +58,6 @@ template <typename T, int kF, bool kArg>
 __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int ES = Elem<T>::kBytes, EPC = Elem<T>::kPerChunk;
-    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = p.stages, CW = p.warps;
     // layout: full[S] | empty[S] | desc[S] | offsets cache | stages
@@ -79,6 +78,7 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
         mbar_init_fence();
     }
     pdl_wait();
+    pdl_launch_dependents();
     if (cache_off)
         for (int i = threadIdx.x; i <= p.B; i += blockDim.x) off_cache[i] = p.tok_off[i];
     __syncthreads();
@@ -595,7 +595,8 @@ __global__ void __launch_bounds__(544, 1) verify_rows_fin(const FinParams q) {
 template <typename T>
 __global__ void __launch_bounds__(256) verify_rows_plain(const VerifyParams p) {
     constexpr int ES = Elem<T>::kBytes;
-    pdl_enter();
+    pdl_wait();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int64_t item = blockIdx.x; item < p.num_items; item += gridDim.x) {
         const int64_t row = item / p.split;
@@ -634,14 +635,24 @@ __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
     constexpr int ES = Elem<T>::kBytes;
     __shared__ int first_reject;
     __shared__ unsigned flags;
-    pdl_enter();
-    // The kernel is a chain of dependent memory round trips, so the loads of each level are
-    // issued together: offsets, skip flag and error word; then a row's draft id and its
-    // partials; then the draft token's logit.
-    const int b = blockIdx.x, tid = threadIdx.x;
-    const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
+    pdl_launch_dependents();
+    // The kernel is a chain of dependent memory round trips.  What the caller passed in -- offsets,
+    // skip flag, then the first sweep's draft ids, then their logits -- is fetched while the
+    // streaming kernel still runs; after it a row waits for its pairs alone.
+    const int b = blockIdx.x, tid = threadIdx.x, sub = tid % G;
+    if (M == 0) pdl_wait();        // no streaming kernel of this call before this one
+    const int64_t i0 = load_input(tok_off + b), i1 = load_input(tok_off + b + 1);
+    const bool skipped = skip != nullptr && load_input(skip + b) != 0;
+    auto draft_logit = [&](int64_t r, bool &id_ok) {
+        const int id = load_input(draft_ids + r);
+        id_ok = id >= 0 && id < V;
+        return id_ok ? Elem<T>::load_l2(logits + (r * ld + id) * ES) : 0.f;
+    };
+    float x = 0.f;
+    bool id_ok = false;
+    if (i0 >= 0 && i1 <= M && sub == 0 && i0 + tid / G < i1 && !skipped) x = draft_logit(i0 + tid / G, id_ok);
+    pdl_wait();
     const unsigned long long err = *err_word;
-    const bool skipped = skip != nullptr && skip[b] != 0;
     const uint32_t internal = (err == epoch) ? (uint32_t)SSD_UTT_INTERNAL : 0u;
     if (i0 < 0 || i1 < i0 || i1 > M) {
         if (tid == 0) {
@@ -660,19 +671,11 @@ __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
     __syncthreads();
     unsigned myflags = 0;
     int myfirst = K;
-    const int sub = tid % G;
     for (int base = 0; base < K; base += kFinishThreads / G) {
         const int i = base + tid / G;
         const bool mine = i < K;
         const int64_t r = i0 + (mine ? i : 0);
-        // the row's pairs and the draft token's logit are fetched together
-        float x = 0.f;
-        bool id_ok = false;
-        if (mine && sub == 0) {
-            const int id = draft_ids[r];
-            id_ok = id >= 0 && id < V;
-            if (id_ok) x = Elem<T>::load(logits + (r * ld + id) * ES);
-        }
+        if (base > 0 && mine && sub == 0) x = draft_logit(r, id_ok);
         const float2 ms = merge_partials<G>(partials + r * P, P, sub);
         if (mine && sub == 0) {
             const RowDecision d = decide_row(x, ms.x, logf(ms.y), id_ok, log_tau, reject_none, reject_all);
@@ -706,22 +709,26 @@ __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
     const uint8_t *__restrict__ skip, const float2 *__restrict__ partials, int P,
     float *__restrict__ stats, const unsigned long long *err_word, unsigned long long epoch) {
     constexpr int ES = Elem<T>::kBytes;
-    pdl_enter();
-    const int b = blockIdx.x, tid = threadIdx.x;
-    const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
-    const unsigned long long err = *err_word;
-    const bool skipped = skip != nullptr && skip[b] != 0;
-    if (i0 < 0 || i1 < i0 || i1 > M || skipped) return;
-    const bool internal = err == epoch;
-    const int sub = tid % G;
+    pdl_launch_dependents();
+    // inputs before the wait, as in verify_finish_kernel
+    const int b = blockIdx.x, tid = threadIdx.x, sub = tid % G;
+    if (M == 0) pdl_wait();        // no streaming kernel of this call before this one
+    const int64_t i0 = load_input(tok_off + b), i1 = load_input(tok_off + b + 1);
+    const bool skipped = skip != nullptr && load_input(skip + b) != 0;
+    const bool sound = !(i0 < 0 || i1 < i0 || i1 > M || skipped);
+    auto draft_logit = [&](int64_t r) {
+        const int64_t local = (int64_t)load_input(draft_ids + r) - col0;
+        return local >= 0 && local < V_local ? Elem<T>::load_l2(logits + (r * ld + local) * ES) : -INFINITY;
+    };
+    float x = -INFINITY;
+    if (sound && sub == 0 && i0 + tid / G < i1) x = draft_logit(i0 + tid / G);
+    pdl_wait();
+    if (!sound) return;
+    const bool internal = *err_word == epoch;
     for (int64_t base = i0; base < i1; base += kFinishThreads / G) {
         const bool mine = base + tid / G < i1;
         const int64_t r = mine ? base + tid / G : base;
-        float x = -INFINITY;
-        if (mine && sub == 0) {
-            const int64_t local = (int64_t)draft_ids[r] - col0;
-            if (local >= 0 && local < V_local) x = Elem<T>::load(logits + (r * ld + local) * ES);
-        }
+        if (base > i0 && mine && sub == 0) x = draft_logit(r);
         const float2 ms = merge_partials<G>(partials + r * P, P, sub);
         if (mine && sub == 0) {
             stats[3 * r + 0] = internal ? __uint_as_float(kStatsInternal) : ms.x;
