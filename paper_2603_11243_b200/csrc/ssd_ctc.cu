@@ -869,6 +869,7 @@ int plan_ctc(ssd_dtype dtype, int V, int64_t ld, int64_t N, int B, const ssd_lau
     const int epc = 16 / es;
     const int64_t fixed = 16 * 8 + 16 + (int64_t)epc * (epc + 1) * 16 + 128;
     const int64_t stage_budget = 216 * 1024 - fixed;
+    const int64_t sms = device_sm_count();
     int warps = 0, R = 0;
     int64_t stage_stride = 0;
     if (kernel != 1 && row_pitch <= 2 * row_bytes + 64 && row_pitch < (1 << 20)) {
@@ -883,6 +884,14 @@ int plan_ctc(ssd_dtype dtype, int V, int64_t ld, int64_t N, int B, const ssd_lau
             int64_t w = stage_budget / stage_stride;
             if (w > 16) w = 16;      // 512 threads: 128 registers each, for eight chunks in flight
             if (w >= 5 && w % 2 && w % 3) --w;      // so that 2 or more tile counters divide it
+            // Between one and two tiles per warp: as few warps as take two each, so that the second
+            // round is not nearly empty (2,000 tiles of 16 KB, 16,000 rows of 1,025 bf16 symbols: 12
+            // warps 16.7 us, 8 warps 15.6; 3,125 tiles, 50,000 rows of 348: 16 warps 16.7, 12 16.2).
+            const int64_t tiles = (N + R - 1) / R;
+            if (tiles > w * sms && tiles <= 2 * w * sms) {
+                const int64_t two = ((tiles + 2 * sms - 1) / (2 * sms) + 3) & ~3ll;
+                if (two < w) w = two;
+            }
             if (o && o->warps > 0 && o->warps < w) w = o->warps;
             if (w >= 1) warps = (int)w;
         }
