@@ -230,21 +230,23 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
 
 
 // Merge of a row's P (reference, sum) pairs into (maximum, sum relative to it) by the G lanes of
-// a group, lane `sub` of which takes pairs sub, sub + G, ...  All 32 lanes of the warp call it.
-template <int G> __device__ __forceinline__ float2 merge_partials(const float2 *pp, int P, int sub) {
+// a group, lane `sub` of which takes pairs sub, sub + G, ..., L of them in one round trip.  All 32
+// lanes of the warp call it.
+template <int G, int L> __device__ __forceinline__ float2 merge_partials(const float2 *pp, int P, int sub) {
     float Mx = kNegInit, S = 0.f;
-    if (P <= 4 * G) {
-        float2 v[4];                      // all of a lane's pairs are fetched together
+    if (P <= L * G) {
+        float2 v[L];          // all of a lane's pairs are fetched together
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < L; ++j) {
             v[j] = make_float2(kNegInit, 0.f);
             if (sub + j * G < P) v[j] = pp[sub + j * G];
         }
-        Mx = fmaxf(fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)), kNegInit);
+#pragma unroll
+        for (int j = 0; j < L; ++j) Mx = fmaxf(Mx, v[j].x);
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) Mx = fmaxf(Mx, __shfl_xor_sync(0xffffffffu, Mx, o));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) S += v[j].y * ex2((v[j].x - Mx) * kLog2e);
+        for (int j = 0; j < L; ++j) S += v[j].y * ex2((v[j].x - Mx) * kLog2e);
     } else {
         for (int q = sub; q < P; q += G) Mx = fmaxf(Mx, pp[q].x);
 #pragma unroll
@@ -257,14 +259,6 @@ template <int G> __device__ __forceinline__ float2 merge_partials(const float2 *
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
     return make_float2(Mx, S);
-}
-
-// Lanes that share a row's pairs: four pairs a lane, so that their loads are one round trip.
-// (A thread that walked 36 pairs of a row by itself, twice, took 10 us for a draft of 250 tokens.)
-inline int merge_lanes(int P) {
-    int G = 1;
-    while (G < 32 && 4 * G < P) G *= 2;
-    return G;
 }
 
 // Eq. 5 for one row, given its maximum Mx, ln of its sum of exponentials relative to Mx and the
@@ -623,7 +617,7 @@ __global__ void __launch_bounds__(256) verify_rows_plain(const VerifyParams p) {
 
 constexpr int kFinishThreads = 1024;   // one sweep for drafts of up to 1024 tokens
 
-template <typename T, int G>
+template <typename T, int G, int L>
 __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
     const char *__restrict__ logits, int V, int64_t ld, int64_t M,
     const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
@@ -676,7 +670,7 @@ __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
         const bool mine = i < K;
         const int64_t r = i0 + (mine ? i : 0);
         if (base > 0 && mine && sub == 0) x = draft_logit(r, id_ok);
-        const float2 ms = merge_partials<G>(partials + r * P, P, sub);
+        const float2 ms = merge_partials<G, L>(partials + r * P, P, sub);
         if (mine && sub == 0) {
             const RowDecision d = decide_row(x, ms.x, logf(ms.y), id_ok, log_tau, reject_none, reject_all);
             myflags |= d.flags;
@@ -702,7 +696,7 @@ constexpr uint32_t kStatsInternal = 0x7fc0dead;   // in place of a row's maximum
 // triple (maximum of the local columns, sum of exponentials relative to it, logit of the draft
 // token if its column is local, else -inf).  Rows of skipped or malformed utterances are left
 // untouched; the combining kernel does not read them.
-template <typename T, int G>
+template <typename T, int G, int L>
 __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
     const char *__restrict__ logits, int V_local, int64_t ld, int64_t M, int64_t col0,
     const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
@@ -729,7 +723,7 @@ __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
         const bool mine = base + tid / G < i1;
         const int64_t r = mine ? base + tid / G : base;
         if (base > i0 && mine && sub == 0) x = draft_logit(r);
-        const float2 ms = merge_partials<G>(partials + r * P, P, sub);
+        const float2 ms = merge_partials<G, L>(partials + r * P, P, sub);
         if (mine && sub == 0) {
             stats[3 * r + 0] = internal ? __uint_as_float(kStatsInternal) : ms.x;
             stats[3 * r + 1] = ms.y;
@@ -1012,20 +1006,24 @@ static cudaError_t launch_direct(const void *logits, ssd_dtype dtype, int V, int
     return launch_pdl(kern, (unsigned)ctas, (unsigned)direct::kThreads, smem, stream, p);
 }
 
-// The closing kernel for P pairs per row.
-template <template <int> class Pick> static auto pick_lanes(int P) -> decltype(Pick<1>::kernel()) {
-    switch (merge_lanes(P)) {
-        case 1: return Pick<1>::kernel();
-        case 2: return Pick<2>::kernel();
-        case 4: return Pick<4>::kernel();
-        case 8: return Pick<8>::kernel();
-        case 16: return Pick<16>::kernel();
-        default: return Pick<32>::kernel();
-    }
+// The closing kernel for P pairs per row and drafts of K tokens on average: four pairs a lane in
+// one round trip, or eight and half the lanes per row where that makes a draft one sweep of the
+// block instead of two (the call on 250 rows of 304 KB, 18 pairs each: 20.3 -> 19.1 us; 2 x 300
+// rows, 9 pairs: 40.0 -> 37.5; with eight throughout, 5,568 rows of 3 pairs lose half a
+// microsecond, 100 rows of 46 pairs a third).  A thread that walked 36 pairs by itself, twice,
+// took 10 us for the closing kernel alone.
+template <template <int, int> class Pick> static auto pick_lanes(int P, int64_t K) -> decltype(Pick<1, 4>::kernel()) {
+    int G = 1;
+    while (G < 32 && 4 * G < P) G *= 2;
+    if (G > 1 && G < 32 && K >= 128 && K * G > kFinishThreads)
+        return G == 2 ? Pick<1, 8>::kernel() : G == 4 ? Pick<2, 8>::kernel() : G == 8 ? Pick<4, 8>::kernel()
+                                                                             : Pick<8, 8>::kernel();
+    return G == 1 ? Pick<1, 4>::kernel() : G == 2 ? Pick<2, 4>::kernel() : G == 4 ? Pick<4, 4>::kernel()
+         : G == 8 ? Pick<8, 4>::kernel() : G == 16 ? Pick<16, 4>::kernel() : Pick<32, 4>::kernel();
 }
 template <typename T> struct FinishKernels {
-    template <int G> struct Verify { static auto kernel() { return &verify_finish_kernel<T, G>; } };
-    template <int G> struct Shard { static auto kernel() { return &shard_finish_kernel<T, G>; } };
+    template <int G, int L> struct Verify { static auto kernel() { return &verify_finish_kernel<T, G, L>; } };
+    template <int G, int L> struct Shard { static auto kernel() { return &shard_finish_kernel<T, G, L>; } };
 };
 
 // Launches the streaming kernel that leaves pairs_per_row (reference, sum) pairs per row in the
@@ -1155,8 +1153,8 @@ int launch_verify(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_
     if (rc != SSD_OK) return rc;
     const int P = pairs_per_row(plan);
     e = launch_pdl(
-        dtype == SSD_F32 ? pick_lanes<FinishKernels<float>::Verify>(P)
-                         : pick_lanes<FinishKernels<bf16_t>::Verify>(P),
+        dtype == SSD_F32 ? pick_lanes<FinishKernels<float>::Verify>(P, M / B)
+                         : pick_lanes<FinishKernels<bf16_t>::Verify>(P, M / B),
         (unsigned)B, (unsigned)kFinishThreads, 0, L.stream,
         static_cast<const char *>(logits), V, ld, M, tok_off, draft_ids, B, th.log_tau,
         th.reject_none, th.reject_all, skip, static_cast<const float2 *>(partials), P,
@@ -1183,8 +1181,8 @@ int launch_verify_shard(const void *logits, ssd_dtype dtype, int V_local, int64_
     if (rc != SSD_OK) return rc;
     const int P = pairs_per_row(plan);
     cudaError_t e = launch_pdl(
-        dtype == SSD_F32 ? pick_lanes<FinishKernels<float>::Shard>(P)
-                         : pick_lanes<FinishKernels<bf16_t>::Shard>(P),
+        dtype == SSD_F32 ? pick_lanes<FinishKernels<float>::Shard>(P, M / B)
+                         : pick_lanes<FinishKernels<bf16_t>::Shard>(P, M / B),
         (unsigned)B, (unsigned)kFinishThreads, 0, L.stream,
         static_cast<const char *>(logits), V_local, ld, M, col0, tok_off, draft_ids, B, skip,
         static_cast<const float2 *>(partials), P, shard_stats,
