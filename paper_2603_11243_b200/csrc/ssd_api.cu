@@ -195,7 +195,7 @@ int32_t ssd_verify(const void *logits, ssd_dtype dtype, int32_t V, int64_t ld,
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{logits, ld, false});
+    int rc = plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{logits, ld, false, skip != nullptr});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < plan.workspace_bytes ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))
@@ -217,7 +217,7 @@ int32_t ssd_verify_shard(const void *logits, ssd_dtype dtype, int32_t V_local, i
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V_local, dtype, opts, &plan, RowsAt{logits, ld, false});
+    int rc = plan_for_query(B, M, V_local, dtype, opts, &plan, RowsAt{logits, ld, false, skip != nullptr});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < plan.workspace_bytes ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))
@@ -297,7 +297,7 @@ int32_t ssd_verify_early_exit(const void *logits, ssd_dtype dtype, int32_t V, in
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{logits, ld, false});
+    int rc = plan_for_query(B, M, V, dtype, opts, &plan, RowsAt{logits, ld, false, skip != nullptr});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < verify_ee_workspace_bytes(B, plan) ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))

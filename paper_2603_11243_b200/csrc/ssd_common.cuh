@@ -474,6 +474,7 @@ struct RowsAt {
     const void *base;
     int64_t ld;
     bool greedy;
+    bool skip;             // some utterances' rows may not be read
 };
 int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts *opts,
                 const RowsAt &at, VerifyPlan *plan);

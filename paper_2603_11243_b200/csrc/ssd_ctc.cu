@@ -420,10 +420,11 @@ __device__ __forceinline__ void reduce_tile(const CtcParams &p, uint32_t stage_a
             const float sc = has ? ex2(d) : 0.f;         // a lane without chunks adds nothing
             const float S = group_sum<G>(Sl * sc);
             const float A2 = group_sum<G>(fmaf(d, Sl, Al) * sc);
-            // fast logarithm and division: absolute error near 1e-6, far inside the tolerance
-            const float lnS = __logf(S);
+            // not __logf, whose absolute error of 4e-7 near 1 is what a confident frame's entropy of
+            // 1e-3 nats would be off by
+            const float lnS = logf(S);
             out.lse = m + (lnS - ml * kLn2);
-            out.H = fmaxf(lnS - kLn2 * __fdividef(A2, S), 0.f);
+            out.H = fmaxf(lnS - kLn2 * (A2 / S), 0.f);
             if (!(S > 0.5f) || !(S < INFINITY) || !(fabsf(m) < INFINITY))
                 out.H = __int_as_float(0x7fc00000);
         }

@@ -862,7 +862,8 @@ unsigned long long next_epoch();
 //     31.1 / 28.6)
 //   bf16, aligned rows of 96 KB and more: the ring while the power cap does not bite (1,500 of
 //     98 KB: 31.9 / 33.7; 8,000: 136 / 141), direct beyond (12,000: 200 / 200; 16,000: 265 / 245;
-//     22,000 of 200 KB: 708 / 664): it spends a fifth fewer instructions on a logit.
+//     22,000 of 200 KB: 708 / 664): it spends a fifth fewer instructions on a logit.  With `skip`
+//     half of the rows are taken to be read (a batch of 1.3 GB, partly gated: 199 / 206).
 //   fp32: the ring (16,000 of 192 KB: 437 / 455; 1,000: 36.1 / 38.8), which has more bytes in
 //     flight and half the logits per byte; the greedy step on few rows: direct (200 of 196 KB:
 //     14.0 / 12.3; 300 of 608 KB: 36.4 / 35.8; 500 of 196 KB: 21.9 / 23.3)
@@ -873,7 +874,7 @@ static int use_direct(int64_t M, int64_t row_bytes, ssd_dtype dtype, int kernel,
     if (o && (o->kernel || o->warps || o->stages || o->stage_bytes || o->fma_exp || o->finish)) return 0;
     const bool few = M < 4ll * sms;
     if (dtype == SSD_F32) return at.greedy && M <= 2ll * sms;
-    if (at.greedy || few || row_bytes < 96 * 1024 || M * row_bytes >= 1200ll << 20) return 1;
+    if (at.greedy || few || row_bytes < 96 * 1024 || M * row_bytes >= (at.skip ? 2400ll : 1200ll) << 20) return 1;
     return (reinterpret_cast<uintptr_t>(at.base) | (uintptr_t)(at.ld * 2)) % 16 != 0;
 }
 
