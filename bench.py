@@ -36,7 +36,7 @@ SMALL_SET_BYTES = 2e9           # below this, three input sets are rotated so th
                                 # inputs in the 126 MB L2; above it one set is many times the L2
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "ncu_traffic.json")
 KERNEL_SOURCES = ["ssd_common.cuh", "ssd_stream.cuh", "ssd_ranges.cuh", "ssd_ctc.cu", "ssd_verify.cu",
-                  "ssd_api.cu"]
+                  "ssd_api.cu", "ssd_direct.cuh"]
 
 
 def parse_args():
@@ -388,7 +388,7 @@ def run_per_config(device, peak, peak_kind, skip_idx, cpu=True):
                "step_frac_of_nominal": round(step_bytes / (ms / K * 1e-3) / 1e9 / NOMINAL_HBM_GBS, 4),
                "l2": l2_note(sets),
                "roofline_ctc": roof("ctc_rows_tma", ctc_b, t_ctc, peak, peak_kind),
-               "roofline_verify": roof("verify_rows_tma", ver_b, t_ver, peak, peak_kind)}
+               "roofline_verify": roof("verify_rows", ver_b, t_ver, peak, peak_kind)}
         if cpu:
             rec["cpu_baseline"] = cpu_baseline(sets[0], budget_s=2.5)
         rec["seconds_spent"] = round(time.time() - t0, 1)
@@ -448,7 +448,8 @@ def run_ours(args):
 
     # ---- the streaming kernels alone, on KERNEL_LAUNCHES further steps that carry events ------
     t_ctc, t_ver, ctc_bytes, ver_bytes = time_kernels(sets, 3 if args.ncu_small else KERNEL_LAUNCHES)
-    vkern = "verify_rows_tma" if args.verify_mode == "full" else "verify_rows_ee"
+    # ssd_verify picks its streaming kernel by size and type: direct loads or the ring
+    vkern = "verify_rows" if args.verify_mode == "full" else "verify_rows_ee"
 
     # ---- end to end: pinned host buffers in, decisions out, every step ---------------------
     e2e = None
