@@ -193,6 +193,8 @@ int32_t ssd_entropy_gate(const float *frame_entropy, const int64_t *frame_off,
  *   all_accepted[b] = (accepted_len[b] == K_b): Eq. 5 holds (vacuously for K_b = 0)
  * tau_slm <= 0 rejects nothing; tau_slm >= 1 rejects everything.  A NaN likelihood or a
  * draft id outside [0,V) is a rejected position.
+ * Logits below -1e30 count as -inf: masking with the type's lowest finite value is masking with
+ * -inf, a row of nothing else included.
  * skip [B] u8 (nullable): nonzero = the utterance was already accepted by the gate; its rows
  * are not read, accepted_len = K_b, all_accepted = 1, its token_logp / row_lse untouched.
  *

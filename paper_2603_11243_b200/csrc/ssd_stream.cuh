@@ -146,13 +146,21 @@ __device__ __forceinline__ void add_chunks(uint32_t a0, int n, int ct, int NT, O
     }
 }
 
+// The reference that goes with a largest element cm (-inf: still none): never below kNegInit.
+// A mask of the type's lowest finite value would otherwise be one, its product with log2e would
+// leave fp32's range, and a thread that met nothing else would report its row as not finite.
+// Against kNegInit such elements add 0, as they do in the closing kernels' merge.
+__device__ __forceinline__ float reference_of(float cm) {
+    return cm > -INFINITY ? fmaxf(cm, kNegInit) : cm;
+}
+
 template <typename T, int kF, bool kArg>
 __device__ __forceinline__ void consume_stage(uint32_t a0, int n, int ct, int NT, Online &st,
                                               int elem0, ArgTrack &at) {
     if (ct >= n) return;
     if (!(st.m > -INFINITY)) {
         // no reference yet (start of a row): the largest element of the first chunk
-        const float cm = chunk_max<T>(lds128(a0 + (uint32_t)ct * 16));
+        const float cm = reference_of(chunk_max<T>(lds128(a0 + (uint32_t)ct * 16)));
         if (cm > -INFINITY) { st.m = cm; st.mh = cm * kLog2e; }
     }
     const Online saved = st;
@@ -163,6 +171,7 @@ __device__ __forceinline__ void consume_stage(uint32_t a0, int n, int ct, int NT
         st = saved;
         float cm = -INFINITY;
         for (int c = ct; c < n; c += NT) cm = fmaxf(cm, chunk_max<T>(lds128(a0 + (uint32_t)c * 16)));
+        cm = reference_of(cm);
         if (cm > st.m) st.raise_to(cm);
         if (st.m > -INFINITY) add_chunks<T, kF, kArg>(a0, n, ct, NT, st, at);
     }
@@ -177,6 +186,13 @@ __device__ __forceinline__ float2 warp_merge(const Online &st) {
     // S == 0 covers lanes that saw nothing (their m is -inf); a NaN sum still propagates
     const float Sw = warp_sum(S == 0.f ? 0.f : S * ex2(fmaf(st.m - M, kLog2e, -ml)));
     return make_float2(M, Sw);
+}
+
+// ln p of a logit x of a row with maximum Mx and lnS the logarithm of its sum relative to it (not
+// x - lse: keeps its accuracy when |x| is large).  NaN, which rejects, for a row with a NaN, a +inf
+// or nothing above kNegInit: of such a row's masked logits none is likely.
+__device__ __forceinline__ float row_logp(float x, float Mx, float lnS) {
+    return fabsf(Mx + lnS) < INFINITY ? (x - Mx) - lnS : __int_as_float(0x7fc00000);
 }
 
 }  // namespace stream

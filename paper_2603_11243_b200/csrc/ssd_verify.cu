@@ -279,7 +279,7 @@ __device__ __forceinline__ RowDecision decide_row(float x, float Mx, float lnS, 
         d.logp = -INFINITY;
         d.reject = true;
     } else {
-        d.logp = (x - Mx) - lnS;      // not x - lse: keeps its accuracy when |x| is large
+        d.logp = row_logp(x, Mx, lnS);
         d.reject = reject_none ? false : (reject_all || !(d.logp > log_tau));
     }
     return d;

@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(576, 1) verify_rows_ee(const EeParams p) {
                     logp = -INFINITY;
                     reject = true;
                 } else {
-                    logp = (sx[slot] - Mx) - lnS;
+                    logp = row_logp(sx[slot], Mx, lnS);
                     reject = p.reject_none ? false : (p.reject_all || !(logp > p.log_tau));   // p <= tau; NaN rejects
                 }
                 if (reject) atomicMin(&p.first_reject[rm.b], rm.pos);

@@ -1,0 +1,113 @@
+"""Rows masked with the type's lowest finite value, with -1e9 or with -inf, through every kernel that
+streams logits rows: all of them give the oracle's values, whatever share of a row is masked."""
+import numpy as np
+import pytest
+import torch
+
+import helpers as H
+from oracle import ref
+from paper_2603_11243_b200 import binding as ssd
+
+pytestmark = pytest.mark.gpu
+
+M, V, B = 60, 20011, 3
+# the default choice, the ring (whole rows, column spans), the ring that finishes its rows itself,
+# and plain loads
+KERNELS = {"auto": {}, "ring": dict(kernel=2, split=1), "spans": dict(kernel=2, split=3),
+           "fin": dict(kernel=2, finish=2, split=1), "plain": dict(kernel=1)}
+
+
+def _inputs(dtype, mask):
+    """Rows 4k: a prefix is masked; 4k+1: everything but one logit; 4k+2: everything but a hundred;
+    4k+3: nothing.  The draft token is one that is left, the largest of its row."""
+    g = torch.Generator().manual_seed(dtype.itemsize)
+    x = torch.randn((M, V), generator=g)
+    for r in range(M):
+        keep = torch.zeros(V, dtype=torch.bool)
+        if r % 4 == 0:
+            keep[12000:] = True
+        elif r % 4 == 1:
+            keep[(r * 331) % V] = True
+        elif r % 4 == 2:
+            keep[torch.randint(0, V, (100,), generator=g)] = True
+        else:
+            keep[:] = True
+        x[r, ~keep] = mask
+    x = x.to(dtype)
+    ids = x.float().argmax(1).to(torch.int32)
+    x[torch.arange(M), ids.long()] = 12.0
+    return x, torch.tensor([0, 20, 20, M]), ids
+
+
+def _masks(dtype):
+    return (torch.finfo(dtype).min, -1.0e9, float("-inf"))
+
+
+def _want(x, off, ids, tau):
+    return ref.verify(H.storage_numpy(x), V, off.numpy(), ids.numpy(), float(np.float32(tau)))
+
+
+@pytest.mark.parametrize("kernel", KERNELS)
+@pytest.mark.parametrize("which", range(3))
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_verify(cuda_device, dtype, which, kernel):
+    x, off, ids = _inputs(dtype, _masks(dtype)[which])
+    dev = cuda_device
+    out = ssd.ssd_verify(x.to(dev), off.to(dev), ids.to(dev), 0.1, opts=H.opts(**KERNELS[kernel]))
+    torch.cuda.synchronize()
+    H.compare_stage2(out, _want(x, off, ids, 0.1), off.numpy(), 0.1)
+
+
+@pytest.mark.parametrize("which", range(3))
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_early_exit_and_shard(cuda_device, dtype, which):
+    x, off, ids = _inputs(dtype, _masks(dtype)[which])
+    dev = cuda_device
+    xd, offd, idsd = x.to(dev), off.to(dev), ids.to(dev)
+    want = _want(x, off, ids, 0.1)
+    o = H.opts(ctas=4, split=1)              # fifteen rows per CTA: the early-exit kernel itself
+    ee = ssd.alloc_early_exit_outputs(M, B, V, ssd.BF16 if dtype == torch.bfloat16 else ssd.F32, dev, o)
+    ssd.ssd_verify_early_exit(xd, offd, idsd, 0.1, out=ee, opts=o)
+    torch.cuda.synchronize()
+    assert (ee["rows_read"].cpu() >= 0).all()
+    H.compare_stage2(ee, want, off.numpy(), 0.1)
+    # the second shard's columns are masked altogether in most of the first rows
+    cut = 12000
+    for opts in (None, H.opts(kernel=2)):
+        stats = torch.stack([
+            ssd.ssd_verify_shard(xd[:, a:b], a, offd, idsd, opts=opts) for a, b in ((0, cut), (cut, V))])
+        both = ssd.ssd_verify_combine(stats, V, offd, idsd, 0.1)
+        torch.cuda.synchronize()
+        H.compare_stage2(both, want, off.numpy(), 0.1)
+
+
+@pytest.mark.parametrize("which", range(3))
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_greedy(cuda_device, dtype, which):
+    x, _, ids = _inputs(dtype, _masks(dtype)[which])
+    want = ref.greedy_step(H.storage_numpy(x), V)
+    for opts in (None, H.opts(kernel=2), H.opts(kernel=2, split=3)):
+        got = ssd.ssd_greedy_step(x.to(cuda_device), opts=opts)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(got["next_token"].cpu().numpy(), want["next_token"])
+        assert not got["row_status"].any()
+        assert np.abs(got["row_lse"].cpu().numpy() - want["row_lse"]).max() <= H.FLOAT_TOL
+
+
+@pytest.mark.parametrize("kernel", KERNELS)
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_a_row_of_the_lowest_value_alone(cuda_device, dtype, kernel):
+    """Nothing is left of such a row: reported and rejected as a row of only -inf is, by every kernel."""
+    x = torch.full((8, V), torch.finfo(dtype).min, dtype=dtype)
+    x[4:] = 0.0
+    off, ids = torch.tensor([0, 4, 8]), torch.zeros(8, dtype=torch.int32)
+    dev = cuda_device
+    out = ssd.ssd_verify(x.to(dev), off.to(dev), ids.to(dev), 1e-6, opts=H.opts(**KERNELS[kernel]))
+    torch.cuda.synchronize()
+    assert H.status_u32(out["utt_status"]).tolist() == [ssd.UTT_NONFINITE, 0]
+    assert out["accepted_len"].tolist() == [0, 4]
+    o = H.opts(ctas=1, split=1)
+    ee = ssd.ssd_verify_early_exit(x.to(dev), off.to(dev), ids.to(dev), 1e-6, opts=o)
+    torch.cuda.synchronize()
+    assert H.status_u32(ee["utt_status"]).tolist() == [ssd.UTT_NONFINITE, 0]
+    assert ee["accepted_len"].tolist() == [0, 4]
