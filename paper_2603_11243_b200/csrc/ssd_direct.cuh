@@ -23,6 +23,12 @@ namespace direct {
 using ranges::kDirectBlockBytes;
 
 constexpr int kThreads = 512, kWarps = kThreads / 32, kCtasPerSm = 2;
+// A lane's sums are joined to its total every so many blocks (even).  With one logit far above the
+// rest in them, sums absorb what each unit adds up to half an ulp: up to 2^-25 of the row's
+// probability a term, for every term that is added one by one.  Of 297 blocks (152,064 bf16
+// logits in one span) that made 9e-6; 16 and 19 joins make 1e-6, below the 3e-6 of a ring thread
+// with its 99 chunks.
+constexpr int kGroupBlocks = 16;
 constexpr float kSpanSumLimit = 1.0e27f;   // below every value a clamped exponential can take
 
 struct DirectParams {
@@ -285,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
         const int64_t slot = (int64_t)cur.row * p.spans + cur.sp;
         const float my_edge = edge;
         const int my_edge_idx = edge_idx, my_unit_elem = unit_elem;
-        float vmax = -INFINITY, Sw = 0.f;
+        float vmax = -INFINITY, Sw = 0.f, total = 0.f;
         int vblk = 0;
         float2 Sa = make_float2(0.f, 0.f), Sb = Sa;
         ref.set<T>(warp_max(fmaxf(unit_max<T>(u), my_edge)));
@@ -298,12 +304,17 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
             }
             add_unit<T, kF>(d, ref, Sa, Sb);
         };
+        while (k > 2) {
+            const int stop = max(2, k - kGroupBlocks);
 #pragma unroll 1
-        for (; k > 2; k -= 2) {
-            load_next(v);
-            add(u, blocks - 1 - k);
-            load_next(u);
-            add(v, blocks - k);
+            for (; k > stop; k -= 2) {
+                load_next(v);
+                add(u, blocks - 1 - k);
+                load_next(u);
+                add(v, blocks - k);
+            }
+            total += (Sa.x + Sa.y) + (Sb.x + Sb.y);
+            Sa = Sb = make_float2(0.f, 0.f);
         }
         if (k == 2) {
             load_next(v);
@@ -325,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
         }
         if (fast) {
             add(u, last);
-            Sw = warp_sum((Sa.x + Sa.y) + (Sb.x + Sb.y) + ex2(fmaf(my_edge, kLog2e, ref.nmh)));
+            Sw = warp_sum(total + ((Sa.x + Sa.y) + (Sb.x + Sb.y) + ex2(fmaf(my_edge, kLog2e, ref.nmh))));
             fast = Sw < kSpanSumLimit;
             Sw *= ex2(-fmaf(ref.m, kLog2e, ref.nmh));   // every exponent carried m*log2e + nmh
         }

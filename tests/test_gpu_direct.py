@@ -133,3 +133,40 @@ def test_malformed_offsets(cuda_device):
     b = _verify(view, off, ids, cuda_device, wide, 0, skip, H.opts(kernel=1))
     for k in ("accepted_len", "all_accepted", "utt_status"):
         assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("V", [n * 512 + d for n in (16, 17, 18, 19, 34, 35) for d in (-1, 0, 1)])
+def test_groups_of_blocks(cuda_device, V):
+    """One span a row, whose blocks end just before, on and after the groups that a lane sums apart."""
+    wide, view, ids = _rows(9, V, 0, V)
+    off = _offsets([4, 5])
+    out = _verify(view, off, ids, cuda_device, wide, 0, opts=H.opts(split=1))
+    orc = ref.verify(H.storage_numpy(view.contiguous()), V, off.numpy(), ids.numpy(), float(np.float32(0.1)))
+    H.compare_stage2(out, orc, off.numpy(), 0.1, require_all_margins=False)
+    got = ssd.ssd_greedy_step(wide.to(cuda_device)[:, :V], opts=H.opts(split=1))
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(got["next_token"].cpu().numpy(), ref.greedy_step(H.storage_numpy(view.contiguous()), V)["next_token"])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", [49152, 152064])
+def test_small_terms_behind_a_peak(cuda_device, V, dtype):
+    """A row's first block (1 KB) holds equal peaks, the rest of the row lies 17 below them: what a
+    unit of it adds to a lane's sum of the peaks is under half an ulp, all of it together is 1.2e-5
+    of the row."""
+    x = torch.full((4, V), -23.0, dtype=dtype)
+    peaks = 1024 // x.element_size()
+    x[:, :peaks] = -6.0
+    want = -6.0 + np.log(peaks + (V - peaks) * np.exp(-17.0))
+    # the terms added one by one: 16 blocks of a group, the groups, four sums, a tree of 32 lanes; each
+    # loses at most 2^-25 of the sum.  An exponential is good to 2^-22, the result to an ulp of it.
+    terms = 16 + -(-V // (16 * peaks)) + 4 + 5
+    bound = terms * 2.0 ** -25 + 2.0 ** -22 + 2.0 ** -23 * abs(want)
+    off = torch.tensor([0, 4]).to(cuda_device)
+    ids = torch.zeros(4, dtype=torch.int32, device=cuda_device)
+    got = [ssd.ssd_greedy_step(x.to(cuda_device), opts=H.opts(split=1))]
+    if dtype == torch.bfloat16:
+        got.append(ssd.ssd_verify(x.to(cuda_device), off, ids, 0.1, opts=H.opts(split=1)))
+    torch.cuda.synchronize()
+    for o in got:
+        assert np.abs(o["row_lse"].cpu().numpy().astype(np.float64) - want).max() <= bound
