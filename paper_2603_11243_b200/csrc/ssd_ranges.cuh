@@ -19,6 +19,16 @@ namespace ranges {
 SSD_HD uintptr_t align_down16(uintptr_t a) { return a & ~(uintptr_t)15; }
 SSD_HD uintptr_t align_up16(uintptr_t a) { return (a + 15) & ~(uintptr_t)15; }
 
+// ---- utterances: the rows [i0, i1) that two neighbouring offsets name, of a matrix of M ---------
+// The offsets are the caller's data and may hold anything: no arithmetic before this check.
+SSD_HD bool rows_sound(int64_t i0, int64_t i1, int64_t M) { return i0 >= 0 && i1 >= i0 && i1 <= M; }
+
+// Row number k of an utterance, -1 where it has none (or its offsets are malformed): what a thread
+// of a closing kernel may fetch before the streaming kernel is through.
+SSD_HD int64_t row_of_utterance(int64_t i0, int64_t i1, int64_t M, int k) {
+    return rows_sound(i0, i1, M) && k < i1 - i0 ? i0 + k : -1;
+}
+
 // ---- frame statistics: one tile = R consecutive rows, fetched as one contiguous range --------
 // The tile's bytes are [gstart, gend).  Its 16-byte-aligned superset [f0, c1) is what lands in
 // the stage (stage byte 0 holds address f0).  Where that superset would leave the matrix

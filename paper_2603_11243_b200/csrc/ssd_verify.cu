@@ -644,11 +644,12 @@ __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
     };
     float x = 0.f;
     bool id_ok = false;
-    if (i0 >= 0 && i1 <= M && sub == 0 && i0 + tid / G < i1 && !skipped) x = draft_logit(i0 + tid / G, id_ok);
+    const int64_t first = skipped || sub != 0 ? -1 : ranges::row_of_utterance(i0, i1, M, tid / G);
+    if (first >= 0) x = draft_logit(first, id_ok);
     pdl_wait();
     const unsigned long long err = *err_word;
     const uint32_t internal = (err == epoch) ? (uint32_t)SSD_UTT_INTERNAL : 0u;
-    if (i0 < 0 || i1 < i0 || i1 > M) {
+    if (!ranges::rows_sound(i0, i1, M)) {
         if (tid == 0) {
             accepted_len[b] = 0; all_accepted[b] = 0;
             utt_status[b] = SSD_UTT_BAD_OFFSETS | internal;
@@ -709,13 +710,14 @@ __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
     if (M == 0) pdl_wait();        // no streaming kernel of this call before this one
     const int64_t i0 = load_input(tok_off + b), i1 = load_input(tok_off + b + 1);
     const bool skipped = skip != nullptr && load_input(skip + b) != 0;
-    const bool sound = !(i0 < 0 || i1 < i0 || i1 > M || skipped);
+    const bool sound = ranges::rows_sound(i0, i1, M) && !skipped;
     auto draft_logit = [&](int64_t r) {
         const int64_t local = (int64_t)load_input(draft_ids + r) - col0;
         return local >= 0 && local < V_local ? Elem<T>::load_l2(logits + (r * ld + local) * ES) : -INFINITY;
     };
     float x = -INFINITY;
-    if (sound && sub == 0 && i0 + tid / G < i1) x = draft_logit(i0 + tid / G);
+    const int64_t first = !sound || sub != 0 ? -1 : ranges::row_of_utterance(i0, i1, M, tid / G);
+    if (first >= 0) x = draft_logit(first);
     pdl_wait();
     if (!sound) return;
     const bool internal = *err_word == epoch;
