@@ -31,6 +31,8 @@ struct Launch {
 // predecessor's tail, and let their successor be scheduled after it: the closing kernel of the
 // same call then begins when everything before the streaming kernel is complete, and fetches
 // (from L2, load_input) what the caller passed in while the streaming kernel still runs.
+// For the same reason no kernel's input is a `const *__restrict__`: that says nothing writes to it
+// while the kernel lives, and lets its loads be moved in front of the wait.
 __device__ __forceinline__ void pdl_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

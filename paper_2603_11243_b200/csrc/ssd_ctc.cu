@@ -680,8 +680,8 @@ __device__ __forceinline__ MaxAt block_max_at(MaxAt x, MaxAt *scratch /* [32] sh
 }
 
 __global__ void __launch_bounds__(kUttThreads) collapse_kernel(
-    const int32_t *__restrict__ frame_argmax, const float *__restrict__ frame_entropy,
-    const int64_t *__restrict__ frame_off, int B, int64_t N, int blank_id, int cap,
+    const int32_t *frame_argmax, const float *frame_entropy,
+    const int64_t *frame_off, int B, int64_t N, int blank_id, int cap,
     int32_t *__restrict__ draft_tokens, int32_t *__restrict__ draft_frames,
     int32_t *__restrict__ draft_len, int32_t *__restrict__ draft_full_len,
     float *__restrict__ utt_max_entropy, uint32_t *__restrict__ utt_status,
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(kUttThreads) collapse_kernel(
 }
 
 __global__ void __launch_bounds__(kUttThreads) gate_kernel(
-    const float *__restrict__ frame_entropy, const int64_t *__restrict__ frame_off, int B,
+    const float *frame_entropy, const int64_t *frame_off, int B,
     int64_t N, float tau, uint8_t *__restrict__ gate_accept, float *__restrict__ max_entropy,
     int32_t *__restrict__ argmax_frame) {
     __shared__ MaxAt scratch[32];
@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(kUttThreads) gate_kernel(
 // largest frame entropy is below tau and no frame was NaN (status bits), its offsets were sound
 // and no wait ran out.  An utterance without frames has maximum 0.
 __global__ void __launch_bounds__(256) gate_from_maxima_kernel(
-    const float *__restrict__ utt_max_entropy, const uint32_t *__restrict__ utt_status, int B,
+    const float *utt_max_entropy, const uint32_t *utt_status, int B,
     float tau, uint8_t *__restrict__ gate_accept, float *__restrict__ max_entropy) {
     pdl_enter();
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) {

@@ -23,8 +23,8 @@ struct SweepPairs {
 
 // One warp per (pair, utterance): 32 log-likelihoods per step, stops at the first reject.
 __global__ void __launch_bounds__(256) sweep_kernel(
-    const float *__restrict__ utt_max_entropy, const float *__restrict__ token_logp,
-    const int64_t *__restrict__ tok_off, int B, int64_t M, const SweepPairs pairs,
+    const float *utt_max_entropy, const float *token_logp,
+    const int64_t *tok_off, int B, int64_t M, const SweepPairs pairs,
     uint8_t *__restrict__ gate_accept, int32_t *__restrict__ accepted_len,
     uint8_t *__restrict__ all_accepted, int32_t *__restrict__ counts) {
     pdl_enter();
@@ -65,9 +65,9 @@ __global__ void __launch_bounds__(256) sweep_kernel(
 // utterances left to the auto-regressive pass (a block scan over the utterances).
 constexpr int kAssembleThreads = 256;
 __global__ void __launch_bounds__(kAssembleThreads) assemble_kernel(
-    const int32_t *__restrict__ tokens, const int64_t *__restrict__ tok_off, int B, int64_t M,
-    const uint8_t *__restrict__ gate_accept, const int32_t *__restrict__ accepted_len,
-    const uint8_t *__restrict__ all_accepted, int32_t *__restrict__ final_tokens,
+    const int32_t *tokens, const int64_t *tok_off, int B, int64_t M,
+    const uint8_t *gate_accept, const int32_t *accepted_len,
+    const uint8_t *all_accepted, int32_t *__restrict__ final_tokens,
     int32_t *__restrict__ final_len, uint8_t *__restrict__ is_final,
     int32_t *__restrict__ ar_count, int32_t *__restrict__ ar_utt, int32_t *__restrict__ ar_resume) {
     __shared__ int warp_tot[2][kAssembleThreads / 32];

@@ -619,10 +619,10 @@ constexpr int kFinishThreads = 1024;   // one sweep for drafts of up to 1024 tok
 
 template <typename T, int G, int L>
 __global__ void __launch_bounds__(kFinishThreads) verify_finish_kernel(
-    const char *__restrict__ logits, int V, int64_t ld, int64_t M,
-    const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
-    float log_tau, int reject_none, int reject_all, const uint8_t *__restrict__ skip,
-    const float2 *__restrict__ partials, int P, float *__restrict__ token_logp,
+    const char *logits, int V, int64_t ld, int64_t M,
+    const int64_t *tok_off, const int32_t *draft_ids, int B,
+    float log_tau, int reject_none, int reject_all, const uint8_t *skip,
+    const float2 *partials, int P, float *__restrict__ token_logp,
     float *__restrict__ row_lse, int32_t *__restrict__ accepted_len,
     uint8_t *__restrict__ all_accepted, uint32_t *__restrict__ utt_status,
     const unsigned long long *err_word, unsigned long long epoch) {
@@ -699,9 +699,9 @@ constexpr uint32_t kStatsInternal = 0x7fc0dead;   // in place of a row's maximum
 // untouched; the combining kernel does not read them.
 template <typename T, int G, int L>
 __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
-    const char *__restrict__ logits, int V_local, int64_t ld, int64_t M, int64_t col0,
-    const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
-    const uint8_t *__restrict__ skip, const float2 *__restrict__ partials, int P,
+    const char *logits, int V_local, int64_t ld, int64_t M, int64_t col0,
+    const int64_t *tok_off, const int32_t *draft_ids, int B,
+    const uint8_t *skip, const float2 *partials, int P,
     float *__restrict__ stats, const unsigned long long *err_word, unsigned long long epoch) {
     constexpr int ES = Elem<T>::kBytes;
     pdl_launch_dependents();
@@ -739,9 +739,9 @@ __global__ void __launch_bounds__(kFinishThreads) shard_finish_kernel(
 // one shard that owns the column has it), then Eq. 5 and the first reject exactly as in
 // verify_finish_kernel.
 __global__ void __launch_bounds__(kFinishThreads) combine_kernel(
-    const float *__restrict__ stats_all, int R, int64_t V_total, int64_t M,
-    const int64_t *__restrict__ tok_off, const int32_t *__restrict__ draft_ids, int B,
-    float log_tau, int reject_none, int reject_all, const uint8_t *__restrict__ skip,
+    const float *stats_all, int R, int64_t V_total, int64_t M,
+    const int64_t *tok_off, const int32_t *draft_ids, int B,
+    float log_tau, int reject_none, int reject_all, const uint8_t *skip,
     float *__restrict__ token_logp, float *__restrict__ row_lse,
     int32_t *__restrict__ accepted_len, uint8_t *__restrict__ all_accepted,
     uint32_t *__restrict__ utt_status) {
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(kFinishThreads) combine_kernel(
 constexpr int kGreedyWarps = 8;
 template <typename T>
 __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
-    const char *__restrict__ logits, int V, int64_t ld, int64_t R, const float4 *__restrict__ partials, int P, int32_t *__restrict__ next_token,
+    const char *logits, int V, int64_t ld, int64_t R, const float4 *partials, int P, int32_t *__restrict__ next_token,
     float *__restrict__ next_logp, float *__restrict__ row_lse, uint32_t *__restrict__ row_status,
     const unsigned long long *err_word, unsigned long long epoch) {
     pdl_enter();

@@ -102,7 +102,7 @@ __device__ __forceinline__ void atom_add_u64_if(unsigned long long &dst, unsigne
 
 // ---- set-up: per-utterance words and the largest draft length ---------------------------------
 __global__ void __launch_bounds__(1024) ee_init_kernel(
-    const int64_t *__restrict__ tok_off, const uint8_t *__restrict__ skip, int B, int64_t M,
+    const int64_t *tok_off, const uint8_t *skip, int B, int64_t M,
     int32_t *__restrict__ first_reject, uint32_t *__restrict__ flags,
     int32_t *__restrict__ rows_read, int32_t *__restrict__ kmax,
     unsigned long long *__restrict__ next_item, unsigned long long first_free) {
@@ -481,9 +481,9 @@ __global__ void __launch_bounds__(576, 1) verify_rows_ee(const EeParams p) {
 }
 
 __global__ void __launch_bounds__(256) ee_finish_kernel(
-    const int64_t *__restrict__ tok_off, const uint8_t *__restrict__ skip, int B, int64_t M,
-    const int32_t *__restrict__ first_reject, const uint32_t *__restrict__ flags,
-    const int32_t *__restrict__ rows_read_ws, int32_t *__restrict__ accepted_len,
+    const int64_t *tok_off, const uint8_t *skip, int B, int64_t M,
+    const int32_t *first_reject, const uint32_t *flags,
+    const int32_t *rows_read_ws, int32_t *__restrict__ accepted_len,
     uint8_t *__restrict__ all_accepted, uint32_t *__restrict__ utt_status,
     int32_t *__restrict__ rows_read, const unsigned long long *err_word,
     unsigned long long epoch) {
