@@ -121,45 +121,77 @@ __device__ __forceinline__ void add_unit(const Unit &v, const Reference &ref, fl
     Sb = fadd2(Sb, tb);
 }
 
-// A span whose sums left fp32's range, or whose first block holds no finite logit to refer to
-// (masked logits, NaN, +inf, a magnitude beyond 4096): two passes over its elements.
+// A span whose sums left fp32's range, or whose first block holds no logit to refer to (masked
+// logits, NaN, +inf, a magnitude beyond 4096), read again with a running maximum per lane: one pass
+// in the same 32-byte units.  Masked vocabularies come here, a prefix of 1 KB is enough, so it must
+// not cost much more than the fast pass.  (One element a lane and step, and a pass of its own for
+// the maximum, took 800 us for 16,000 rows of 98 KB with a masked first half that take 273 unmasked;
+// this takes MEASURED.)
 struct SpanResult {
     float m, S, vmax;
     int vidx;
 };
-template <typename T>
-__device__ __noinline__ SpanResult span_exact(const DirectParams &p, int64_t row, int sp, int lane) {
+template <typename T, bool kArg>
+__device__ __noinline__ SpanResult span_running_max(const DirectParams &p, int64_t row, int sp, int lane) {
     constexpr int ES = Elem<T>::kBytes;
+    constexpr float kLowest = -3.402823466e38f;      // finite, so that x - m is -inf or 0 for a masked x
     const char *x = p.logits + row * p.row_pitch;
     const ranges::RowUnits ru = ranges::row_units(reinterpret_cast<uintptr_t>(x), p.row_bytes);
     const ranges::UnitSpan us = ranges::unit_span(ru, p.spans, sp, p.span_blocks);
-    const int n = (us.hi - us.lo) / ES, first = us.lo / ES;
-    x += us.lo;
+    int rest = us.uhi - us.ulo - lane * 32;
+    const char *at = x + us.ulo + lane * 32;
+    const int e = lane < 16 ? us.lo + lane * ES : us.uhi + (lane - 16) * ES;
+    float edge = -INFINITY;
+    if (e < (lane < 16 ? us.ulo : us.hi)) edge = Elem<T>::load(x + e);
+    // (x - m) * log2e throughout, not x * log2e - m * log2e: a mask of the type's lowest value would
+    // leave fp32's range there
+    float m = fmaxf(edge, kLowest), S = ex2((edge - m) * kLog2e), total = 0.f, vmax = -INFINITY;
+    int blk = 0, vblk = 0;
+    auto add = [&](const Unit &d) {
+        const float um = unit_max<T>(d);
+        if (kArg && um > vmax) { vmax = um; vblk = blk; }
+        if (um > m) {
+            const float sc = ex2((m - um) * kLog2e);
+            S *= sc;
+            total *= sc;
+            m = um;
+        }
+        const float2 nm = make_float2(-m, -m), sc = make_float2(kLog2e, kLog2e);
+        float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+            float2 a[2];
+            if (ES == 4) {
+                a[0] = make_float2(__uint_as_float(d.r[k]), __uint_as_float(d.r[k + 1]));
+                a[0] = fmul2(fadd2(a[0], nm), sc);
+                t = fadd2(t, make_float2(ex2(a[0].x), ex2(a[0].y)));
+            } else {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    a[q] = fmul2(fadd2(make_float2(bf16_lo(d.r[k + q]), bf16_hi(d.r[k + q])), nm), sc);
+                    a[q] = make_float2(ex2(a[q].x), ex2(a[q].y));
+                }
+                t = fadd2(t, fadd2(a[0], a[1]));
+            }
+        }
+        S += t.x + t.y;
+        if (++blk % kGroupBlocks == 0) { total += S; S = 0.f; }
+    };
+#pragma unroll 1
+    for (; rest > 0; rest -= kDirectBlockBytes, at += kDirectBlockBytes) add(load_unit(at));
     SpanResult r;
+    r.m = warp_max(m);
+    r.S = warp_sum((S + total) * ex2((m - r.m) * kLog2e));
     r.vmax = -INFINITY;
     r.vidx = INT_MAX;
-    for (int i = lane; i < n; i += 32) {
-        const float v = Elem<T>::load(x + (size_t)i * ES);
-        if (v > r.vmax) { r.vmax = v; r.vidx = first + i; }
+    if (kArg) {
+        r.vmax = warp_max(fmaxf(vmax, edge));
+        int idx = INT_MAX;
+        if (edge == r.vmax && edge > -INFINITY) idx = e / ES;
+        if (vmax == r.vmax && vmax > -INFINITY)
+            idx = min(idx, us.ulo / ES + lane * (32 / ES) + vblk * (kDirectBlockBytes / ES));
+        r.vidx = __reduce_min_sync(0xffffffffu, idx);
     }
-    const float vm = warp_max(r.vmax);
-    r.vidx = __reduce_min_sync(0xffffffffu, r.vmax == vm ? r.vidx : INT_MAX);
-    r.vmax = r.m = vm;
-    float S = 0.f;
-    if (vm > -INFINITY) {
-        // (x - vm) * log2e, not x * log2e - vm * log2e: a mask of the type's lowest value would
-        // leave fp32's range there
-        for (int i = lane; i < n; i += 32) S += ex2((Elem<T>::load(x + (size_t)i * ES) - vm) * kLog2e);
-        S = warp_sum(S);
-    } else {
-        // only -inf adds nothing; NaN has to show
-        for (int i = lane; i < n; i += 32) {
-            const float v = Elem<T>::load(x + (size_t)i * ES);
-            if (v != v) S = v;
-        }
-        S = warp_sum(S);
-    }
-    r.S = S;
     return r;
 }
 
@@ -283,9 +315,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
         if (rest > 0) d = load_unit(at);
     };
 
+    auto begin = [&](Unit &d) {
+        open();
+        if (blocks > 1) load_next(d); else load_last(d);
+    };
+
     Unit u, v;
-    open();
-    if (blocks > 1) load_next(u); else load_last(u);
+    begin(u);
     for (;;) {
         Reference ref;
         const int64_t slot = (int64_t)cur.row * p.spans + cur.sp;
@@ -330,10 +366,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
         // the next span's first block is on its way before this span is finished
         step();
         settle();
-        if (cur.valid) {
-            open();
-            if (blocks > 1) load_next(v); else load_last(v);
-        }
+        if (cur.valid) begin(v);
         if (fast) {
             add(u, last);
             Sw = warp_sum(total + ((Sa.x + Sa.y) + (Sb.x + Sb.y) + ex2(fmaf(my_edge, kLog2e, ref.nmh))));
@@ -355,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
                 out.vidx = __reduce_min_sync(0xffffffffu, idx);
             }
         } else {
-            out = span_exact<T>(p, slot / p.spans, (int)(slot % p.spans), lane);
+            out = span_running_max<T, kArg>(p, slot / p.spans, (int)(slot % p.spans), lane);
         }
         if (lane == 0) {
             if (kArg) reinterpret_cast<float4 *>(p.partials)[slot] =
