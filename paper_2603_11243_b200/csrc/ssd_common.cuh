@@ -453,6 +453,14 @@ int launch_gate_from_maxima(const float *utt_max_entropy, const uint32_t *utt_st
                             float tau, uint8_t *gate_accept, float *max_entropy,
                             cudaStream_t stream);
 
+namespace direct {
+// Column spans per row, one warp and one pair each, and 1 KB blocks per span.
+struct Cut {
+    int spans, blocks;
+};
+constexpr int kCuts = 6;
+}  // namespace direct
+
 struct VerifyPlan {
     int kernel;        // 1 plain loads, 2 bulk-copy pipeline
     int ctas;
@@ -464,8 +472,8 @@ struct VerifyPlan {
     int partials;      // partial (max, sum) pairs per row = split * warps
     int finish_inside; // rows are finalised inside the streaming kernel (no closing kernel)
     int direct;        // rows are streamed by the direct-load kernel
-    int spans;         // direct-load kernel: column spans per row, one warp and one pair each
-    int span_blocks;   // direct-load kernel: blocks per span
+    direct::Cut cut[direct::kCuts];   // direct-load kernel: how rows are cut, for M, M/2, M/4 ... read
+    int pairs;         // direct-load kernel: pairs per row, the most spans of any cut
     int direct_ctas;
     size_t smem_bytes;
     size_t fin_smem_bytes;

@@ -33,16 +33,16 @@ constexpr float kSpanSumLimit = 1.0e27f;   // below every value a clamped expone
 
 struct DirectParams {
     const char *logits;
-    int V;
     int64_t row_pitch;
     int row_bytes;
     int64_t M;
-    int spans, span_blocks;   // column spans per row, blocks per span (see plan_spans)
+    Cut cut[kCuts];        // how rows are cut: cut[k] where at most M >> k of them are read
+    int pairs;             // pairs per row in `partials`
     const int64_t *tok_off;
     int B;
     const uint8_t *skip;
     int table;             // count the rows to read per utterance in shared memory first
-    void *partials;        // [M, spans] float2 (reference, sum), or float4 with the arg max
+    void *partials;        // [M, pairs] float2 (reference, sum), or float4 with the arg max
 };
 
 // One lane's 32-byte piece of a block.
@@ -131,13 +131,15 @@ struct SpanResult {
     float m, S, vmax;
     int vidx;
 };
+// It takes what it needs by value: with the address of the kernel's parameters taken, every thread of
+// the kernel began by copying them to local memory (the call on 5,568 rows of 24 KB: 32.3 us, now
+// 29.6; the greedy step on 1,024 rows of 304 KB: 54.9, now 51.7).
 template <typename T, bool kArg>
-__device__ __noinline__ SpanResult span_running_max(const DirectParams &p, int64_t row, int sp, int lane) {
+__device__ __noinline__ SpanResult span_running_max(const char *x, int row_bytes, Cut cut, int sp, int lane) {
     constexpr int ES = Elem<T>::kBytes;
     constexpr float kLowest = -3.402823466e38f;      // finite, so that x - m is -inf or 0 for a masked x
-    const char *x = p.logits + row * p.row_pitch;
-    const ranges::RowUnits ru = ranges::row_units(reinterpret_cast<uintptr_t>(x), p.row_bytes);
-    const ranges::UnitSpan us = ranges::unit_span(ru, p.spans, sp, p.span_blocks);
+    const ranges::RowUnits ru = ranges::row_units(reinterpret_cast<uintptr_t>(x), row_bytes);
+    const ranges::UnitSpan us = ranges::unit_span(ru, cut.spans, sp, cut.blocks);
     int rest = us.uhi - us.ulo - lane * 32;
     const char *at = x + us.ulo + lane * 32;
     const int e = lane < 16 ? us.lo + lane * ES : us.uhi + (lane - 16) * ES;
@@ -222,6 +224,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     pdl_wait();
     pdl_launch_dependents();
     int rows = (int)p.M;
+    Cut cut = p.cut[0];
     if (table) {
         const int per = (p.B + kThreads - 1) / kThreads, b0 = (int)threadIdx.x * per;
         int32_t mine = 0;
@@ -245,6 +248,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
             total += t;
         }
         rows = total;
+#pragma unroll
+        for (int q = 1; q < kCuts; ++q)
+            if (rows <= (int)(p.M >> q)) cut = p.cut[q];
         for (int b = b0; b < min(p.B, b0 + per); ++b) act[b] += before;
         if (threadIdx.x == 0) act[p.B] = total;
         __syncthreads();
@@ -253,16 +259,17 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     // item k of warp w is number w + k * (warps of the grid) of the rows * spans items, counted
     // so that neighbours go to different CTAs
     const unsigned gw = blockIdx.x + gridDim.x * warp, GW = gridDim.x * kWarps;
-    const int da = (int)(GW / (unsigned)p.spans), ds = (int)(GW % (unsigned)p.spans);
+    const unsigned ns = (unsigned)cut.spans;
+    const int da = (int)(GW / ns), ds = (int)(GW % ns);
     Cursor cur;
-    cur.a = (int)(gw / (unsigned)p.spans);
-    cur.sp = (int)(gw % (unsigned)p.spans);
+    cur.a = (int)(gw / ns);
+    cur.sp = (int)(gw % ns);
     cur.b = -1;
     cur.shift = 0;
     int b_end = 0;                       // rows to read up to and with utterance b
     auto step = [&]() {
         cur.a += da; cur.sp += ds;
-        if (cur.sp >= p.spans) { cur.sp -= p.spans; ++cur.a; }
+        if (cur.sp >= cut.spans) { cur.sp -= cut.spans; ++cur.a; }
     };
     auto settle = [&]() {
         if (table) {
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     auto open = [&]() {
         const char *x = p.logits + (int64_t)cur.row * p.row_pitch;
         const ranges::RowUnits ru = ranges::row_units(reinterpret_cast<uintptr_t>(x), p.row_bytes);
-        const ranges::UnitSpan us = ranges::unit_span(ru, p.spans, cur.sp, p.span_blocks);
+        const ranges::UnitSpan us = ranges::unit_span(ru, cut.spans, cur.sp, cut.blocks);
         const int bytes = us.uhi - us.ulo;
         at = x + us.ulo + lane * 32;
         blocks = (bytes + kDirectBlockBytes - 1) / kDirectBlockBytes;
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     begin(u);
     for (;;) {
         Reference ref;
-        const int64_t slot = (int64_t)cur.row * p.spans + cur.sp;
+        const int row = cur.row, sp = cur.sp;
         const float my_edge = edge;
         const int my_edge_idx = edge_idx, my_unit_elem = unit_elem;
         float vmax = -INFINITY, Sw = 0.f, total = 0.f;
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
         float2 Sa = make_float2(0.f, 0.f), Sb = Sa;
         ref.set<T>(warp_max(fmaxf(unit_max<T>(u), my_edge)));
         bool fast = fabsf(ref.m) < 4096.f;
-        int k = fast ? blocks - 1 : 0;      // blocks that follow the one in u
+        int left = fast ? blocks - 1 : 0;   // blocks that follow the one in u
         auto add = [&](const Unit &d, int blk) {
             if (kArg) {
                 const float m = unit_max<T>(d);
@@ -340,24 +347,24 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
             }
             add_unit<T, kF>(d, ref, Sa, Sb);
         };
-        while (k > 2) {
-            const int stop = max(2, k - kGroupBlocks);
+        while (left > 2) {
+            const int stop = max(2, left - kGroupBlocks);
 #pragma unroll 1
-            for (; k > stop; k -= 2) {
+            for (; left > stop; left -= 2) {
                 load_next(v);
-                add(u, blocks - 1 - k);
+                add(u, blocks - 1 - left);
                 load_next(u);
-                add(v, blocks - k);
+                add(v, blocks - left);
             }
             total += (Sa.x + Sa.y) + (Sb.x + Sb.y);
             Sa = Sb = make_float2(0.f, 0.f);
         }
-        if (k == 2) {
+        if (left == 2) {
             load_next(v);
             add(u, blocks - 3);
             load_last(u);
             add(v, blocks - 2);
-        } else if (k == 1) {
+        } else if (left == 1) {
             load_last(v);
             add(u, blocks - 2);
             u = v;
@@ -388,12 +395,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
                 out.vidx = __reduce_min_sync(0xffffffffu, idx);
             }
         } else {
-            out = span_running_max<T, kArg>(p, slot / p.spans, (int)(slot % p.spans), lane);
+            out = span_running_max<T, kArg>(p.logits + (int64_t)row * p.row_pitch, p.row_bytes, cut, sp, lane);
         }
-        if (lane == 0) {
-            if (kArg) reinterpret_cast<float4 *>(p.partials)[slot] =
+        if (kArg) {
+            if (lane == 0) reinterpret_cast<float4 *>(p.partials)[(int64_t)row * p.pairs + sp] =
                 make_float4(out.m, out.S, out.vmax, __int_as_float(out.vidx));
-            else reinterpret_cast<float2 *>(p.partials)[slot] = make_float2(out.m, out.S);
+        } else {
+            // pairs that this cut has no span for add nothing
+            const int at = sp + lane * cut.spans;
+            if (at < p.pairs) reinterpret_cast<float2 *>(p.partials)[(int64_t)row * p.pairs + at] =
+                lane == 0 ? make_float2(out.m, out.S) : make_float2(kNegInit, 0.f);
         }
         if (!cur.valid) return;
         u = v;
@@ -410,17 +421,37 @@ inline bool table_fits(int B, int64_t M) {
 // three blocks' worth of instructions of its own (reference, merge, the next span's addresses).
 // (A finer cut of the rows that do not fill a round, so that every warp gets the same bytes, was
 // slower throughout: 22.4 against 21.1 us on 250 rows of 304 KB, 95 against 93.5 on 5,568 of 98.)
-inline void plan_spans(int64_t M, int64_t row_bytes, int warps, int most, int *spans, int *span_blocks) {
+inline Cut plan_spans(int64_t M, int64_t row_bytes, int warps, int most) {
     const int64_t nb = row_blocks(row_bytes);
     int64_t best = 0;
+    Cut cut{1, (int)nb};
     for (int rounds = 1; rounds <= 16; ++rounds) {
         int64_t ns = M > 0 ? (int64_t)rounds * warps / M : 1;
         ns = ns < 1 ? 1 : ns > most ? most : ns;
         const int64_t bps = (nb + ns - 1) / ns;
         ns = (nb + bps - 1) / bps;
         const int64_t cost = (M * ns + warps - 1) / warps * (bps + 3);
-        if (best == 0 || cost < best) { best = cost; *span_blocks = (int)bps; *spans = (int)ns; }
+        if (best == 0 || cost < best) { best = cost; cut = Cut{(int)ns, (int)bps}; }
         if (M > 0 && (int64_t)rounds * warps / M >= most) break;
+    }
+    return cut;
+}
+
+// With `skip` only the kernel knows how many rows are read, and the cut for all of a large batch's rows
+// leaves most warps without one where few are.  So such a batch (a row per warp and more) has a cut
+// for every halving of its rows, of up to eight spans, and the kernel takes the one for what its table
+// counted.  One cut, cuts, and the ring for comparison, us: 43,000 rows of 200 KB of which 330 are
+// read 58.5, 21.1, 22.4; 46,000 of 304 KB, 990: 117, 66.7, 72.0; 30,000 of 98 KB, 2,800: 62.4, 50.4,
+// 53.0; all 43,000: 1,276, 1,270, 1,361.  (pairs > spans of a cut only here: at most sixteen, a lane
+// each.)
+constexpr int kMostSpansSkipping = 8;
+inline void plan_cuts(int64_t M, int64_t row_bytes, int warps, int most, bool may_skip, Cut *cut, int *pairs) {
+    cut[0] = plan_spans(M, row_bytes, warps, most);
+    *pairs = cut[0].spans;
+    const int fine = most < kMostSpansSkipping ? most : kMostSpansSkipping;
+    for (int k = 1; k < kCuts; ++k) {
+        cut[k] = may_skip && M >= warps ? plan_spans(M >> k, row_bytes, warps, fine) : cut[0];
+        if (cut[k].spans > *pairs) *pairs = cut[k].spans;
     }
 }
 

@@ -949,11 +949,13 @@ int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts 
     if (pl.direct) {
         pl.direct_ctas = (o && o->ctas > 0) ? o->ctas : direct::kCtasPerSm * sms;
         if (o && o->split > 0) {
-            pl.spans = split;
-            pl.span_blocks = (direct::row_blocks(row_bytes) + split - 1) / split;
+            pl.pairs = split;
+            for (direct::Cut &c : pl.cut)
+                c = direct::Cut{split, (direct::row_blocks(row_bytes) + split - 1) / split};
         } else {
-            direct::plan_spans(M, row_bytes, pl.direct_ctas * direct::kWarps,
-                               pl.partials < 64 ? pl.partials : 64, &pl.spans, &pl.span_blocks);
+            direct::plan_cuts(M, row_bytes, pl.direct_ctas * direct::kWarps,
+                              pl.partials < 64 ? pl.partials : 64, at.skip && direct::table_fits(B, M),
+                              pl.cut, &pl.pairs);
         }
     }
     // header | two words per utterance | partials
@@ -984,7 +986,7 @@ static size_t partials_offset(int B) {
 }
 
 // Pairs per row that the streaming kernel of a plan leaves.
-static int pairs_per_row(const VerifyPlan &plan) { return plan.direct ? plan.spans : plan.partials; }
+static int pairs_per_row(const VerifyPlan &plan) { return plan.direct ? plan.pairs : plan.partials; }
 
 // fp32 logits come here with the arg max only (see use_direct).
 template <bool kArg>
@@ -994,11 +996,12 @@ static cudaError_t launch_direct(const void *logits, ssd_dtype dtype, int V, int
     const int es = dtype == SSD_F32 ? 4 : 2;
     direct::DirectParams p{};
     p.logits = static_cast<const char *>(logits);
-    p.V = V; p.row_pitch = ld * es; p.row_bytes = V * es; p.M = M;
-    p.spans = plan.spans; p.span_blocks = plan.span_blocks;
+    p.row_pitch = ld * es; p.row_bytes = V * es; p.M = M;
+    for (int k = 0; k < direct::kCuts; ++k) p.cut[k] = plan.cut[k];
+    p.pairs = plan.pairs;
     p.tok_off = tok_off; p.B = B; p.skip = skip; p.partials = partials;
     p.table = skip && direct::table_fits(B, M);
-    const int64_t items = M * plan.spans;
+    const int64_t items = M * plan.pairs;
     const int64_t ctas = items < plan.direct_ctas ? items : plan.direct_ctas;
     const size_t smem = p.table ? (size_t)(B + 1) * sizeof(int32_t) : 0;
     // one pair in eight on the FMA pipe is the best split under the power cap (22,000 rows of

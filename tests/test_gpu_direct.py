@@ -170,3 +170,40 @@ def test_small_terms_behind_a_peak(cuda_device, V, dtype):
     torch.cuda.synchronize()
     for o in got:
         assert np.abs(o["row_lse"].cpu().numpy().astype(np.float64) - want).max() <= bound
+
+
+@pytest.mark.parametrize("V,col0", [(700, 0), (8003, 1)])
+@pytest.mark.parametrize("B", [64, 2046, 2500])
+def test_shares_of_a_large_batch(cuda_device, B, V, col0):
+    """More rows than warps, all, half, and ever fewer of them read: the row counts around those at
+    which the kernel changes its cut; with 2,500 utterances it cannot count and keeps one."""
+    M, dev = 5000, cuda_device
+    g = torch.Generator(device=dev).manual_seed(V + B)
+    wide = torch.randn((M, V + 3), generator=g, device=dev).bfloat16()
+    x = wide[:, col0:col0 + V]
+    ids = torch.randint(0, V, (M,), generator=g, device=dev, dtype=torch.int32)
+    # utterance lengths of 1 and more, so that the rows read can be set to one
+    rng = np.random.default_rng(B)
+    cuts = np.sort(rng.choice(np.arange(1, M), size=B - 1, replace=False))
+    off = torch.tensor(np.concatenate([[0], cuts, [M]]), dtype=torch.int64)
+    lens = np.diff(off.numpy())
+    plain = ssd.ssd_verify(x, off.to(dev), ids, 0.1, opts=H.opts(kernel=1))
+    for target in (M, M // 2 + 40, M // 2, M // 4, M // 8 + 1, M // 16, M // 32, M // 32 + 1, 60, 1):
+        skip, left = np.ones(B, np.uint8), target
+        for b in rng.permutation(B):
+            if lens[b] <= left:
+                skip[b], left = 0, left - lens[b]
+        out = ssd.alloc_verify_outputs(M, B, dev, ssd.ssd_verify_workspace_bytes(B, M, V, ssd.BF16))
+        for t in (out["token_logp"], out["row_lse"]):
+            t.fill_(7.0)
+        out["workspace"].fill_(0xff)                     # pairs that nobody writes would be NaN
+        ssd.ssd_verify(x, off.to(dev), ids, 0.1, skip=torch.from_numpy(skip).to(dev), out=out)
+        torch.cuda.synchronize()
+        read = torch.from_numpy(np.repeat(skip == 0, lens)).to(dev)
+        for k in ("token_logp", "row_lse"):
+            d = (out[k][read] - plain[k][read]).abs()
+            assert d.numel() == 0 or float(d.max()) <= H.FLOAT_TOL, (k, target)
+            assert bool((out[k][~read] == 7.0).all()), (k, target)
+        was_read = torch.from_numpy(skip == 0).to(dev)
+        assert torch.equal(out["accepted_len"][was_read], plain["accepted_len"][was_read]), target
+        assert not out["utt_status"].any()

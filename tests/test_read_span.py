@@ -84,6 +84,15 @@ def test_verify_reads_with_forced_shapes():
                 assert r.hi == BASE + mis + _extent(M, V + 3, V, 2)
 
 
+def test_verify_reads_of_a_large_batch():
+    """More rows than the direct-load kernel has warps: the finer cuts that it may take when some are
+    skipped are replayed as well."""
+    for V, pad, mis in itertools.product((1, 700, 4099, 8192), (0, 3), (0, 2, 18)):
+        r = ssd.ssd_verify_read_span(BASE + mis, ssd.BF16, V, V + pad, 5000, B=40)
+        assert r.faults == 0 and r.lo == BASE + mis, (V, pad, mis)
+        assert r.hi == BASE + mis + _extent(5000, V + pad, V, 2), (V, pad, mis)
+
+
 def test_read_span_argument_errors():
     with pytest.raises(ssd.SsdError):
         ssd.ssd_ctc_draft_read_span(BASE + 1, ssd.BF16, 8, 8, 4)        # off the element size
