@@ -7,13 +7,17 @@ module without a built libssd.so, or calling it with host tensors, raises.
 
 The calls of a decoding step, with result buffers given and no launch options, are marshalled by
 _ssd_call (csrc/ssd_call.cpp); whatever it does not take -- it answers None -- goes the general way
-through ctypes, which is also where wrong arguments are named.
+through ctypes, which is also where wrong arguments are named.  Without _ssd_call.so, or with one
+built for another torch, every call goes that way.
 """
 import ctypes as C
 import os
+import warnings
 from typing import Callable, Dict, List, Optional
 
 import torch
+
+from . import build as _build
 
 F32, BF16 = 0, 1
 UTT_NONFINITE, UTT_BAD_DRAFT_ID, UTT_BAD_OFFSETS, UTT_INTERNAL = 1, 2, 4, 0x80000000
@@ -45,16 +49,26 @@ _lib = None
 _call = None
 
 
+class _Declines:
+    """In the place of a _ssd_call that cannot be used: every call goes the general way."""
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _native():
     global _call
     if _call is None:
         lib()
         try:
-            from . import _ssd_call
+            from . import _ssd_call as call
+            want = "_ssd_call for " + _build.built_for()
+            if call.built_for != want:
+                raise ImportError("it is %r, not %r" % (call.built_for, want))
         except ImportError as e:
-            raise ImportError("_ssd_call.so is not built: run `python -m paper_2603_11243_b200.build` "
-                              "(needs nvcc and a host compiler)") from e
-        _call = _ssd_call
+            warnings.warn("_ssd_call.so cannot be used (%s): calls are marshalled through ctypes, which takes "
+                          "several times longer; run `python -m paper_2603_11243_b200.build`" % e, RuntimeWarning)
+            call = _Declines()
+        _call = call
     return _call
 
 

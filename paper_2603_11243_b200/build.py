@@ -17,6 +17,17 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "--use_fast_math=false", "-Xcompiler", "-fPIC", "-shared", "-cudart", "shared"]
 
 
+def built_for() -> str:
+    """What _ssd_call.so has to have been built with to be usable here: it sees torch's C++ types."""
+    import torch
+    return "torch %s, %s" % (torch.__version__, sysconfig.get_config_var("SOABI"))
+
+
+def _other_torch() -> bool:
+    with open(CALL, "rb") as f:
+        return b"_ssd_call for " + built_for().encode() + b"\0" not in f.read()
+
+
 def _stale(target: str, deps) -> bool:
     if not os.path.exists(target):
         return True
@@ -42,7 +53,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         _run([nvcc] + flags + (["-Xptxas", "-v"] if verbose else []) +
              [os.path.join(CSRC, s) for s in SOURCES] + ["-Xlinker", "-soname=libssd.so", "-o", tmp],
              LIB, tmp, verbose)
-    if force or _stale(CALL, [CALL_SOURCE, HEADER]):
+    if force or _stale(CALL, [CALL_SOURCE, HEADER]) or _other_torch():
         import torch
         root = os.path.dirname(torch.__file__)
         cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
@@ -50,7 +61,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
                os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
         tmp = CALL + ".tmp.%d" % os.getpid()
         _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-              "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] +
+              "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+              '-DSSD_BUILT_FOR="%s"' % built_for()] +
              [f for d in inc for f in ("-isystem", d)] + [CALL_SOURCE, "-o", tmp, "-L" + HERE, "-l:libssd.so",
               "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
               "-Wl,-rpath,$ORIGIN"], CALL, tmp, verbose)

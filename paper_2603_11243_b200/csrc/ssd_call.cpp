@@ -337,6 +337,8 @@ PyMethodDef methods[] = {SSD_METHOD(ctc_draft), SSD_METHOD(gate_from_maxima), SS
                          SSD_METHOD(verify_combine), SSD_METHOD(assemble), SSD_METHOD(greedy_step),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_ssd_call", nullptr, -1, methods};
+// torch's C++ types change from release to release: the binding compares before the first call
+const char kBuiltFor[] = "_ssd_call for " SSD_BUILT_FOR;
 
 }  // namespace
 
@@ -349,5 +351,10 @@ PyMODINIT_FUNC PyInit__ssd_call() {
     SSD_KEY(all_accepted) SSD_KEY(rows_read) SSD_KEY(final_tokens) SSD_KEY(final_len)
     SSD_KEY(is_final) SSD_KEY(ar_count) SSD_KEY(ar_utt) SSD_KEY(ar_resume) SSD_KEY(next_token)
     SSD_KEY(next_logp) SSD_KEY(row_status)
-    return PyModule_Create(&module);
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", kBuiltFor) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
 }

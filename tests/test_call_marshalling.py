@@ -1,9 +1,13 @@
 """The native marshalling of the hot calls: what it does not take goes the general way and raises
 what that raises; what it takes computes what the general way computes."""
+import sys
+import warnings
+
 import pytest
 import torch
 
 import helpers as H
+import paper_2603_11243_b200
 from paper_2603_11243_b200 import binding as ssd
 from paper_2603_11243_b200 import build as ssd_build
 
@@ -45,6 +49,31 @@ def test_errors_are_those_of_the_general_way():
         ssd.ssd_verify_combine(x, 4, off, ids, 0.1, out=out)
     with pytest.raises(KeyError):
         ssd.ssd_verify(x, off, ids, 0.1, out={})
+
+
+@pytest.mark.parametrize("broken", ["absent", "of another torch"])
+def test_without_a_usable_extension_calls_go_the_general_way(monkeypatch, broken):
+    monkeypatch.setattr(ssd, "_call", None)
+    if broken == "absent":
+        monkeypatch.setitem(sys.modules, "paper_2603_11243_b200._ssd_call", None)      # import raises
+        monkeypatch.delattr(paper_2603_11243_b200, "_ssd_call", raising=False)
+    else:
+        monkeypatch.setattr(ssd_build, "built_for", lambda: "torch 1.0, cp30")
+    x, off, ids, out = _verify_inputs("cpu")
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        with pytest.raises(ValueError, match="must be a CUDA tensor"):
+            ssd.ssd_verify(x, off, ids, 0.1, out=out)
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")                                           # said once
+        with pytest.raises(ValueError, match="must be a CUDA tensor"):
+            ssd.ssd_greedy_step(x, out=dict(out, next_token=ids))
+
+
+def test_the_extension_is_rebuilt_for_another_torch(monkeypatch):
+    assert not ssd_build._other_torch()
+    assert ssd._native().built_for == "_ssd_call for " + ssd_build.built_for()
+    monkeypatch.setattr(ssd_build, "built_for", lambda: "torch 1.0, cp30")
+    assert ssd_build._other_torch()
 
 
 @pytest.mark.gpu
