@@ -121,7 +121,8 @@ template <typename Body> PyObject *guarded(Py_ssize_t have, Py_ssize_t want, Bod
     }
 }
 
-void need_dict(PyObject *o) { if (!PyDict_Check(o)) throw Unhandled{}; }
+// a subclass may answer for its items itself
+void need_dict(PyObject *o) { if (!PyDict_CheckExact(o)) throw Unhandled{}; }
 
 // ctc_draft(logits, frame_off, blank_id, max_draft_len, V, out)
 PyObject *ctc_draft(PyObject *, PyObject *const *a, Py_ssize_t n) {

@@ -127,3 +127,94 @@ def test_same_results_both_ways(cuda_device):
     with pytest.raises(ssd.SsdError) as e:
         ssd.ssd_verify(x, off, ids, 0.1, out=dict(out, workspace=out["workspace"][:16]))
     assert e.value.code == ssd.ERR_WORKSPACE
+
+
+@pytest.mark.gpu
+def test_every_hot_call_is_taken_and_computes_the_same(cuda_device, monkeypatch):
+    """The eight functions asked directly: each answers a status, not None.  Then all eight through the
+    binding, natively and with an extension that declines everything."""
+    dev, B, N, M, V = cuda_device, 3, 40, 25, 700
+    g = torch.Generator().manual_seed(8)
+    ctc = torch.randn((N, 60), generator=g).to(dev)
+    logits = torch.randn((M, V), generator=g).bfloat16().to(dev)
+    f_off = torch.tensor([0, 13, 13, N], dtype=torch.int64, device=dev)
+    t_off = torch.tensor([0, 9, 9, M], dtype=torch.int64, device=dev)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32).to(dev)
+    i32, f32, u8 = torch.int32, torch.float32, torch.uint8
+    zeros = lambda n, t: torch.zeros((n,), dtype=t, device=dev)
+
+    def outputs():
+        o = dict(
+            draft=ssd.alloc_ctc_outputs(N, B, dev), gate=dict(gate_accept=zeros(B, u8), max_entropy=zeros(B, f32)),
+            verify=ssd.alloc_verify_outputs(M, B, dev, ssd.ssd_verify_workspace_bytes(B, M, V, ssd.BF16)),
+            early=ssd.alloc_early_exit_outputs(M, B, V, ssd.BF16, dev),
+            stats=torch.zeros((2, M, 3), dtype=f32, device=dev), combine=ssd.alloc_verify_outputs(M, B, dev, 0),
+            final=dict(final_tokens=zeros(M, i32), final_len=zeros(B, i32), is_final=zeros(B, u8),
+                       ar_count=zeros(1, i32), ar_utt=zeros(B, i32), ar_resume=zeros(B, i32)),
+            greedy=dict(next_token=zeros(M, i32), next_logp=zeros(M, f32), row_lse=zeros(M, f32),
+                        row_status=zeros(M, i32),
+                        workspace=zeros(ssd.ssd_greedy_step_workspace_bytes(M, V, ssd.BF16), u8)))
+        for d in o.values():
+            for t in d.values() if isinstance(d, dict) else ():
+                t.zero_()
+        return o
+
+    def native(o):
+        call, d, a, v = ssd._native(), o["draft"], o["gate"], o["verify"]
+        half, ws = V // 2, o["verify"]["workspace"]
+        yield "ctc_draft", call.ctc_draft(ctc, f_off, 0, 10, None, d)
+        yield "gate_from_maxima", call.gate_from_maxima(d["utt_max_entropy"], d["utt_status"], 3.6, a)
+        yield "verify", call.verify(logits, t_off, ids, 0.001, a["gate_accept"], None, v)
+        yield "verify_early_exit", call.verify_early_exit(logits, t_off, ids, 0.001, None, None, o["early"])
+        for r in (0, 1):
+            yield "verify_shard", call.verify_shard(logits[:, r * half:(r + 1) * half], r * half, t_off, ids, None,
+                                                    None, o["stats"][r], ws)
+        yield "verify_combine", call.verify_combine(o["stats"], V, t_off, ids, 0.001, None, o["combine"])
+        yield "assemble", call.assemble(ids, t_off, a["gate_accept"], v["accepted_len"], v["all_accepted"], o["final"])
+        yield "greedy_step", call.greedy_step(logits, None, o["greedy"])
+
+    def bound(o):
+        d, a, v = o["draft"], o["gate"], o["verify"]
+        half, ws = V // 2, o["verify"]["workspace"]
+        ssd.ssd_ctc_draft(ctc, f_off, 0, 10, out=d)
+        ssd.ssd_entropy_gate_from_maxima(d["utt_max_entropy"], d["utt_status"], 3.6, out=a)
+        ssd.ssd_verify(logits, t_off, ids, 0.001, skip=a["gate_accept"], out=v)
+        ssd.ssd_verify_early_exit(logits, t_off, ids, 0.001, out=o["early"])
+        for r in (0, 1):
+            ssd.ssd_verify_shard(logits[:, r * half:(r + 1) * half], r * half, t_off, ids, stats=o["stats"][r],
+                                 workspace=ws)
+        ssd.ssd_verify_combine(o["stats"], V, t_off, ids, 0.001, out=o["combine"])
+        ssd.ssd_assemble(ids, t_off, a["gate_accept"], v["accepted_len"], v["all_accepted"], out=o["final"])
+        ssd.ssd_greedy_step(logits, out=o["greedy"])
+
+    ways = [outputs() for _ in range(3)]
+    for name, rc in native(ways[0]):
+        assert rc == ssd.OK, (name, rc)
+    bound(ways[1])
+    monkeypatch.setattr(ssd, "_call", ssd._Declines())
+    bound(ways[2])
+    torch.cuda.synchronize()
+    assert int(ways[0]["draft"]["draft_len"].sum()) > 0 and int(ways[0]["final"]["ar_count"]) > 0
+    for way in ways[1:]:
+        for part, d in ways[0].items():
+            for k, t in d.items() if isinstance(d, dict) else [("", d)]:
+                if k != "workspace":
+                    assert torch.equal(t, way[part][k] if k else way[part]), (part, k)
+
+
+@pytest.mark.gpu
+def test_a_dict_that_answers_for_itself(cuda_device):
+    """Result buffers in a dict subclass are whatever its item access says, not what it stores."""
+    class Elsewhere(dict):
+        def __getitem__(self, key):
+            return other[key]
+
+        def get(self, key, default=None):
+            return other.get(key, default)
+
+    x, off, ids, out = _verify_inputs(cuda_device)
+    other = {k: torch.zeros_like(t) for k, t in out.items()}
+    out["accepted_len"].fill_(-5)
+    ssd.ssd_verify(x, off, ids, 0.001, out=Elsewhere(out))
+    torch.cuda.synchronize()
+    assert other["accepted_len"].tolist() == [6] and out["accepted_len"].tolist() == [-5]
