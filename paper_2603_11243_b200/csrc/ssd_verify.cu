@@ -800,14 +800,16 @@ __global__ void __launch_bounds__(kFinishThreads) combine_kernel(
 }
 
 // Greedy step: merges the partials of a row, one warp per row.  A partial is (reference, sum,
-// largest logit, an index at or up to one 32-byte unit before its first occurrence): the unit is
-// looked through here, once per row, instead of once per column span in the streaming kernel.
+// largest logit, an index).  The ring's index is that of the logit's first occurrence; the direct-load
+// kernel's (kUnit) lies up to one 32-byte unit before it, and the unit is looked through here, once per
+// row instead of once per column span.  (The look-up is a dependent load: 400 fp32 rows of 128 KB,
+// which the ring reads, 15.3 us with it, 14.3 without; 1,024 of 192 KB 36.5, 35.4.)
 constexpr int kGreedyWarps = 8;
-template <typename T>
+template <typename T, bool kUnit>
 __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
-    const char *logits, int V, int64_t ld, int64_t R, const float4 *partials, int P, int32_t *__restrict__ next_token,
-    float *__restrict__ next_logp, float *__restrict__ row_lse, uint32_t *__restrict__ row_status,
-    const unsigned long long *err_word, unsigned long long epoch) {
+    const char *logits, int V, int64_t ld, int64_t R, const float4 *partials, int P,
+    int32_t *__restrict__ next_token, float *__restrict__ next_logp, float *__restrict__ row_lse,
+    uint32_t *__restrict__ row_status, const unsigned long long *err_word, unsigned long long epoch) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t r = (int64_t)blockIdx.x * kGreedyWarps + (threadIdx.x >> 5);
@@ -830,7 +832,7 @@ __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
     }
     S = warp_sum(S);
     vi = __reduce_min_sync(0xffffffffu, vi);
-    if (vi >= 0 && vi < V) {
+    if (kUnit && vi >= 0 && vi < V) {
         const int64_t e = (int64_t)vi + lane;
         const bool hit = lane < 32 / Elem<T>::kBytes && e < V &&
                          Elem<T>::load(logits + (r * ld + e) * Elem<T>::kBytes) == vm;
@@ -1258,7 +1260,10 @@ int launch_greedy(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_
         e = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_end), L.stream);
         if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     }
-    e = launch_pdl(dtype == SSD_F32 ? greedy_finish_kernel<float> : greedy_finish_kernel<bf16_t>,
+    auto finish = dtype == SSD_F32 ? greedy_finish_kernel<float, false> : greedy_finish_kernel<bf16_t, false>;
+    if (plan.direct)
+        finish = dtype == SSD_F32 ? greedy_finish_kernel<float, true> : greedy_finish_kernel<bf16_t, true>;
+    e = launch_pdl(finish,
                    (unsigned)((R + kGreedyWarps - 1) / kGreedyWarps),
                    (unsigned)(kGreedyWarps * 32), 0, L.stream, p.logits, V, ld, R,
                    static_cast<const float4 *>(partials), pairs_per_row(plan), next_token, next_logp,
