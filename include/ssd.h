@@ -406,6 +406,7 @@ int32_t ssd_verify_combine(const float *stats_all, int32_t R, int64_t V_total,
  *   kernel   2: a kernel of wide reads would run (bulk copies, or 32-byte loads whose units
  *            are held to the row in the same way); 1: the plain-load kernel, which indexes
  *            elements one by one (lo, hi are then the matrix's own extent)
+ *   direct   ssd_verify: 1 where those wide reads are the 32-byte loads
  * so a caller -- the tests do -- can assert faults == 0, lo >= base_addr and
  * hi <= base_addr + ((rows - 1) * ld + V) * element size for any shape and misalignment.
  * Errors: SSD_ERR_NULL, SSD_ERR_ARG, SSD_ERR_DTYPE, SSD_ERR_ALIGN (base_addr not a multiple of
@@ -415,7 +416,7 @@ typedef struct ssd_read_span {
     uint64_t lo, hi;
     int64_t faults;
     int32_t kernel;
-    int32_t reserved;
+    int32_t direct;
 } ssd_read_span;
 int32_t ssd_ctc_draft_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, int64_t ld,
                                 int64_t N, const ssd_launch_opts *opts, ssd_read_span *out);

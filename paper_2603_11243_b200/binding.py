@@ -170,7 +170,7 @@ def ssd_verify_workspace_bytes(B, M, V, dtype_code, opts=None) -> int:
 class ReadSpan(C.Structure):
     """Mirror of ssd_read_span (include/ssd.h)."""
     _fields_ = [("lo", C.c_uint64), ("hi", C.c_uint64), ("faults", C.c_int64),
-                ("kernel", C.c_int32), ("reserved", C.c_int32)]
+                ("kernel", C.c_int32), ("direct", C.c_int32)]
 
 
 def ssd_ctc_draft_read_span(base_addr: int, dtype_code: int, V: int, ld: int, N: int,

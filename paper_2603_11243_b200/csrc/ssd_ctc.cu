@@ -420,8 +420,10 @@ __device__ __forceinline__ void reduce_tile(const CtcParams &p, uint32_t stage_a
             const float sc = has ? ex2(d) : 0.f;         // a lane without chunks adds nothing
             const float S = group_sum<G>(Sl * sc);
             const float A2 = group_sum<G>(fmaf(d, Sl, Al) * sc);
-            // not __logf, whose absolute error of 4e-7 near 1 is what a confident frame's entropy of
-            // 1e-3 nats would be off by
+            // The logarithm and the division are the accurate ones.  That is not what a confident
+            // frame's entropy of 1e-3 nats is off by (1e-6, with __logf too): A holds terms t * 2^t
+            // relative to the lane's first chunk, t up to 17 and more, and is re-based by a
+            // difference of that size.
             const float lnS = logf(S);
             out.lse = m + (lnS - ml * kLn2);
             out.H = fmaxf(lnS - kLn2 * (A2 / S), 0.f);

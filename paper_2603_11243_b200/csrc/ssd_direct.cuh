@@ -29,7 +29,7 @@ constexpr int kThreads = 512, kWarps = kThreads / 32, kCtasPerSm = 2;
 // logits in one span) that made 9e-6; 16 and 19 joins make 1e-6, below the 3e-6 of a ring thread
 // with its 99 chunks.
 constexpr int kGroupBlocks = 16;
-constexpr float kSpanSumLimit = 1.0e27f;   // below every value a clamped exponential can take
+using ranges::kSpanSumLimit;
 
 struct DirectParams {
     const char *logits;
@@ -68,10 +68,8 @@ template <typename T> __device__ __forceinline__ float unit_max(const Unit &v) {
 }
 
 // What a span's exponentials are taken relative to: one logit m of the warp's first block, as
-// nmh = -fl(m * log2e), and for the FMA-pipe exponential a floor and a ceiling around m as
-// packed bf16 pairs.  They are rounded towards m, so that with |m| < 4096 (a bf16 step of at
-// most 16) both stay within [69, 85] of it: the floor's exponential is below 2^-99, the
-// ceiling's between 2^99 and 2^123, which the span's range check sees.
+// nmh = -fl(m * log2e), and for the FMA-pipe exponential a floor and a ceiling around m (ssd_ranges.cuh)
+// as packed bf16 pairs.  |m| < 4096.
 struct Reference {
     float m, nmh;
     uint32_t floor2 = 0, ceil2 = 0;
@@ -79,11 +77,8 @@ struct Reference {
         m = to;
         nmh = -(to * kLog2e);
         if (Elem<T>::kBytes == 2) {
-            uint32_t lo = __float_as_uint(to - 85.f), hi = __float_as_uint(to + 85.f);
-            lo += (lo & 0x80000000u) ? 0u : 0xffffu;
-            hi += (hi & 0x80000000u) ? 0xffffu : 0u;
-            floor2 = (lo >> 16) * 0x10001u;
-            ceil2 = (hi >> 16) * 0x10001u;
+            floor2 = ranges::bf16_floor(to) * 0x10001u;
+            ceil2 = ranges::bf16_ceiling(to) * 0x10001u;
         }
     }
 };

@@ -6,6 +6,7 @@
 #pragma once
 
 #include <stdint.h>
+#include <string.h>
 
 namespace ssd {
 namespace ranges {
@@ -168,6 +169,31 @@ SSD_HD UnitSpan unit_span(const RowUnits &r, int ns, int sp, int per_span) {
     s.hi = sp == ns - 1 ? r.row : s.uhi;
     return s;
 }
+
+// ---- the FMA-pipe exponential's range around a span's reference ------------------------------
+// A floor and a ceiling 85 below and above a bf16 reference m, |m| < 4096, as bf16 bits rounded
+// towards m.  Where 85 more crosses a power of two a bf16 step is as large as 32 (m = 4032: 4117
+// becomes 4096), so both lie within [64, 85] of m.
+SSD_HD uint32_t float_bits(float f) {
+#if defined(__CUDA_ARCH__)
+    return __float_as_uint(f);
+#else
+    uint32_t u;
+    memcpy(&u, &f, sizeof u);
+    return u;
+#endif
+}
+SSD_HD uint32_t bf16_floor(float m) {
+    const uint32_t lo = float_bits(m - 85.f);
+    return (lo + ((lo & 0x80000000u) ? 0u : 0xffffu)) >> 16;
+}
+SSD_HD uint32_t bf16_ceiling(float m) {
+    const uint32_t hi = float_bits(m + 85.f);
+    return (hi + ((hi & 0x80000000u) ? 0xffffu : 0u)) >> 16;
+}
+// Below e^64 = 6.2e27, which the exponential of any ceiling reaches: a span with a logit above its
+// ceiling is over this limit.  A term at its floor is below e^-64 = 1.6e-28 of the reference's.
+constexpr float kSpanSumLimit = 1.0e27f;
 
 }  // namespace ranges
 }  // namespace ssd

@@ -81,7 +81,7 @@ int32_t ssd_ctc_draft_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, 
     out->hi = sp.hi ? sp.hi : base_addr;
     out->faults = sp.faults;
     out->kernel = plan.kernel;
-    out->reserved = 0;
+    out->direct = 0;
     return SSD_OK;
 }
 
@@ -174,7 +174,7 @@ int32_t ssd_verify_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, int
     out->hi = sp.hi ? sp.hi : base_addr;
     out->faults = sp.faults;
     out->kernel = plan.kernel;
-    out->reserved = 0;
+    out->direct = plan.direct;
     return SSD_OK;
 }
 

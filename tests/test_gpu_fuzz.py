@@ -130,6 +130,14 @@ def test_stage2_wide_odd_rows(cuda_device, V, dtype):
     np.testing.assert_array_equal(gr["next_token"].cpu().numpy(), want["next_token"])
 
 
+@pytest.mark.parametrize("V", [50001, 55553, 56700, 100003, 152065])
+def test_stage2_wide_odd_rows_through_the_ring(cuda_device, V, monkeypatch):
+    """The same for the ring on bf16 rows, which take direct loads unless it is asked for."""
+    make = H.opts
+    monkeypatch.setattr(H, "opts", lambda **kw: make(kernel=2, **kw))
+    test_stage2_wide_odd_rows(cuda_device, V, torch.bfloat16)
+
+
 @pytest.mark.parametrize("seed", range(12))
 def test_greedy_random(cuda_device, seed):
     rng = np.random.default_rng(3000 + seed)

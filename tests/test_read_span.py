@@ -72,6 +72,28 @@ def test_verify_reads_stay_inside_each_row(dtype, es):
     assert checked_bulk > 300
 
 
+@pytest.mark.parametrize("dtype,es", [(ssd.F32, 4), (ssd.BF16, 2)])
+def test_verify_reads_of_the_kernel_by_choice_and_of_the_ring(dtype, es):
+    """The same shapes as the library's own choice and with the ring forced, which the early-exit kernel
+    shares its arithmetic with: most bf16 shapes go to direct loads by themselves."""
+    ring = ssd.LaunchOpts()
+    ring.kernel = 2
+    reached = {"ring": 0, "direct": 0}
+    for V in (1, 2, 7, 8, 9, 33, 1000, 4097, 32000, 49152, 49153, 100352, 152065):
+        for pad, M in itertools.product((0, 1, 5), (1, 3, 149, 1200)):
+            if V > 50000 and M > 149:
+                continue
+            for mis in range(0, 16, es) if M < 20 else (0, es):
+                for o in (None, ring):
+                    r = ssd.ssd_verify_read_span(BASE + mis, dtype, V, V + pad, M, B=3, opts=o)
+                    assert r.faults == 0 and r.kernel == 2, (V, pad, M, mis)
+                    assert r.lo == BASE + mis and r.hi == BASE + mis + _extent(M, V + pad, V, es), (V, pad, M, mis)
+                    assert not (o and r.direct)
+                    reached["direct" if r.direct else "ring"] += 1
+    assert reached["ring"] > 400
+    assert reached["direct"] > 400 if dtype == ssd.BF16 else reached["direct"] == 0
+
+
 def test_verify_reads_with_forced_shapes():
     for V, M in itertools.product((7, 1025, 49153), (1, 5, 300)):
         for split, stage_bytes, warps in ((1, 1024, 4), (3, 4096, 16), (7, 1024, 8), (64, 2048, 12),
