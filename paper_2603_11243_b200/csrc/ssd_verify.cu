@@ -58,6 +58,8 @@ template <typename T, int kF, bool kArg>
 __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int ES = Elem<T>::kBytes, EPC = Elem<T>::kPerChunk;
+    // the greedy step's closing kernel reads nothing ahead of its own wait
+    if (kArg) pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = p.stages, CW = p.warps;
     // layout: full[S] | empty[S] | desc[S] | offsets cache | stages
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
         mbar_init_fence();
     }
     pdl_wait();
-    pdl_launch_dependents();
+    if (!kArg) pdl_launch_dependents();
     if (cache_off)
         for (int i = threadIdx.x; i <= p.B; i += blockDim.x) off_cache[i] = p.tok_off[i];
     __syncthreads();
