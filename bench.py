@@ -8,8 +8,10 @@ A step is one pass of the whole path over one ragged batch.  One JSON line is pr
 utterances/s with the inputs resident in HBM, the same metric end to end from pinned host
 buffers, the HBM roofline fraction of the streaming kernels (timed with CUDA events that the
 library records around them, on at least 24 launches whatever K is), the clocks seen under load,
-the CPU oracle timed on the host cores as a reported baseline, and the same figures for the
-other benchmark configurations in `per_config`.  `--impl reference` times that oracle alone.
+the CPU oracle timed on the host cores as a reported baseline, and for every other benchmark
+configuration utterances/s and three fractions of the HBM peak (whole step, frame statistics kernel,
+verification kernel) in `per_config`.  The line is kept under 2,900 characters; `--details FILE`
+writes the whole record.  `--impl reference` times that oracle alone.
 """
 import argparse
 import datetime
@@ -57,6 +59,7 @@ def parse_args():
                     help="full: ssd_verify reads every row of every verified utterance (the "
                          "benchmark metric); early_exit: ssd_verify_early_exit in its place, a "
                          "separate mode whose line says so in config.verify_mode")
+    ap.add_argument("--details", default=None, metavar="FILE", help="write the whole record to FILE")
     ap.add_argument("--sweep", default=None, metavar="FILE",
                     help="time every point of the throughput sweep (configuration 4) and write one "
                          "JSON line per point to FILE instead of the benchmark line")
@@ -290,6 +293,16 @@ def roof(kernel, nbytes, times_ms, peak, peak_kind):
             "min_launch_us": round(best * 1e3, 2)}
 
 
+def verify_kernel(s, w) -> str:
+    """The streaming kernel that ssd_verify runs on this batch: the library picks it by size, type and
+    alignment, and its host-side replay says which."""
+    from paper_2603_11243_b200 import binding as ssd
+    x = s["vb"].logits
+    span = ssd.ssd_verify_read_span(x.data_ptr(), ssd.BF16 if w.dtype == "bf16" else ssd.F32, w.V_llm,
+                                    x.stride(0), x.shape[0], s["B"])
+    return "verify_rows_direct" if span.direct else "verify_rows_tma"
+
+
 def timed_steps(sets, K, W, barrier=None):
     """W warm-up steps, then K steps between two events with a synchronize on both sides.
     Returns (ms for the K steps, wall-clock window, kernels launched in the window)."""
@@ -340,7 +353,7 @@ def l2_note(sets):
 
 
 def workload_string(idx, base, w, batch_lengths):
-    return ("configs[%s] %s: B=%s utterances per GPU, T~%s[%d,%d], V_ctc=%d, V_llm=%d, "
+    return ("configuration %s, %s: B=%s utterances per GPU, T~%s[%d,%d], V_ctc=%d, V_llm=%d, "
             "draft_len<=%d, %s logits (fp32 accumulation)" %
             (idx, base.name,
              w.B if batch_lengths is None else
@@ -349,15 +362,15 @@ def workload_string(idx, base, w, batch_lengths):
              w.t_dist, w.t_lo, w.t_hi, w.V_ctc, w.V_llm, w.max_draft_len, w.dtype))
 
 
-PER_CONFIG = [("configs[1]", 1, None), ("configs[2]", 2, None),
-              ("configs[4] B=64 V_llm=49152 bf16", 4, (64, 49152, "bf16")),
-              ("configs[4] B=64 V_llm=152064 bf16", 4, (64, 152064, "bf16")),
-              ("configs[4] B=64 V_llm=49152 f32", 4, (64, 49152, "f32")),
-              ("configs[4] B=64 V_llm=152064 f32", 4, (64, 152064, "f32")),
-              ("configs[4] B=1024 V_llm=49152 bf16", 4, (1024, 49152, "bf16")),
-              ("configs[4] B=1024 V_llm=49152 f32", 4, (1024, 49152, "f32")),
-              ("configs[4] B=1 V_llm=32000 bf16", 4, (1, 32000, "bf16")),
-              ("configs[4] B=1 V_llm=152064 f32", 4, (1, 152064, "f32"))]
+PER_CONFIG = [("1", 1, None), ("2", 2, None),
+              ("4 B=64 V_llm=49152 bf16", 4, (64, 49152, "bf16")),
+              ("4 B=64 V_llm=152064 bf16", 4, (64, 152064, "bf16")),
+              ("4 B=64 V_llm=49152 f32", 4, (64, 49152, "f32")),
+              ("4 B=64 V_llm=152064 f32", 4, (64, 152064, "f32")),
+              ("4 B=1024 V_llm=49152 bf16", 4, (1024, 49152, "bf16")),
+              ("4 B=1024 V_llm=49152 f32", 4, (1024, 49152, "f32")),
+              ("4 B=1 V_llm=32000 bf16", 4, (1, 32000, "bf16")),
+              ("4 B=1 V_llm=152064 f32", 4, (1, 152064, "f32"))]
 
 
 def run_per_config(device, peak, peak_kind, skip_idx, cpu=True):
@@ -388,7 +401,7 @@ def run_per_config(device, peak, peak_kind, skip_idx, cpu=True):
                "step_frac_of_nominal": round(step_bytes / (ms / K * 1e-3) / 1e9 / NOMINAL_HBM_GBS, 4),
                "l2": l2_note(sets),
                "roofline_ctc": roof("ctc_rows_tma", ctc_b, t_ctc, peak, peak_kind),
-               "roofline_verify": roof("verify_rows", ver_b, t_ver, peak, peak_kind)}
+               "roofline_verify": roof(verify_kernel(sets[0], w), ver_b, t_ver, peak, peak_kind)}
         if cpu:
             rec["cpu_baseline"] = cpu_baseline(sets[0], budget_s=2.5)
         rec["seconds_spent"] = round(time.time() - t0, 1)
@@ -448,8 +461,7 @@ def run_ours(args):
 
     # ---- the streaming kernels alone, on KERNEL_LAUNCHES further steps that carry events ------
     t_ctc, t_ver, ctc_bytes, ver_bytes = time_kernels(sets, 3 if args.ncu_small else KERNEL_LAUNCHES)
-    # ssd_verify picks its streaming kernel by size and type: direct loads or the ring
-    vkern = "verify_rows" if args.verify_mode == "full" else "verify_rows_ee"
+    vkern = verify_kernel(sets[0], w) if args.verify_mode == "full" else "verify_rows_ee"
 
     # ---- end to end: pinned host buffers in, decisions out, every step ---------------------
     e2e = None
@@ -505,8 +517,39 @@ def run_ours(args):
     if world == 1 and not args.ncu_small and not args.no_per_config:
         line["per_config"] = run_per_config(device, peak, peak_kind, args.config,
                                             cpu=not args.no_cpu_baseline)
-    print(json.dumps(line), flush=True)
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f, indent=1)
+    print(short_line(line), flush=True)
     D.finalize()
+
+
+LINE_LIMIT = 2900
+
+
+def short_line(line) -> str:
+    """The record as one line of at most LINE_LIMIT characters: what a reader of the last few thousand
+    characters of the output has to see, the parts that explain it as far as they fit."""
+    keep = ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_kind", "frac_best", "traffic",
+            "avg_launch_us")
+    out = dict(line)
+    out["roofline"] = {k: line["roofline"][k] for k in keep if k in line["roofline"]}
+    for k in ("roofline_ctc", "roofline_verify"):
+        out[k] = {q: line[k][q] for q in ("achieved", "frac", "avg_launch_us") if q in line[k]}
+    if "per_config" in out:
+        out["per_config"] = {name: [r["value"], r["step_frac_of_peak"], r["roofline_ctc"]["frac"],
+                                    r["roofline_verify"]["frac"]]
+                             for name, r in line["per_config"].items()}
+    out["config"] = dict(out["config"])
+    text = json.dumps(out)
+    # the longest explanations go first
+    for where, key in ((out, "next_rows"), (out, "decisions"), (out["config"], "calls_per_step"),
+                       (out, "cpu_baseline"), (out, "per_config")):
+        if len(text) <= LINE_LIMIT:
+            break
+        where.pop(key, None)
+        text = json.dumps(out)
+    return text
 
 
 def time_next_rows(sets, device, peak):
@@ -796,14 +839,14 @@ def run_reference(args):
         oracle_pass(h, w, starts[i], starts[i] + u)
     sec = time.perf_counter() - t0
     value = K * u / sec
-    sample = ("%d utterance(s) per step out of a %d-utterance batch of configs[%d] (window "
+    sample = ("%d utterance(s) per step out of a %d-utterance batch of configuration %d (window "
               "sliding over them), whole path in the fp64 C oracle, %d thread(s)" %
               (u, pool, args.config, threads))
     line = {"impl": "reference", "metric": METRIC, "value": round(value, 3), "unit": UNIT,
             "n_gpus": args.gpus, "steps": K, "warmup": W, "ms_per_step": round(sec / K * 1e3, 3),
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
             "data": "synthetic",
-            "config": {"workload": "configs[%d] %s (CPU oracle on a bounded sample per step)" %
+            "config": {"workload": "configuration %d, %s (CPU oracle on a bounded sample per step)" %
                                    (args.config, base.name), "sample": sample},
             "cpu_baseline": {"value": round(value, 3), "unit": UNIT, "cores": threads,
                              "kind": "oracle", "sample": sample},
