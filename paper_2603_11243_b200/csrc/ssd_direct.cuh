@@ -4,9 +4,10 @@
 //
 // A warp works on one span of columns of one row at a time and reads it with 32-byte loads
 // straight into registers: no shared memory, no barriers, no hand-over between warps.  What
-// bounds it on long batches is the 1 kW power cap (a kernel that only reads takes 611 us for 4.4
-// GB there, the ring 710, this one 665), so what counts is instructions per logit: 4.8 against
-// 6.0 of the ring.  148 x 32 warps keep two blocks of 1 KB each in flight (one where a span ends: the
+// bounds it on long batches is the 1 kW power cap (between events, a kernel that only reads takes 611
+// us for 4.4 GB there, the ring 710, this one 665), so what counts is instructions per logit: 4.3 of
+// 304 KB rows here, 6.0 of 98 KB rows in the ring (executed instructions as ncu counts them).
+// 148 x 32 warps keep two blocks of 1 KB each in flight (one where a span ends: the
 // next span's second block is asked for when its first has given the reference), the block loop
 // holds nothing but the loads, the sums and a counter, and everything that happens once per span
 // (reference, range check, merge of the lanes) is done once for the warp instead of once per
