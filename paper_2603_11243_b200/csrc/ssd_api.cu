@@ -217,7 +217,7 @@ int32_t ssd_verify_shard(const void *logits, ssd_dtype dtype, int32_t V_local, i
     const int es = dtype == SSD_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(logits) % es) return SSD_ERR_ALIGN;
     VerifyPlan plan;
-    int rc = plan_for_query(B, M, V_local, dtype, opts, &plan, RowsAt{logits, ld, false, skip != nullptr});
+    int rc = plan_for_query(B, M, V_local, dtype, opts, &plan, RowsAt{logits, ld, false, skip != nullptr, true});
     if (rc != SSD_OK) return rc;
     if (B > 0 && (!workspace || workspace_bytes < plan.workspace_bytes ||
                   reinterpret_cast<uintptr_t>(workspace) % 256))

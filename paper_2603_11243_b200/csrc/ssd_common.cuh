@@ -55,24 +55,46 @@ cudaError_t ensure_l1(const void *kernel, size_t smem);
 void count_launch();     // one more kernel launched by this host thread (ssd_launch_count)
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                       cudaStream_t stream, Args... args) {
+cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned cluster, unsigned grid, unsigned block, size_t smem,
+                            cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(block, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     count_launch();
     if (smem <= kSmallSmem) {
         const cudaError_t e = ensure_l1(reinterpret_cast<const void *>(kernel), smem);
         if (e != cudaSuccess) return e;
     }
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
+                       cudaStream_t stream, Args... args) {
+    return launch_clusters(kernel, 1u, grid, block, smem, stream, args...);
+}
+
+// ---- thread-block clusters ---------------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// where the shared-memory address `own` lies in the CTA of that rank
+__device__ __forceinline__ uint32_t cluster_address(uint32_t own, int rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(own), "r"(rank));
+    return a;
 }
 
 // ---- shared-memory addresses and mbarriers ---------------------------------------------------
@@ -475,6 +497,10 @@ struct VerifyPlan {
     direct::Cut cut[direct::kCuts];   // direct-load kernel: how rows are cut, for M, M/2, M/4 ... read
     int pairs;         // direct-load kernel: pairs per row, the most spans of any cut
     int direct_ctas;
+    int whole;         // rows are dealt to clusters and closed in the same launch
+    direct::Cut whole_cut;
+    int whole_cluster_log2, whole_clusters;
+    size_t whole_smem_bytes;
     size_t smem_bytes;
     size_t fin_smem_bytes;
     size_t workspace_bytes;
@@ -485,6 +511,7 @@ struct RowsAt {
     int64_t ld;
     bool greedy;
     bool skip;             // some utterances' rows may not be read
+    bool shard;
 };
 int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts *opts,
                 const RowsAt &at, VerifyPlan *plan);

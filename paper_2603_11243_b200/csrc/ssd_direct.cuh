@@ -131,7 +131,9 @@ struct SpanResult {
 // It takes what it needs by value: with the address of the kernel's parameters taken, every thread of
 // the kernel began by copying them to local memory (the call on 5,568 rows of 24 KB: 32.3 us, now
 // 29.6; the greedy step on 1,024 rows of 304 KB: 54.9, now 51.7).
-template <typename T, bool kArg>
+// (kCaller: a copy for each kernel.  ptxas 12.9 crashes on one called by a kernel with cluster barriers
+// and by another.)
+template <typename T, bool kArg, int kCaller>
 __device__ __noinline__ SpanResult span_running_max(const char *x, int row_bytes, Cut cut, int sp, int lane) {
     constexpr int ES = Elem<T>::kBytes;
     constexpr float kLowest = -3.402823466e38f;      // finite, so that x - m is -inf or 0 for a masked x
@@ -211,56 +213,27 @@ struct Cursor {
     bool valid;
 };
 
-template <typename T, int kF, bool kArg>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const DirectParams p) {
-    constexpr int ES = Elem<T>::kBytes;
-    extern __shared__ int32_t act[];
-    __shared__ int32_t warp_tot[kWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool table = p.table != 0;
-    pdl_wait();
-    pdl_launch_dependents();
-    int rows = (int)p.M;
-    Cut cut = p.cut[0];
-    if (table) {
-        const int per = (p.B + kThreads - 1) / kThreads, b0 = (int)threadIdx.x * per;
-        int32_t mine = 0;
-        for (int b = b0; b < min(p.B, b0 + per); ++b) {
-            const int64_t i0 = p.tok_off[b], i1 = p.tok_off[b + 1];
-            act[b] = mine;
-            if (!(i0 < 0 || i1 < i0 || i1 > p.M || p.skip[b])) mine += (int32_t)(i1 - i0);
-        }
-        int32_t incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) warp_tot[warp] = incl;
-        __syncthreads();
-        int32_t before = incl - mine, total = 0;
-        for (int w = 0; w < kWarps; ++w) {
-            const int32_t t = warp_tot[w];
-            if (w < warp) before += t;
-            total += t;
-        }
-        rows = total;
-#pragma unroll
-        for (int q = 1; q < kCuts; ++q)
-            if (rows <= (int)(p.M >> q)) cut = p.cut[q];
-        for (int b = b0; b < min(p.B, b0 + per); ++b) act[b] += before;
-        if (threadIdx.x == 0) act[p.B] = total;
-        __syncthreads();
-    }
+// Which spans a warp takes: number gw, gw + GW, ... of rows * spans.  Row index a stands for
+// row first + a * stride of those to read: of the table's, or of the matrix (then, unless `all`, rows
+// of skipped utterances are passed over).
+struct Deal {
+    unsigned gw, GW;
+    int rows, first, stride;
+    bool table, all;
+};
 
-    // item k of warp w is number w + k * (warps of the grid) of the rows * spans items, counted
-    // so that neighbours go to different CTAs
-    const unsigned gw = blockIdx.x + gridDim.x * warp, GW = gridDim.x * kWarps;
+// Streams the spans dealt to this warp and hands each one's result to emit(row, a, span, result),
+// called by all lanes.  opened() is called once, when the first block is on its way.
+template <typename T, int kF, bool kArg, int kCaller, typename Opened, typename Emit>
+__device__ __forceinline__ void stream_spans(const DirectParams &p, const Cut cut, const Deal deal,
+                                             const int32_t *act, Opened opened, Emit emit) {
+    constexpr int ES = Elem<T>::kBytes;
+    const int lane = threadIdx.x & 31;
     const unsigned ns = (unsigned)cut.spans;
-    const int da = (int)(GW / ns), ds = (int)(GW % ns);
+    const int da = (int)(deal.GW / ns), ds = (int)(deal.GW % ns);
     Cursor cur;
-    cur.a = (int)(gw / ns);
-    cur.sp = (int)(gw % ns);
+    cur.a = (int)(deal.gw / ns);
+    cur.sp = (int)(deal.gw % ns);
     cur.b = -1;
     cur.shift = 0;
     int b_end = 0;                       // rows to read up to and with utterance b
@@ -269,26 +242,27 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
         if (cur.sp >= cut.spans) { cur.sp -= cut.spans; ++cur.a; }
     };
     auto settle = [&]() {
-        if (table) {
-            cur.valid = cur.a < rows;
-            if (cur.valid && cur.a >= b_end) {
-                do b_end = act[++cur.b + 1]; while (b_end <= cur.a);
+        if (deal.table) {
+            cur.valid = cur.a < deal.rows;
+            const int at = deal.first + cur.a * deal.stride;
+            if (cur.valid && at >= b_end) {
+                do b_end = act[++cur.b + 1]; while (b_end <= at);
                 cur.shift = (int)p.tok_off[cur.b] - act[cur.b];
             }
-            cur.row = cur.a + cur.shift;
+            cur.row = at + cur.shift;
             return;
         }
         for (;;) {
-            cur.valid = cur.a < rows;
-            cur.row = cur.a;
-            if (!cur.valid || !p.skip) return;
+            cur.valid = cur.a < deal.rows;
+            cur.row = deal.first + cur.a * deal.stride;
+            if (!cur.valid || deal.all) return;
             const int b = utterance_of_row(p.tok_off, p.B, cur.row);
             if (b < 0 || !p.skip[b]) return;
             step();
         }
     };
     settle();
-    if (!cur.valid) return;
+    if (!cur.valid) { opened(); return; }
 
     // the span the cursor stands on: this lane's address in its first block, blocks, bytes of
     // the last block from this lane's unit on, the element this lane has of the row's two edges
@@ -326,9 +300,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
 
     Unit u, v;
     begin(u);
+    opened();
     for (;;) {
         Reference ref;
-        const int row = cur.row, sp = cur.sp;
+        const int row = cur.row, a = cur.a, sp = cur.sp;
         const float my_edge = edge;
         const int my_edge_idx = edge_idx, my_unit_elem = unit_elem;
         float vmax = -INFINITY, Sw = 0.f, total = 0.f;
@@ -382,8 +357,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
             out.m = ref.m;
             out.S = Sw;
             if (kArg) {
-                // a lane's maximum is known to a unit: its first element stands for it, and the
-                // closing kernel looks the position up
+                // a lane's maximum is known to a unit: its first element stands for it, and
+                // whoever closes the row looks the position up
                 out.vmax = warp_max(fmaxf(vmax, my_edge));
                 int idx = INT_MAX;
                 if (my_edge == out.vmax && my_edge > -INFINITY) idx = my_edge_idx;
@@ -392,8 +367,33 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
                 out.vidx = __reduce_min_sync(0xffffffffu, idx);
             }
         } else {
-            out = span_running_max<T, kArg>(p.logits + (int64_t)row * p.row_pitch, p.row_bytes, cut, sp, lane);
+            out = span_running_max<T, kArg, kCaller>(p.logits + (int64_t)row * p.row_pitch, p.row_bytes, cut, sp, lane);
         }
+        emit(row, a, sp, out);
+        if (!cur.valid) return;
+        u = v;
+    }
+}
+
+template <typename T, int kF, bool kArg>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const DirectParams p) {
+    extern __shared__ int32_t act[];
+    __shared__ int32_t warp_tot[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool table = p.table != 0;
+    pdl_wait();
+    pdl_launch_dependents();
+    int rows = (int)p.M;
+    Cut cut = p.cut[0];
+    if (table) {
+        rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, nullptr, warp_tot);
+#pragma unroll
+        for (int q = 1; q < kCuts; ++q)
+            if (rows <= (int)(p.M >> q)) cut = p.cut[q];
+    }
+    // counted so that neighbours go to different CTAs
+    const Deal deal{blockIdx.x + gridDim.x * warp, gridDim.x * kWarps, rows, 0, 1, table, p.skip == nullptr};
+    stream_spans<T, kF, kArg, 0>(p, cut, deal, act, [] {}, [&](int row, int, int sp, const SpanResult &out) {
         if (kArg) {
             if (lane == 0) reinterpret_cast<float4 *>(p.partials)[(int64_t)row * p.pairs + sp] =
                 make_float4(out.m, out.S, out.vmax, __int_as_float(out.vidx));
@@ -403,9 +403,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
             if (at < p.pairs) reinterpret_cast<float2 *>(p.partials)[(int64_t)row * p.pairs + at] =
                 lane == 0 ? make_float2(out.m, out.S) : make_float2(kNegInit, 0.f);
         }
-        if (!cur.valid) return;
-        u = v;
-    }
+    });
 }
 
 inline bool table_fits(int B, int64_t M) {

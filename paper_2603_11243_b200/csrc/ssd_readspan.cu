@@ -101,6 +101,34 @@ int32_t ssd_verify_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, int
     const int64_t row_pitch = ld * es, row_bytes = (int64_t)V * es;
     const uintptr_t base = (uintptr_t)base_addr;
     Span sp;
+    // the spans of every row, as the direct-load kernels cut it
+    auto walk_cut = [&](const direct::Cut &cut, int most) {
+        for (int64_t row = 0; row < M; ++row) {
+            const uintptr_t g0 = base + (uintptr_t)(row * row_pitch);
+            const ranges::RowUnits r = ranges::row_units(g0, (int)row_bytes);
+            bool ok = r.units == 0 || (g0 + (uintptr_t)r.head) % 32 == 0;
+            ok = ok && r.head >= 0 && r.head < 32 && r.units % 32 == 0;
+            ok = ok && r.row - r.head - r.units >= 0 && r.row - r.head - r.units < 32;
+            ok = ok && cut.spans <= most;
+            int at = 0;                // the spans must tile the row in order
+            for (int s = 0; s < cut.spans; ++s) {
+                const ranges::UnitSpan c = ranges::unit_span(r, cut.spans, s, cut.blocks);
+                ok = ok && c.lo == at && c.ulo >= c.lo && c.uhi >= c.ulo && c.hi >= c.uhi;
+                ok = ok && c.ulo - c.lo < 32 && c.hi - c.uhi < 32 && (c.uhi - c.ulo) % 32 == 0;
+                sp.add(g0 + (uintptr_t)c.lo, g0 + (uintptr_t)c.hi);
+                at = c.hi;
+            }
+            ok = ok && at == r.row;
+            if (!ok) ++sp.faults;
+        }
+    };
+    // a greedy step's and a shard's rows may be dealt to clusters instead
+    for (int greedy = 0; greedy < 2; ++greedy) {
+        VerifyPlan whole;
+        const RowsAt at{reinterpret_cast<const void *>((uintptr_t)base_addr), ld, greedy == 1, false, greedy == 0};
+        if (plan_verify(greedy ? 0 : B, M, V, dtype, opts, at, &whole) == SSD_OK && whole.whole)
+            walk_cut(whole.whole_cut, 128);
+    }
     if (plan.direct) {
         // with a skip flag per utterance the rows may be cut more finely (kCuts)
         VerifyPlan skipping = plan;
@@ -112,24 +140,7 @@ int32_t ssd_verify_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, int
             const direct::Cut cut = k < 0 ? plan.cut[0] : skipping.cut[k];
             const direct::Cut before = k < 1 ? plan.cut[0] : skipping.cut[k - 1];
             if (k >= 0 && cut.spans == before.spans && cut.blocks == before.blocks) continue;
-            for (int64_t row = 0; row < M; ++row) {
-                const uintptr_t g0 = base + (uintptr_t)(row * row_pitch);
-                const ranges::RowUnits r = ranges::row_units(g0, (int)row_bytes);
-                bool ok = r.units == 0 || (g0 + (uintptr_t)r.head) % 32 == 0;
-                ok = ok && r.head >= 0 && r.head < 32 && r.units % 32 == 0;
-                ok = ok && r.row - r.head - r.units >= 0 && r.row - r.head - r.units < 32;
-                ok = ok && cut.spans <= (k < 0 ? plan.pairs : skipping.pairs);
-                int at = 0;                // the spans must tile the row in order
-                for (int s = 0; s < cut.spans; ++s) {
-                    const ranges::UnitSpan c = ranges::unit_span(r, cut.spans, s, cut.blocks);
-                    ok = ok && c.lo == at && c.ulo >= c.lo && c.uhi >= c.ulo && c.hi >= c.uhi;
-                    ok = ok && c.ulo - c.lo < 32 && c.hi - c.uhi < 32 && (c.uhi - c.ulo) % 32 == 0;
-                    sp.add(g0 + (uintptr_t)c.lo, g0 + (uintptr_t)c.hi);
-                    at = c.hi;
-                }
-                ok = ok && at == r.row;
-                if (!ok) ++sp.faults;
-            }
+            walk_cut(cut, k < 0 ? plan.pairs : skipping.pairs);
         }
     } else if (plan.kernel == 2) {
         const int max_chunks = plan.stage_bytes >> 4;

@@ -27,6 +27,7 @@
 #include "ssd_direct.cuh"
 #include "ssd_ranges.cuh"
 #include "ssd_stream.cuh"
+#include "ssd_whole.cuh"
 
 namespace ssd {
 
@@ -801,11 +802,7 @@ __global__ void __launch_bounds__(kFinishThreads) combine_kernel(
     }
 }
 
-// Greedy step: merges the partials of a row, one warp per row.  A partial is (reference, sum,
-// largest logit, an index).  The ring's index is that of the logit's first occurrence; the direct-load
-// kernel's (kUnit) lies up to one 32-byte unit before it, and the unit is looked through here, once per
-// row instead of once per column span.  (The look-up is a dependent load: 400 fp32 rows of 128 KB,
-// which the ring reads, 15.3 us with it, 14.3 without; 1,024 of 192 KB 36.5, 35.4.)
+// Greedy step: closes the rows whose partials the streaming kernel left, one warp per row.
 constexpr int kGreedyWarps = 8;
 template <typename T, bool kUnit>
 __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
@@ -817,39 +814,14 @@ __global__ void __launch_bounds__(kGreedyWarps * 32) greedy_finish_kernel(
     const int64_t r = (int64_t)blockIdx.x * kGreedyWarps + (threadIdx.x >> 5);
     if (r >= R) return;
     const float4 *pp = partials + r * P;
-    float Mx = kNegInit, vm = -INFINITY;
-    for (int q = lane; q < P; q += 32) {
-        const float4 v = pp[q];
-        Mx = fmaxf(Mx, v.x);
-        vm = fmaxf(vm, v.z);
-    }
-    Mx = warp_max(Mx);
-    vm = warp_max(vm);
-    float S = 0.f;
-    int vi = INT_MAX;
-    for (int q = lane; q < P; q += 32) {
-        const float4 v = pp[q];
-        S += v.y * ex2((v.x - Mx) * kLog2e);
-        if (v.z == vm) vi = min(vi, __float_as_int(v.w));
-    }
-    S = warp_sum(S);
-    vi = __reduce_min_sync(0xffffffffu, vi);
-    if (kUnit && vi >= 0 && vi < V) {
-        const int64_t e = (int64_t)vi + lane;
-        const bool hit = lane < 32 / Elem<T>::kBytes && e < V &&
-                         Elem<T>::load(logits + (r * ld + e) * Elem<T>::kBytes) == vm;
-        const unsigned hits = __ballot_sync(0xffffffffu, hit);
-        if (hits) vi += __ffs(hits) - 1;
-    }
+    const GreedyRow g = greedy_row<T, kUnit>([&](int q) { return pp[q]; }, P,
+                                             logits + r * ld * Elem<T>::kBytes, V, lane);
     if (lane == 0) {
-        const float lnS = logf(S);
-        const float lse = Mx + lnS;
-        uint32_t st = (*err_word == epoch) ? (uint32_t)SSD_UTT_INTERNAL : 0u;
-        if (!(fabsf(lse) < INFINITY)) st |= SSD_UTT_NONFINITE;
-        next_token[r] = (vi < 0 || vi >= V) ? 0 : vi;
-        if (next_logp) next_logp[r] = (vm - Mx) - lnS;
-        if (row_lse) row_lse[r] = lse;
-        if (row_status) row_status[r] = st;
+        const uint32_t internal = (*err_word == epoch) ? (uint32_t)SSD_UTT_INTERNAL : 0u;
+        next_token[r] = g.token;
+        if (next_logp) next_logp[r] = g.logp;
+        if (row_lse) row_lse[r] = g.lse;
+        if (row_status) row_status[r] = g.status | internal;
     }
 }
 
@@ -882,6 +854,75 @@ static int use_direct(int64_t M, int64_t row_bytes, ssd_dtype dtype, int kernel,
     if (dtype == SSD_F32) return at.greedy && M <= 2ll * sms;
     if (at.greedy || few || row_bytes < 96 * 1024 || M * row_bytes >= (at.skip ? 2400ll : 1200ll) << 20) return 1;
     return (reinterpret_cast<uintptr_t>(at.base) | (uintptr_t)(at.ld * 2)) % 16 != 0;
+}
+
+// How rows are dealt to clusters that close them (rows_whole): column spans, cluster size and number
+// of clusters with the fewest block steps of a warp, counted as plan_spans counts them; that number,
+// or 0 where a CTA's pairs do not fit.
+static int64_t plan_whole(int64_t M, int64_t row_bytes, int sms, const RowsAt &at, int B, VerifyPlan *pl) {
+    constexpr size_t kMostSmem = 12 * 1024;      // little enough for the L1-heavy split
+    const int64_t nb = direct::row_blocks(row_bytes);
+    const size_t pair = at.greedy ? sizeof(float4) : sizeof(float2), draft = at.greedy ? 0 : sizeof(float2);
+    int64_t best = 0;
+    for (int clog = 0; clog <= 3; ++clog) {
+        const int C = 1 << clog, W = C * direct::kWarps;
+        // clusters of four and eight CTAs do not fill the GPU's clusters of SMs: 71 of 74 and 33 of 37
+        // run at a time, and one more waits for the longest of those (300 rows of 98 KB on 35 clusters
+        // of eight: 13.9 us; on 32, 10.0)
+        const int64_t most = (int64_t)direct::kCtasPerSm * sms / C * (clog == 3 ? 22 : clog == 2 ? 24 : 25) / 25;
+        const int64_t nc = M < most ? M : most > 0 ? most : 1;
+        const int64_t q = (M + nc - 1) / nc;
+        for (int rounds = 1; rounds <= 16; ++rounds) {
+            int64_t ns = (int64_t)rounds * W / q;
+            ns = ns < 1 ? 1 : ns > 128 ? 128 : ns;
+            const int64_t bps = (nb + ns - 1) / ns;
+            ns = (nb + bps - 1) / bps;
+            const size_t smem = (size_t)((q + C - 1) / C) * (ns * pair + draft) + (at.skip ? (size_t)(B + 1) * 4 : 0);
+            const int64_t cost = (q * ns + W - 1) / W * (bps + 3);
+            if (smem > kMostSmem || (best != 0 && cost >= best)) continue;
+            best = cost;
+            pl->whole_cut = direct::Cut{(int)ns, (int)bps};
+            pl->whole_cluster_log2 = clog;
+            pl->whole_clusters = (int)nc;
+            pl->whole_smem_bytes = smem;
+        }
+    }
+    return best;
+}
+
+// Whether the rows of a greedy step or a shard are closed by the clusters that read them.  Measured,
+// us a call, passes back to back on one B200, before (pair kernel or, on fp32, ring, and a closing
+// kernel) and after:
+//   greedy step, bf16: 1 row of 98 KB 5.3 / 4.0, 24 rows 5.3 / 4.3, 148 7.6 / 6.4, 1,024 21.5 / 19.4;
+//     of 304 KB: 24 rows 7.4 / 5.7, 200 14.5 / 14.0, 700 38.2 / 36.8, 1,024 51.3 / 49.6
+//   greedy step, fp32, rows of 196 KB: 24 rows 5.9 / 5.4, 300 15.9 / 14.4, 600 25.3 / 21.9, 1,024
+//     35.1 / 33.7, 2,000 62.1 / 61.1; 2,000 of 128 KB 43.7 / 45.2: eight rows an SM and more stay
+//     with the ring
+//   shard, bf16, rows of 24 KB: 250 rows 5.8 / 5.4, 1,500 10.5 / 9.6, 5,352 26.4 / 25.1
+//   shard, fp32: 600 rows of 16 KB 9.1 / 5.1, 12,000 75 / 34; 5,352 of 32 KB 37.0 / 30.3, 1,500 of 76
+//     KB 23.5 / 20.5; 12,000 of 152 KB 260 / 268: long rows of long batches stay with the ring, as
+//     in use_direct, where rows start on 16-byte boundaries (12,000 of 64,004 bytes 138 / 113)
+// Whole rows do not always come out even over the clusters.  Where that takes clusters of four and
+// more in more than a few rows each, or a third more steps, the pair kernel's finer deal is better
+// (600 rows of 32 KB 7.7 / 8.7; the greedy step on 74 of 304 KB 9.3 / 9.9).  With skip flags on a
+// row per warp and more only the kernel knows how many are read, and plan_cuts has cuts for that.
+static int use_whole(int B, int64_t M, int64_t row_bytes, ssd_dtype dtype, int sms, const ssd_launch_opts *o,
+                     const RowsAt &at, VerifyPlan *pl) {
+    if (!(at.greedy || at.shard) || M == 0 || pl->kernel != 2 || row_bytes >= (1ll << 30) || M >= (1ll << 30)) return 0;
+    if (o && (o->kernel || o->ctas || o->split || o->warps || o->stages || o->stage_bytes || o->fma_exp || o->finish))
+        return 0;
+    const int warps = direct::kCtasPerSm * sms * direct::kWarps;
+    if (at.skip && (M >= warps || !direct::table_fits(B, M))) return 0;
+    if (dtype == SSD_F32 && at.greedy && M >= 8ll * sms) return 0;
+    if (dtype == SSD_F32 && at.shard && row_bytes >= 72 * 1024 && M * row_bytes >= 300ll << 20 &&
+        (reinterpret_cast<uintptr_t>(at.base) | (uintptr_t)(at.ld * 4)) % 16 == 0)
+        return 0;
+    const int64_t cost = plan_whole(M, row_bytes, sms, at, B, pl);
+    if (cost == 0) return 0;
+    if (dtype == SSD_F32) return 1;
+    const direct::Cut c = direct::plan_spans(M, row_bytes, warps, 64);
+    const int64_t pairs = (M * c.spans + warps - 1) / warps * (c.blocks + 3);
+    return pl->whole_cluster_log2 >= 2 ? cost <= pairs + 1 && M <= 8ll * pl->whole_clusters : 3 * cost <= 4 * pairs + 3;
 }
 
 // Workspace: [0,256) header (error word, finished-CTA counter), two words per utterance, then
@@ -962,6 +1003,7 @@ int plan_verify(int B, int64_t M, int V, ssd_dtype dtype, const ssd_launch_opts 
                               pl.cut, &pl.pairs);
         }
     }
+    pl.whole = use_whole(B, M, row_bytes, dtype, sms, o, at, &pl);
     // header | two words per utterance | partials
     pl.workspace_bytes = 256 + (((size_t)(B > 0 ? B : 0) * 16 + 255) & ~(size_t)255) +
                          (size_t)M * pl.partials * sizeof(float2);
@@ -1014,6 +1056,36 @@ static cudaError_t launch_direct(const void *logits, ssd_dtype dtype, int V, int
     auto kern = direct::verify_rows_direct<bf16_t, kArg ? 0 : 1, kArg>;
     if (kArg && dtype == SSD_F32) kern = direct::verify_rows_direct<float, 0, true>;
     return launch_pdl(kern, (unsigned)ctas, (unsigned)direct::kThreads, smem, stream, p);
+}
+
+// The one launch of a call whose rows are closed where they are read.
+template <int kEnd>
+static int launch_whole(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_t M, const int64_t *tok_off,
+                        int B, const uint8_t *skip, const whole::EndParams &end, const VerifyPlan &plan,
+                        const Launch &L) {
+    const ssd_launch_opts *o = L.opts;
+    const int es = dtype == SSD_F32 ? 4 : 2;
+    direct::DirectParams p{};
+    p.logits = static_cast<const char *>(logits);
+    p.row_pitch = ld * es; p.row_bytes = V * es; p.M = M;
+    p.cut[0] = plan.whole_cut;
+    p.tok_off = tok_off; p.B = B; p.skip = skip; p.table = skip != nullptr;
+    whole::EndParams e = end;
+    e.cluster_log2 = plan.whole_cluster_log2;
+    e.V = V;
+    constexpr int kF = kEnd == whole::kGreedy ? 0 : 1;       // as in launch_direct
+    void (*kern)(const direct::DirectParams, const whole::EndParams) = whole::rows_whole<bf16_t, kF, kEnd>;
+    if (dtype == SSD_F32) kern = whole::rows_whole<float, 0, kEnd>;
+    const unsigned cluster = 1u << plan.whole_cluster_log2;
+    cudaError_t err = cudaSuccess;
+    if (o && o->ev_begin) err = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_begin), L.stream);
+    if (err == cudaSuccess)
+        err = launch_clusters(kern, cluster, (unsigned)plan.whole_clusters * cluster, (unsigned)direct::kThreads,
+                              plan.whole_smem_bytes, L.stream, p, e);
+    if (err == cudaSuccess) err = cudaGetLastError();
+    if (err == cudaSuccess && o && o->ev_end) err = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_end), L.stream);
+    if (err != cudaSuccess) { record_cuda_error(err); return SSD_ERR_CUDA; }
+    return SSD_OK;
 }
 
 // The closing kernel for P pairs per row and drafts of K tokens on average: four pairs a lane in
@@ -1185,6 +1257,11 @@ int launch_verify_shard(const void *logits, ssd_dtype dtype, int V_local, int64_
     if (B == 0) return SSD_OK;
     unsigned long long *err_word = static_cast<unsigned long long *>(workspace);
     float2 *partials = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + partials_offset(B));
+    if (plan.whole) {
+        whole::EndParams end{};
+        end.col0 = col0; end.draft_ids = draft_ids; end.stats = shard_stats;
+        return launch_whole<whole::kShard>(logits, dtype, V_local, ld, M, tok_off, B, skip, end, plan, L);
+    }
     const unsigned long long epoch = next_epoch();
     const int rc = launch_verify_rows(logits, dtype, V_local, ld, M, tok_off, B, skip, workspace,
                                       epoch, plan, L);
@@ -1232,6 +1309,11 @@ int launch_greedy(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_
     const ssd_launch_opts *o = L.opts;
     unsigned long long *err_word = static_cast<unsigned long long *>(workspace);
     float4 *partials = reinterpret_cast<float4 *>(static_cast<char *>(workspace) + 256);
+    if (plan.whole) {
+        whole::EndParams end{};
+        end.token = next_token; end.logp = next_logp; end.lse = row_lse; end.status = row_status;
+        return launch_whole<whole::kGreedy>(logits, dtype, V, ld, R, nullptr, 0, nullptr, end, plan, L);
+    }
     const unsigned long long epoch = next_epoch();
     VerifyParams p{};
     p.logits = static_cast<const char *>(logits);

@@ -1,0 +1,70 @@
+"""Rows closed by the clusters that read them (the greedy step and a rank's statistics on most sizes)
+against the oracle and the plain-load kernel: one to eight CTAs a cluster, rows that do not come out
+even over the clusters, rows of less than a unit and of several spans, offsets that name no row, some
+twice or leave some out."""
+import numpy as np
+import pytest
+import torch
+
+import helpers as H
+from oracle import ref
+from paper_2603_11243_b200 import binding as ssd
+
+pytestmark = pytest.mark.gpu
+
+
+def _matrix(R, V, dtype, seed, pad=7):
+    g = torch.Generator()
+    g.manual_seed(seed)
+    return (torch.randn((R, V + pad), generator=g) * 3.0).to(dtype)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("R,V", [(1, 1), (1, 70001), (2, 33), (31, 9000), (33, 513), (73, 4097), (147, 1039),
+                                 (149, 15), (285, 2048), (297, 3001), (593, 600), (1025, 514)])
+def test_greedy_step(cuda_device, R, V, dtype):
+    wide = _matrix(R, V, dtype, 3 * R + V)
+    for r in range(0, R, 5):                       # the largest value twice: the first counts
+        wide[r, 2 + V // 3] = wide[r, 1 + V] = 40.0
+    want = ref.greedy_step(H.storage_numpy(wide[:, 2:2 + V].contiguous()), V)
+    before = ssd.lib().ssd_launch_count()
+    got = ssd.ssd_greedy_step(wide.to(cuda_device)[:, 2:2 + V])
+    torch.cuda.synchronize()
+    assert ssd.lib().ssd_launch_count() - before == 1
+    np.testing.assert_array_equal(got["next_token"].cpu().numpy(), want["next_token"])
+    assert np.abs(got["row_lse"].cpu().numpy() - want["row_lse"]).max() <= H.FLOAT_TOL
+    assert np.abs(got["next_logp"].cpu().numpy() - want["next_logp"]).max() <= H.FLOAT_TOL
+
+
+# [0, M] as it should be; a gap before, between and after; one utterance's end before its start; one
+# past the matrix; two that overlap
+OFFSETS = {"sound": lambda M: [0, M // 3, M // 3, M], "gaps": lambda M: [M // 5, M // 2, M - 1],
+           "reversed": lambda M: [0, M // 2, M // 4, M], "past": lambda M: [0, M // 2, M + 3],
+           "twice": lambda M: [0, M // 2, M // 4, M // 2, M // 3, M]}
+
+
+@pytest.mark.parametrize("offsets", sorted(OFFSETS))
+@pytest.mark.parametrize("skipping", [False, True])
+@pytest.mark.parametrize("M,V,dtype", [(8, 513, torch.bfloat16), (61, 5001, torch.float32), (299, 1100, torch.bfloat16),
+                                       (640, 257, torch.float32), (1500, 1024, torch.bfloat16)])
+def test_shard_statistics(cuda_device, M, V, dtype, skipping, offsets):
+    x = _matrix(M, V, dtype, M)[:, 3:3 + V].to(cuda_device)
+    off = torch.tensor(OFFSETS[offsets](M), dtype=torch.int64, device=cuda_device)
+    B, col0 = off.numel() - 1, 1000
+    g = torch.Generator()
+    g.manual_seed(M + 1)
+    ids = torch.randint(0, col0 + 2 * V, (M,), generator=g, dtype=torch.int32).to(cuda_device)
+    skip = torch.tensor([b % 2 for b in range(B)], dtype=torch.uint8, device=cuda_device) if skipping else None
+    size = max(256, ssd.ssd_verify_workspace_bytes(B, M, V, ssd.F32 if dtype == torch.float32 else ssd.BF16))
+    got, want = (torch.full((M, 3), 7.5, device=cuda_device) for _ in range(2))
+    before = ssd.lib().ssd_launch_count()
+    ssd.ssd_verify_shard(x, col0, off, ids, skip=skip, stats=got,
+                         workspace=torch.zeros((size,), dtype=torch.uint8, device=cuda_device))
+    assert ssd.lib().ssd_launch_count() - before == 1
+    ssd.ssd_verify_shard(x, col0, off, ids, skip=skip, stats=want, opts=H.opts(kernel=1))
+    torch.cuda.synchronize()
+    # the same rows written, the draft logits as they are, the pairs for one log-sum-exp
+    assert torch.equal(got == 7.5, want == 7.5)
+    assert torch.equal(got[:, 2], want[:, 2])
+    lse = [s[:, 0].double() + s[:, 1].double().log() for s in (got, want)]
+    assert float((lse[0] - lse[1]).abs().max()) <= H.FLOAT_TOL
