@@ -195,18 +195,16 @@ __device__ __forceinline__ float row_logp(float x, float Mx, float lnS) {
     return fabsf(Mx + lnS) < INFINITY ? (x - Mx) - lnS : __int_as_float(0x7fc00000);
 }
 
-// Rows to read before each utterance (act[B]: their total, which is returned) and, if `shift` is
-// given, what to add to such a count to have the row, both in shared memory.  Called by all threads
-// of the block; warp_tot has a word per warp.
+// Rows to read before each utterance (act[B]: their total, which is returned), in shared memory.
+// Called by all threads of the block; warp_tot has a word per warp.
 __device__ __forceinline__ int count_rows(const int64_t *tok_off, const uint8_t *skip, int B, int64_t M,
-                                          int32_t *act, int32_t *shift, int32_t *warp_tot) {
+                                          int32_t *act, int32_t *warp_tot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, threads = blockDim.x;
     const int per = (B + threads - 1) / threads, b0 = (int)threadIdx.x * per;
     int32_t mine = 0;
     for (int b = b0; b < min(B, b0 + per); ++b) {
         const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
         act[b] = mine;
-        if (shift) shift[b] = (int32_t)i0 - mine;
         if (!(i0 < 0 || i1 < i0 || i1 > M || skip[b])) mine += (int32_t)(i1 - i0);
     }
     int32_t incl = mine;
@@ -223,12 +221,47 @@ __device__ __forceinline__ int count_rows(const int64_t *tok_off, const uint8_t 
         if (w < warp) before += t;
         total += t;
     }
-    for (int b = b0; b < min(B, b0 + per); ++b) {
-        act[b] += before;
-        if (shift) shift[b] -= before;
-    }
+    for (int b = b0; b < min(B, b0 + per); ++b) act[b] += before;
     if (threadIdx.x == 0) act[B] = total;
     __syncthreads();
+    return total;
+}
+// The same by one warp, for itself, and what to add to such a count to have the row.
+__device__ __forceinline__ int count_rows_by_warp(const int64_t *tok_off, const uint8_t *skip, int B, int64_t M,
+                                                  int32_t *act, int32_t *shift) {
+    constexpr int L = 4;                 // utterances a lane has in flight
+    const int lane = threadIdx.x & 31;
+    int total = 0;
+    for (int b0 = 0; b0 < B; b0 += 32 * L) {
+        int64_t i0[L], i1[L];
+        int skipped[L];
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int b = min(b0 + 32 * j + lane, B - 1);
+            i0[j] = tok_off[b];
+            i1[j] = tok_off[b + 1];
+            skipped[j] = skip[b];
+        }
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int b = b0 + 32 * j + lane;
+            const bool read = b < B && !skipped[j] && i0[j] >= 0 && i1[j] >= i0[j] && i1[j] <= M;
+            const int mine = read ? (int)(i1[j] - i0[j]) : 0;
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (b < B) {
+                act[b] = total + incl - mine;
+                shift[b] = (int)i0[j] - (total + incl - mine);
+            }
+            total += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+    if (lane == 0) act[B] = total;
+    __syncwarp();
     return total;
 }
 // The utterance that has row number `at`, below the total: the last one with no more than that many

@@ -46,6 +46,7 @@ struct VerifyParams {
     const int64_t *tok_off;
     int B;
     const uint8_t *skip;
+    int table;            // count the rows to read per utterance in shared memory first
     float2 *partials;
     int partials_per_row;
     int warps;            // consumer warps
@@ -63,16 +64,18 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
     if (kArg) pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = p.stages, CW = p.warps;
-    // layout: full[S] | empty[S] | desc[S] | offsets cache | stages
+    // layout: full[S] | empty[S] | desc[S] | rows to read before each utterance and what takes the
+    // count of such rows to a row of the matrix | stages
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t full0 = sbase, empty0 = sbase + S * 8;
     StageDesc *desc = reinterpret_cast<StageDesc *>(smem + 2 * S * 8);
-    const bool cache_off = p.skip != nullptr && p.B + 1 <= kOffCacheMax;
-    int64_t *off_cache = reinterpret_cast<int64_t *>(smem + 2 * S * 8 + S * sizeof(StageDesc));
+    const bool table = p.table != 0;
+    int32_t *act = reinterpret_cast<int32_t *>(smem + 2 * S * 8 + S * sizeof(StageDesc));
+    int32_t *shift = act + (table ? p.B + 1 : 0);
     const uint32_t hdr = (uint32_t)((2 * S * 8 + S * sizeof(StageDesc) +
-                                     (cache_off ? (size_t)(p.B + 1) * 8 : 0) + 127) & ~(size_t)127);
+                                     (table ? (size_t)(p.B + 1) * 8 : 0) + 127) & ~(size_t)127);
     const uint32_t stage0 = sbase + hdr;
     unsigned char *stage0_ptr = smem + hdr;
 
@@ -80,29 +83,36 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
         for (int s = 0; s < S; ++s) { mbar_init(full0 + s * 8, 1); mbar_init(empty0 + s * 8, CW); }
         mbar_init_fence();
     }
+    __syncthreads();             // the barriers are there
     pdl_wait();
     if (!kArg) pdl_launch_dependents();
-    if (cache_off)
-        for (int i = threadIdx.x; i <= p.B; i += blockDim.x) off_cache[i] = p.tok_off[i];
-    __syncthreads();
 
     const int64_t row_bytes = (int64_t)p.V * ES;
 
     if (warp == 0) {
         // =============================== producer ===============================
-        const int64_t *offs = cache_off ? off_cache : p.tok_off;
+        // With skip flags only rows that are read are dealt out (with more utterances or rows than
+        // the table takes, skipped ones are passed over instead): a batch of which nothing is read
+        // costs a CTA its look at the flags, by this warp alone.  (56 utterances, 20,000 rows of 98
+        // KB, none read: the call 5.8 us with every row looked up, 3.5 with a count by the whole
+        // block; but 50 rows of 128 KB 6.4 and 7.2.)
+        int64_t num_items = p.num_items;
+        if (table) num_items = (int64_t)count_rows_by_warp(p.tok_off, p.skip, p.B, p.M, act, shift) * p.split;
         int s = 0;                  // stage to fill next, and the phase of its barriers
         uint32_t ph = 0;
         bool failed = false;
         const int max_chunks = p.stage_bytes >> 4;
         for (int64_t k0 = 0; !failed; k0 += 32) {
             const int64_t first = (int64_t)blockIdx.x + k0 * gridDim.x;
-            if (first >= p.num_items) break;
+            if (first >= num_items) break;
             const int64_t mine = first + (int64_t)lane * gridDim.x;
-            const int64_t my_row = mine / p.split;
-            bool active = mine < p.num_items;
-            if (active && p.skip) {
-                const int b = utterance_of_row(offs, p.B, my_row);
+            int64_t my_row = mine / p.split;
+            const int my_span = (int)(mine - my_row * p.split);
+            bool active = mine < num_items;
+            if (active && table) {
+                my_row += shift[utterance_of_count(act, p.B, (int)my_row)];
+            } else if (active && p.skip) {
+                const int b = utterance_of_row(p.tok_off, p.B, my_row);
                 active = !(b >= 0 && p.skip[b]);
             }
             unsigned todo = __ballot_sync(0xffffffffu, active);
@@ -110,7 +120,7 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
                 const int src = __ffs(todo) - 1;
                 todo &= todo - 1;
                 const int64_t row = __shfl_sync(0xffffffffu, my_row, src);
-                const int sp = (int)(__shfl_sync(0xffffffffu, mine, src) - row * p.split);
+                const int sp = __shfl_sync(0xffffffffu, my_span, src);
                 const ranges::RowGeom geom = ranges::row_geom(
                     reinterpret_cast<uintptr_t>(p.logits), row, p.ld * ES, row_bytes);
                 const uintptr_t g0 = geom.g0, g1 = geom.g1, f0 = geom.f0;
@@ -1120,6 +1130,7 @@ static int launch_verify_rows(const void *logits, ssd_dtype dtype, int V, int64_
     p.logits = static_cast<const char *>(logits);
     p.V = V; p.ld = ld; p.M = M; p.split = plan.split; p.num_items = M * plan.split;
     p.tok_off = tok_off; p.B = B; p.skip = skip;
+    p.table = skip && direct::table_fits(B, M);
     p.partials = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + partials_offset(B));
     p.partials_per_row = plan.partials;
     p.warps = plan.warps; p.stages = plan.stages; p.stage_bytes = plan.stage_bytes;
