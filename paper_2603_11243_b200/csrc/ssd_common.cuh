@@ -387,6 +387,18 @@ template <> struct Elem<float> {
 // An input of the call, read before the streaming kernel of the same call is through.
 template <typename V> __device__ __forceinline__ V load_input(const V *p) { return __ldcg(p); }
 
+// Loads that are issued where they are written, whatever condition their values are used under later.
+__device__ __forceinline__ int load_now(const uint8_t *p) {
+    int v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int load_now(const int32_t *p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 struct bf16_t { uint16_t bits; };
 template <> struct Elem<bf16_t> {
     static constexpr int kBytes = 2;

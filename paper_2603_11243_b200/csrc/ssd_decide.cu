@@ -73,11 +73,15 @@ __global__ void __launch_bounds__(kAssembleThreads) assemble_kernel(
     __shared__ int warp_tot[2][kAssembleThreads / 32];
     pdl_enter();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // all five words in one round trip: with `gate || all ? K : accepted` each was asked for when the
+    // one before it had come back
     auto prefix_len = [&](int b, bool &fin) {
         const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
+        const int gate = load_now(gate_accept + b), all = load_now(all_accepted + b);
+        const int accepted = load_now(accepted_len + b);
         const int K = (i0 < 0 || i1 < i0 || i1 > M) ? 0 : (int)min(i1 - i0, (int64_t)INT_MAX);
-        fin = gate_accept[b] != 0 || all_accepted[b] != 0;
-        return fin ? K : max(0, min(accepted_len[b], K));
+        fin = (gate | all) != 0;
+        return fin ? K : max(0, min(accepted, K));
     };
     if ((int)blockIdx.x < B) {
         const int b = blockIdx.x;

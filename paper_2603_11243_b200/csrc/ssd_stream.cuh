@@ -204,8 +204,9 @@ __device__ __forceinline__ int count_rows(const int64_t *tok_off, const uint8_t 
     int32_t mine = 0;
     for (int b = b0; b < min(B, b0 + per); ++b) {
         const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
+        const int skipped = load_now(skip + b);
         act[b] = mine;
-        if (!(i0 < 0 || i1 < i0 || i1 > M || skip[b])) mine += (int32_t)(i1 - i0);
+        if (!(i0 < 0 || i1 < i0 || i1 > M || skipped)) mine += (int32_t)(i1 - i0);
     }
     int32_t incl = mine;
 #pragma unroll

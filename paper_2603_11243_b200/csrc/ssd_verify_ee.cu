@@ -112,12 +112,13 @@ __global__ void __launch_bounds__(1024) ee_init_kernel(
     int mx = 0;
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
         const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
+        const int skipped = skip ? load_now(skip + b) : 0;
         const bool ok = !(i0 < 0 || i1 < i0 || i1 > M);
         const int K = ok ? (int)min(i1 - i0, (int64_t)INT_MAX) : 0;
         first_reject[b] = K;
         flags[b] = ok ? 0u : (uint32_t)SSD_UTT_BAD_OFFSETS;
         rows_read[b] = 0;
-        if (ok && !(skip && skip[b])) mx = max(mx, K);
+        if (ok && !skipped) mx = max(mx, K);
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) warp_max_sh[threadIdx.x >> 5] = mx;
