@@ -469,6 +469,7 @@ struct CtcPlan {
     int fma_exp;            // pairs per bf16 chunk whose exponential runs on the FMA pipe
     int64_t num_tiles;
     size_t smem_bytes, workspace_bytes;
+    int direct, d_lanes, d_units;      // rows are read into registers: lanes a row, units a lane
 };
 int plan_ctc(ssd_dtype dtype, int V, int64_t ld, int64_t N, int B, const ssd_launch_opts *opts,
              CtcPlan *plan);

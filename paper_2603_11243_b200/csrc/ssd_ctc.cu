@@ -14,11 +14,17 @@
 #include <math.h>
 
 #include "ssd_common.cuh"
+#include "ssd_ctc_direct.cuh"
 #include "ssd_ranges.cuh"
 
 namespace ssd {
 
 namespace {
+
+using ctc::group_max;
+using ctc::group_min;
+using ctc::group_sum;
+using ctc::RowOut;
 
 constexpr uint32_t kNanInternal = 0x7fc0dead;  // entropy payload written when a wait ran out
 
@@ -103,27 +109,6 @@ __device__ __forceinline__ void entropy_chunk<bf16_t>(const uint4 &w, float nmh,
     entropy_pair(make_float2(bf16_lo(z), bf16_hi(z)), nmh, Sa, Aa);
     entropy_pair(make_float2(bf16_lo(u), bf16_hi(u)), nmh, Sb, Ab);
 }
-
-template <int G> __device__ __forceinline__ float group_max(float v) {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-template <int G> __device__ __forceinline__ int group_min(int v) {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-template <int G> __device__ __forceinline__ float group_sum(float v) {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-struct RowOut {
-    float lse, H;
-    int arg;
-};
 
 // Geometry of one row inside a stage: the 16-byte chunks [cf, cl] it touches and which
 // elements of the first and last chunk are its own.
@@ -618,6 +603,52 @@ __global__ void __launch_bounds__(512, 1) ctc_rows_tma(const CtcParams p) {
     }
 }
 
+// ---- rows straight into registers ----------------------------------------------------------------
+// Writes a row's results (lane `sub` of the G lanes that share it).
+template <typename T, int G>
+__device__ __forceinline__ void write_row(const CtcParams &p, int64_t row, const char *x, const RowOut &out, int sub) {
+    if (sub == 0) {
+        p.frame_entropy[row] = out.H;
+        p.frame_argmax[row] = out.arg;
+        if (p.frame_lse) p.frame_lse[row] = out.lse;
+    }
+    if (p.frame_logprob)
+        for (int e = sub; e < p.V; e += G)
+            p.frame_logprob[row * p.ld + e] = Elem<T>::load(x + (int64_t)e * Elem<T>::kBytes) - out.lse;
+}
+
+// fp32 rows are asked for while the one before is closed (130,000 rows of 516 bytes 20.1 -> 19.0 us, 50,000
+// 11.9 -> 11.2); with bf16, which needs the registers for its unpacked pairs, that was slower (50,000
+// rows of 2 KB 29.6 -> 31.0).
+template <typename T, int G, int U>
+__global__ void __launch_bounds__(direct::kThreads, direct::kCtasPerSm) ctc_rows_direct(const CtcParams p) {
+    constexpr int ES = Elem<T>::kBytes, RPW = 32 / G;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % G;
+    const int64_t passes = (p.N + RPW - 1) / RPW, step = (int64_t)gridDim.x * (blockDim.x >> 5);
+    int64_t pass = blockIdx.x + (int64_t)gridDim.x * warp;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (pass >= passes) return;
+    auto row_at = [&](int64_t r) { return p.logits + min(r, p.N - 1) * p.ld * ES; };
+    int64_t row = pass * RPW + lane / G;
+    const char *x = row_at(row);
+    ctc::Row<T, G, U> v;
+    v.load(x, p.V * ES, sub);
+    for (;;) {
+        const int64_t next = row + step * RPW;
+        pass += step;
+        constexpr bool kAhead = ES == 4;
+        const RowOut out = ctc::reduce_row<T, G, U>(v, x, p.V * ES, sub, [&] {
+            if (kAhead && pass < passes) v.load(row_at(next), p.V * ES, sub);
+        });
+        if (row < p.N) write_row<T, G>(p, row, x, out, sub);
+        if (pass >= passes) return;
+        if (!kAhead) v.load(row_at(next), p.V * ES, sub);
+        row = next;
+        x = row_at(row);
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) ctc_rows_plain(const CtcParams p) {
     constexpr int ES = Elem<T>::kBytes;
@@ -830,6 +861,41 @@ unsigned long long next_epoch() {
     return 0x55D0000000000000ull | (c & 0x0000ffffffffffffull);
 }
 
+// How the lanes of a warp share rows that are read into registers, for `warps` warps: the fewest
+// instructions of a warp, counted as so many a unit, an element of the ragged ends and a row.
+static int64_t lanes_for(ssd_dtype dtype, int V, int64_t rows, int64_t warps, int *G, int *U) {
+    const int es = dtype == SSD_F32 ? 4 : 2;
+    const int units = (int)((int64_t)V * es / 32);
+    int64_t best = 0;
+    for (int g = 8; g <= 32; g *= 2) {
+        const int u = units > g ? (units + g - 1) / g : 1;
+        if (u > ctc::kMostUnits) continue;
+        const int64_t passes = (rows * g + 31) / 32;
+        const int64_t cost = (passes + warps - 1) / warps * (u * (es == 4 ? 34 : 66) + (64 / es + g - 1) / g * 8 + 130);
+        if (best != 0 && cost >= best) continue;
+        best = cost; *G = g; *U = u;
+    }
+    return best;
+}
+
+// Whether rows are read into registers.  The lanes that share a row, and with them the order of its
+// sums, are the same whatever the grid.  Measured, the call (with its collapse) by bulk-copy tiles and
+// from registers, us on one B200, rows not in L2:
+//   bf16: 200 rows of 2 KB 5.5 / 4.5, 4,500 of 700 bytes 5.9 / 5.6, 9,600 of 2 KB 11.4 / 10.2, 16,000
+//     17.5 / 13.1, 9,600 of 4 KB 18.0 / 13.9, 50,000 of 700 bytes (34 MB) 18.3 / 15.9, 30,000 of 2
+//     KB (61 MB) 20.6 / 21.7, 50,000 28.0 / 29.6, 130,000 54 / 62: beyond 40 MB instructions bound both,
+//     and the tiles' few lanes per row spend fewer of them on what is done once per row
+//   fp32, half the logits per byte: 9,600 rows of 4 KB 15.4 / 11.3, 130,000 of 516 bytes (66 MB) 24.7 /
+//     19.0, 30,000 of 4 KB (122 MB) 25.6 / 24.9, 50,000 37.3 / 37.2, 130,000 81.8 / 84.5
+static void plan_direct(ssd_dtype dtype, int V, int64_t N, const ssd_launch_opts *o, CtcPlan *pl) {
+    if (o && (o->kernel || o->split || o->stages || o->stage_bytes || o->fma_exp)) return;
+    const int es = dtype == SSD_F32 ? 4 : 2;
+    const int64_t sms = device_sm_count(), row_bytes = (int64_t)V * es;
+    if (sms <= 0 || N < 1 || row_bytes / 32 > 32 * ctc::kMostUnits) return;
+    if (N > (dtype == SSD_F32 ? 200ll << 20 : 40ll << 20) / row_bytes) return;
+    pl->direct = lanes_for(dtype, V, N, sms * direct::kCtasPerSm * direct::kWarps, &pl->d_lanes, &pl->d_units) != 0;
+}
+
 // Kernel and launch shape of the frame-statistics pass for these sizes.
 // G lanes share a row, a warp works on 32/G rows at a time (one pass), and a tile is a whole
 // number of passes.  Few lanes per row spread the per-pass work (row geometry, masked first and
@@ -915,6 +981,7 @@ int plan_ctc(ssd_dtype dtype, int V, int64_t ld, int64_t N, int B, const ssd_lau
           (size_t)warps * stage_stride
         : 0;
     pl.workspace_bytes = 2048;      // the tile counters, 256 bytes apart, and room to spare
+    plan_direct(dtype, V, N, o, &pl);
     *plan = pl;
     return SSD_OK;
 }
@@ -924,6 +991,22 @@ template <typename T, int kF> void (*pick_ctc(int G))(const CtcParams) {
     return G == 2 ? ctc_rows_tma<T, 2, kF> : G == 4 ? ctc_rows_tma<T, 4, kF>
          : G == 8 ? ctc_rows_tma<T, 8, kF> : G == 16 ? ctc_rows_tma<T, 16, kF>
                                                      : ctc_rows_tma<T, 32, kF>;
+}
+template <typename T> void (*pick_direct(int G, int U))(const CtcParams) {
+    switch (G * 8 + U) {
+        case 8 * 8 + 1: return ctc_rows_direct<T, 8, 1>;
+        case 8 * 8 + 2: return ctc_rows_direct<T, 8, 2>;
+        case 8 * 8 + 3: return ctc_rows_direct<T, 8, 3>;
+        case 8 * 8 + 4: return ctc_rows_direct<T, 8, 4>;
+        case 16 * 8 + 1: return ctc_rows_direct<T, 16, 1>;
+        case 16 * 8 + 2: return ctc_rows_direct<T, 16, 2>;
+        case 16 * 8 + 3: return ctc_rows_direct<T, 16, 3>;
+        case 16 * 8 + 4: return ctc_rows_direct<T, 16, 4>;
+        case 32 * 8 + 1: return ctc_rows_direct<T, 32, 1>;
+        case 32 * 8 + 2: return ctc_rows_direct<T, 32, 2>;
+        case 32 * 8 + 3: return ctc_rows_direct<T, 32, 3>;
+        default: return ctc_rows_direct<T, 32, 4>;
+    }
 }
 }  // namespace
 
@@ -947,7 +1030,15 @@ int launch_ctc_rows(const void *logits, ssd_dtype dtype, int V, int64_t ld, int6
         e = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_begin), L.stream);
         if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
     }
-    if (kernel != 1) {
+    if (plan.direct) {
+        const int64_t most = o && o->ctas > 0 ? o->ctas : (int64_t)device_sm_count() * direct::kCtasPerSm;
+        const unsigned threads = o && o->warps > 0 && o->warps < direct::kWarps ? o->warps * 32 : direct::kThreads;
+        const int64_t passes = (N * plan.d_lanes + 31) / 32;
+        e = launch_pdl(dtype == SSD_F32 ? pick_direct<float>(plan.d_lanes, plan.d_units)
+                                        : pick_direct<bf16_t>(plan.d_lanes, plan.d_units),
+                       (unsigned)(passes < most ? passes : most), threads, 0, L.stream, p);
+        if (e != cudaSuccess) { record_cuda_error(e); return SSD_ERR_CUDA; }
+    } else if (kernel != 1) {
         p.rows_per_tile = R; p.stages = 1; p.warps = plan.warps;
         p.stage_stride = plan.stage_stride;
         p.iters = plan.iters; p.tail_from = plan.tail_from;
