@@ -296,26 +296,43 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
     }
     Mx = warp_max(Mx);
     vm = warp_max(vm);
-    float S = 0.f;
+    // Sums are taken relative to the largest logit, and its own exponential, which every sum of a
+    // partial that holds it carries with an error of 2^-22, is exchanged for 1 in one of them: what is
+    // left over 1 is all that the logarithm of a confident row is about.
+    const bool plain = vm > kNegInit;
+    const float base = plain ? vm : Mx;
     int vi = INT_MAX;
     for (int q = lane; q < P; q += 32) {
         const float4 v = get(q);
-        S += v.y * ex2((v.x - Mx) * kLog2e);
         if (v.z == vm) vi = min(vi, __float_as_int(v.w));
     }
-    S = warp_sum(S);
     vi = __reduce_min_sync(0xffffffffu, vi);
-    if (kUnit && vi >= 0 && vi < V) {
+    const int found = vi;
+    float beside = -INFINITY;
+    if (kUnit && vi >= 0 && vi < V) {             // on its way while the sums are joined
         const int64_t e = (int64_t)vi + lane;
-        const bool hit = lane < 32 / Elem<T>::kBytes && e < V &&
-                         Elem<T>::load(row + e * Elem<T>::kBytes) == vm;
-        const unsigned hits = __ballot_sync(0xffffffffu, hit);
+        if (lane < 32 / Elem<T>::kBytes && e < V) beside = Elem<T>::load(row + e * Elem<T>::kBytes);
+    }
+    float S = 0.f;
+    for (int q = lane; q < P; q += 32) {
+        const float4 v = get(q);
+        float sum = v.y;
+        if (plain && v.z == vm && __float_as_int(v.w) == found) {     // one partial: each has its own indexes
+            const float nmh = -(v.x * kLog2e);
+            sum -= ex2(fmaf(vm, kLog2e, nmh)) * ex2(-fmaf(v.x, kLog2e, nmh));
+        }
+        S += sum * ex2((v.x - base) * kLog2e);
+    }
+    S = warp_sum(S);
+    if (kUnit) {
+        const unsigned hits = __ballot_sync(0xffffffffu, beside == vm && vm > -INFINITY);
         if (hits) vi += __ffs(hits) - 1;
     }
     GreedyRow g;
-    const float lnS = logf(S);
-    g.lse = Mx + lnS;
-    g.logp = (vm - Mx) - lnS;
+    // what is left is not negative but for rounding; a NaN stays one
+    const float lnS = plain ? log1pf(S < 0.f ? 0.f : S) : logf(S);
+    g.lse = base + lnS;
+    g.logp = (vm - base) - lnS;
     g.status = fabsf(g.lse) < INFINITY ? 0u : (uint32_t)SSD_UTT_NONFINITE;
     g.token = (vi < 0 || vi >= V) ? 0 : vi;
     return g;
