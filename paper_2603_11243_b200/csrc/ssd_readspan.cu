@@ -141,19 +141,18 @@ int32_t ssd_verify_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, int
         if (plan_verify(greedy ? 0 : B, M, V, dtype, opts, at, &whole) == SSD_OK && whole.whole)
             walk_cut(whole.whole_cut, 128);
     }
+    // with a skip flag per utterance the rows may be cut more finely (kCuts), and fp32 rows be read by the
+    // direct-load kernel at all
+    VerifyPlan skipping;
+    if (plan_verify(B, M, V, dtype, opts, RowsAt{reinterpret_cast<const void *>((uintptr_t)base_addr), ld, false, true},
+                    &skipping) != SSD_OK)
+        skipping = plan;
+    for (int k = 0; skipping.direct && k < direct::kCuts; ++k) {
+        const direct::Cut cut = skipping.cut[k], before = skipping.cut[k > 0 ? k - 1 : 0];
+        if (k == 0 || cut.spans != before.spans || cut.blocks != before.blocks) walk_cut(cut, skipping.pairs);
+    }
     if (plan.direct) {
-        // with a skip flag per utterance the rows may be cut more finely (kCuts)
-        VerifyPlan skipping = plan;
-        if (plan_verify(B, M, V, dtype, opts,
-                        RowsAt{reinterpret_cast<const void *>((uintptr_t)base_addr), ld, false, true},
-                        &skipping) != SSD_OK || !skipping.direct)
-            skipping = plan;
-        for (int k = -1; k < direct::kCuts; ++k) {
-            const direct::Cut cut = k < 0 ? plan.cut[0] : skipping.cut[k];
-            const direct::Cut before = k < 1 ? plan.cut[0] : skipping.cut[k - 1];
-            if (k >= 0 && cut.spans == before.spans && cut.blocks == before.blocks) continue;
-            walk_cut(cut, k < 0 ? plan.pairs : skipping.pairs);
-        }
+        walk_cut(plan.cut[0], plan.pairs);
     } else if (plan.kernel == 2) {
         const int max_chunks = plan.stage_bytes >> 4;
         for (int64_t row = 0; row < M; ++row) {

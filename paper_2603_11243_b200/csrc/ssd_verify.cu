@@ -852,16 +852,20 @@ unsigned long long next_epoch();
 //     98 KB: 31.9 / 33.7; 8,000: 136 / 141), direct beyond (12,000: 200 / 200; 16,000: 265 / 245;
 //     22,000 of 200 KB: 708 / 664): it spends a fifth fewer instructions on a logit.  With `skip`
 //     half of the rows are taken to be read (a batch of 1.3 GB, partly gated: 199 / 206).
-//   fp32: the ring (16,000 of 192 KB: 437 / 455; 1,000: 36.1 / 38.8), which has more bytes in
-//     flight and half the logits per byte; the greedy step on few rows: direct (200 of 196 KB:
-//     14.0 / 12.3; 300 of 608 KB: 36.4 / 35.8; 500 of 196 KB: 21.9 / 23.3)
+//   fp32, up to 400 MB: direct (50 rows of 240 KB 11.7 / 9.0, 100 15.3 / 11.6; 250 of 128 KB 13.8 / 11.7,
+//     600 19.8 / 18.0, 1,500 35.9 / 35.1; 600 of 608 KB 63.6 / 58.6; 3,000 of 128 KB 63.1 / 62.1): the ring
+//     cuts few rows into spans of 32 KB and hands each over.  Beyond: the ring (6,000 of 128 KB 117.0 /
+//     118.3, 6,000 of 240 KB 208.8 / 213.0, 16,000 of 192 KB 437 / 455), which has more bytes in flight and
+//     half the logits per byte.  That is with skip flags, as behind a gate; without, the ring throughout,
+//     which is what ssd_verify_read_span replays for fp32.  The greedy step on few rows: direct (200 of
+//     196 KB: 14.0 / 12.3; 300 of 608 KB: 36.4 / 35.8; 500 of 196 KB: 21.9 / 23.3)
 // The greedy step on bf16 rows: direct (1,024 of 304 KB: 59.5 / 55.1; 24 of 98 KB: 14.0 / 12.6).
 static int use_direct(int64_t M, int64_t row_bytes, ssd_dtype dtype, int kernel, int sms,
                       const ssd_launch_opts *o, const RowsAt &at) {
     if (kernel != 2 || row_bytes >= (1ll << 30) || M >= (1ll << 30)) return 0;
     if (o && (o->kernel || o->warps || o->stages || o->stage_bytes || o->fma_exp || o->finish)) return 0;
     const bool few = M < 4ll * sms;
-    if (dtype == SSD_F32) return at.greedy && M <= 2ll * sms;
+    if (dtype == SSD_F32) return at.greedy ? M <= 2ll * sms : at.skip && M * row_bytes < 400ll << 20;
     if (at.greedy || few || row_bytes < 96 * 1024 || M * row_bytes >= (at.skip ? 2400ll : 1200ll) << 20) return 1;
     return (reinterpret_cast<uintptr_t>(at.base) | (uintptr_t)(at.ld * 2)) % 16 != 0;
 }
@@ -1044,7 +1048,6 @@ static size_t partials_offset(int B) {
 // Pairs per row that the streaming kernel of a plan leaves.
 static int pairs_per_row(const VerifyPlan &plan) { return plan.direct ? plan.pairs : plan.partials; }
 
-// fp32 logits come here with the arg max only (see use_direct).
 template <bool kArg>
 static cudaError_t launch_direct(const void *logits, ssd_dtype dtype, int V, int64_t ld, int64_t M,
                                  const int64_t *tok_off, int B, const uint8_t *skip, void *partials,
@@ -1064,7 +1067,7 @@ static cudaError_t launch_direct(const void *logits, ssd_dtype dtype, int V, int
     // 200 KB: none 694 us, one 674, two 683); with the arg max none is (1,024 of 304 KB: 55.1
     // against 55.9)
     auto kern = direct::verify_rows_direct<bf16_t, kArg ? 0 : 1, kArg>;
-    if (kArg && dtype == SSD_F32) kern = direct::verify_rows_direct<float, 0, true>;
+    if (dtype == SSD_F32) kern = direct::verify_rows_direct<float, 0, kArg>;
     return launch_pdl(kern, (unsigned)ctas, (unsigned)direct::kThreads, smem, stream, p);
 }
 
