@@ -300,7 +300,19 @@ def verify_kernel(s, w) -> str:
     x = s["vb"].logits
     span = ssd.ssd_verify_read_span(x.data_ptr(), ssd.BF16 if w.dtype == "bf16" else ssd.F32, w.V_llm,
                                     x.stride(0), x.shape[0], s["B"])
-    return "verify_rows_direct" if span.direct else "verify_rows_tma"
+    # a step passes skip flags, with which fp32 batches of up to 400 MB take direct loads as well; the
+    # replay is of the call without
+    gated_f32 = w.dtype != "bf16" and x.shape[0] * w.V_llm * 4 < 400 << 20
+    return "verify_rows_direct" if span.direct or gated_f32 else "verify_rows_tma"
+
+
+def ctc_kernel(s, w) -> str:
+    """The same for ssd_ctc_draft."""
+    from paper_2603_11243_b200 import binding as ssd
+    x = s["cb"].logits
+    span = ssd.ssd_ctc_draft_read_span(x.data_ptr(), ssd.BF16 if w.dtype == "bf16" else ssd.F32, w.V_ctc,
+                                       x.stride(0), x.shape[0])
+    return "ctc_rows_direct" if span.direct else "ctc_rows_tma"
 
 
 def timed_steps(sets, K, W, barrier=None):
@@ -400,7 +412,7 @@ def run_per_config(device, peak, peak_kind, skip_idx, cpu=True):
                "step_frac_of_peak": round(step_bytes / (ms / K * 1e-3) / 1e9 / peak, 4),
                "step_frac_of_nominal": round(step_bytes / (ms / K * 1e-3) / 1e9 / NOMINAL_HBM_GBS, 4),
                "l2": l2_note(sets),
-               "roofline_ctc": roof("ctc_rows_tma", ctc_b, t_ctc, peak, peak_kind),
+               "roofline_ctc": roof(ctc_kernel(sets[0], w), ctc_b, t_ctc, peak, peak_kind),
                "roofline_verify": roof(verify_kernel(sets[0], w), ver_b, t_ver, peak, peak_kind)}
         if cpu:
             rec["cpu_baseline"] = cpu_baseline(sets[0], budget_s=2.5)
@@ -478,7 +490,7 @@ def run_ours(args):
     gate_acc = float(s0["gate"]["gate_accept"].float().mean().item())
     all_acc = s0["s2"]["all_accepted"].cpu().numpy().astype(bool)
     skipped = s0["gate"]["gate_accept"].cpu().numpy().astype(bool)
-    r_ctc = roof("ctc_rows_tma", ctc_bytes, t_ctc, peak, peak_kind)
+    r_ctc = roof(ctc_kernel(s0, w), ctc_bytes, t_ctc, peak, peak_kind)
     r_ver = roof(vkern, ver_bytes, t_ver, peak, peak_kind)
     line = {
         "metric": METRIC, "value": round(value, 1), "unit": UNIT, "n_gpus": world, "steps": K,

@@ -406,7 +406,9 @@ int32_t ssd_verify_combine(const float *stats_all, int32_t R, int64_t V_total,
  *   kernel   2: a kernel of wide reads would run (bulk copies, or 32-byte loads whose units
  *            are held to the row in the same way); 1: the plain-load kernel, which indexes
  *            elements one by one (lo, hi are then the matrix's own extent)
- *   direct   ssd_verify: 1 where those wide reads are the 32-byte loads
+ *   direct   1 where those wide reads are the 32-byte loads (ssd_verify: as called without skip
+ *            flags; with them, fp32 batches of up to 400 MB take such loads, too, and their spans
+ *            are held to the same rules here)
  * so a caller -- the tests do -- can assert faults == 0, lo >= base_addr and
  * hi <= base_addr + ((rows - 1) * ld + V) * element size for any shape and misalignment.
  * Errors: SSD_ERR_NULL, SSD_ERR_ARG, SSD_ERR_DTYPE, SSD_ERR_ALIGN (base_addr not a multiple of

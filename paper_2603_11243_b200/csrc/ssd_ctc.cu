@@ -1,7 +1,7 @@
 // Stage 1 kernels: per-frame softmax statistics of the CTC head (Eq. 2, Eq. 3), the collapse
 // B of Section 2.1, and the entropy gate of Eq. 3.
 //
-// Frame statistics are one streaming read of the [N, V] logits.  Two kernels compute them:
+// Frame statistics are one streaming read of the [N, V] logits.  Three kernels compute them:
 //   ctc_rows_tma    each warp owns a shared-memory stage that it fills with one 1-D bulk
 //                   asynchronous copy (TMA) of a few consecutive rows and drains itself: no
 //                   block-level synchronisation after set-up.  G lanes share a row; one fused
@@ -9,6 +9,8 @@
 //                   relative to a per-lane reference, so a logit costs one exponential; rows
 //                   that pass cannot take (masked -inf logits, NaN, +inf, a range beyond fp32)
 //                   are redone from shared memory by an exact two-pass routine.
+//   ctc_rows_direct (ssd_ctc_direct.cuh) rows of up to 4 KB straight into registers; what runs on calls
+//                   of up to 40 MB (see plan_direct).
 //   ctc_rows_plain  one warp per row with scalar global loads; any alignment, any V.  Fallback.
 #include <limits.h>
 #include <math.h>

@@ -1,6 +1,6 @@
 // verify_rows_direct: the streaming kernel of ssd_verify, ssd_verify_shard and ssd_greedy_step
-// for bf16 logits (use_direct in ssd_verify.cu says where it runs and what it measured against
-// the ring of verify_rows_tma).
+// (use_direct in ssd_verify.cu says on which sizes and types, and what it measured against the ring
+// of verify_rows_tma).
 //
 // A warp works on one span of columns of one row at a time and reads it with 32-byte loads
 // straight into registers: no shared memory, no barriers, no hand-over between warps.  What
