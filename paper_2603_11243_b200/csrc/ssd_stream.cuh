@@ -288,12 +288,29 @@ struct GreedyRow {
 };
 template <typename T, bool kUnit, typename Get>
 __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row, int V, int lane) {
+    // three looks at the partials: held in registers where they are few enough, since in the workspace
+    // each look is a round trip (450 rows of 220 KB, 10 partials each: 20.9 us the call, 21.8 with three)
+    constexpr int L = 4;
+    float4 held[L];
+    const bool few = P <= 32 * L;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+        held[j] = make_float4(kNegInit, 0.f, -INFINITY, __int_as_float(INT_MAX));
+        if (few && 32 * j + lane < P) held[j] = get(32 * j + lane);
+    }
+    auto each = [&](auto look) {
+        if (few) {
+#pragma unroll
+            for (int j = 0; j < L; ++j) look(held[j]);
+        } else {
+            for (int q = lane; q < P; q += 32) look(get(q));
+        }
+    };
     float Mx = kNegInit, vm = -INFINITY;
-    for (int q = lane; q < P; q += 32) {
-        const float4 v = get(q);
+    each([&](const float4 &v) {
         Mx = fmaxf(Mx, v.x);
         vm = fmaxf(vm, v.z);
-    }
+    });
     Mx = warp_max(Mx);
     vm = warp_max(vm);
     // Sums are taken relative to the largest logit, and its own exponential, which every sum of a
@@ -302,10 +319,9 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
     const bool plain = vm > kNegInit;
     const float base = plain ? vm : Mx;
     int vi = INT_MAX;
-    for (int q = lane; q < P; q += 32) {
-        const float4 v = get(q);
+    each([&](const float4 &v) {
         if (v.z == vm) vi = min(vi, __float_as_int(v.w));
-    }
+    });
     vi = __reduce_min_sync(0xffffffffu, vi);
     const int found = vi;
     float beside = -INFINITY;
@@ -314,15 +330,14 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
         if (lane < 32 / Elem<T>::kBytes && e < V) beside = Elem<T>::load(row + e * Elem<T>::kBytes);
     }
     float S = 0.f;
-    for (int q = lane; q < P; q += 32) {
-        const float4 v = get(q);
+    each([&](const float4 &v) {
         float sum = v.y;
         if (plain && v.z == vm && __float_as_int(v.w) == found) {     // one partial: each has its own indexes
             const float nmh = -(v.x * kLog2e);
             sum -= ex2(fmaf(vm, kLog2e, nmh)) * ex2(-fmaf(v.x, kLog2e, nmh));
         }
         S += sum * ex2((v.x - base) * kLog2e);
-    }
+    });
     S = warp_sum(S);
     if (kUnit) {
         const unsigned hits = __ballot_sync(0xffffffffu, beside == vm && vm > -INFINITY);
