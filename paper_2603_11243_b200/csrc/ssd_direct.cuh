@@ -350,7 +350,9 @@ __device__ __forceinline__ void stream_spans(const DirectParams &p, const Cut cu
             add(u, last);
             Sw = warp_sum(total + ((Sa.x + Sa.y) + (Sb.x + Sb.y) + ex2(fmaf(my_edge, kLog2e, ref.nmh))));
             fast = Sw < kSpanSumLimit;
-            Sw *= ex2(-fmaf(ref.m, kLog2e, ref.nmh));   // every exponent carried m*log2e + nmh
+            // every exponent carried m*log2e + nmh; with the arg max the reference's own is then exactly 1
+            const float carried = fmaf(ref.m, kLog2e, ref.nmh);
+            if (kArg) Sw /= ex2(carried); else Sw *= ex2(-carried);
         }
         SpanResult out;
         if (fast) {

@@ -178,13 +178,16 @@ __device__ __forceinline__ void consume_stage(uint32_t a0, int n, int ct, int NT
     if (kArg) resolve_arg<T>(a0, elem0, at);
 }
 
-// Warp-level merge of the lanes' (m, S) into one pair relative to the warp maximum.
-__device__ __forceinline__ float2 warp_merge(const Online &st) {
+// Warp-level merge of the lanes' (m, S) into one pair relative to the warp maximum.  Exponents carried
+// +ml: it is taken out, with the arg max by a division, after which a logit equal to the warp's maximum
+// has added exactly 1 (see greedy_row).
+template <bool kArg> __device__ __forceinline__ float2 warp_merge(const Online &st) {
     const float S = st.total();
-    const float ml = fmaf(st.m, kLog2e, -st.mh);        // exponents carried +ml: take it out
+    const float ml = fmaf(st.m, kLog2e, -st.mh);
     const float M = warp_max(st.m);
     // S == 0 covers lanes that saw nothing (their m is -inf); a NaN sum still propagates
-    const float Sw = warp_sum(S == 0.f ? 0.f : S * ex2(fmaf(st.m - M, kLog2e, -ml)));
+    const float rebased = kArg ? S / ex2(ml) * ex2((st.m - M) * kLog2e) : S * ex2(fmaf(st.m - M, kLog2e, -ml));
+    const float Sw = warp_sum(S == 0.f ? 0.f : rebased);
     return make_float2(M, Sw);
 }
 
@@ -313,9 +316,12 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
     });
     Mx = warp_max(Mx);
     vm = warp_max(vm);
-    // Sums are taken relative to the largest logit, and its own exponential, which every sum of a
-    // partial that holds it carries with an error of 2^-22, is exchanged for 1 in one of them: what is
-    // left over 1 is all that the logarithm of a confident row is about.
+    // Sums are taken relative to the largest logit, and its own exponential is taken out of the one partial
+    // that holds it: what is left beside it is all that the logarithm of a confident row is about.  It is
+    // taken in the form that the partial has it, with one rounding: 1 where the logit is the partial's
+    // reference, a quotient that both carry what rounding left out of x * log2e above a reference of the
+    // fast pass (below 4,096), and a power of the difference elsewhere (1e10 * log2e is rounded by 440:
+    // neither part of the quotient is in fp32's range).
     const bool plain = vm > kNegInit;
     const float base = plain ? vm : Mx;
     int vi = INT_MAX;
@@ -334,7 +340,8 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
         float sum = v.y;
         if (plain && v.z == vm && __float_as_int(v.w) == found) {     // one partial: each has its own indexes
             const float nmh = -(v.x * kLog2e);
-            sum -= ex2(fmaf(vm, kLog2e, nmh)) * ex2(-fmaf(v.x, kLog2e, nmh));
+            sum -= fabsf(v.x) < 4096.f ? ex2(fmaf(vm, kLog2e, nmh)) / ex2(fmaf(v.x, kLog2e, nmh))
+                                       : ex2((vm - v.x) * kLog2e);
         }
         S += sum * ex2((v.x - base) * kLog2e);
     });

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
             __syncwarp();
             if (lane == 0) mbar_arrive(empty0 + s * 8);
             if (flags & kFlagLast) {
-                const float2 r = warp_merge(st);
+                const float2 r = warp_merge<kArg>(st);
                 if (kArg) {
                     // warp arg max: largest value, lowest index among the lanes that hold it
                     const float vm = warp_max(at.vmax);
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(544, 1) verify_rows_fin(const FinParams q) {
             consume_stage<T, kF, false>(stage0 + (uint32_t)s * p.stage_bytes, n, ct, NT, st, 0, unused);
             if (flags & kFlagLast) {
                 const int slot = (int)desc[s].slot;
-                const float2 r = warp_merge(st);
+                const float2 r = warp_merge<false>(st);
                 if (lane == 0) spart[slot * CW + cw] = r;
                 st.reset();
             }

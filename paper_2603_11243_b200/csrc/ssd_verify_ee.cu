@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(576, 1) verify_rows_ee(const EeParams p) {
             __syncwarp();
             if (lane == 0) mbar_arrive(empty0 + s * 8);      // the stage first: its next copy can start
             if (flags & kFlagLast) {
-                const float2 r = warp_merge(st);
+                const float2 r = warp_merge<false>(st);
                 if (lane == 0) {
                     spart[slot * CW + cw] = r;
                     mbar_arrive(rowdone0 + slot * 8);        // releases this and the logit above

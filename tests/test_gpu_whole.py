@@ -36,6 +36,39 @@ def test_greedy_step(cuda_device, R, V, dtype):
     assert np.abs(got["next_logp"].cpu().numpy() - want["next_logp"]).max() <= H.FLOAT_TOL
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", [600, 9000])
+@pytest.mark.parametrize("split", [0, 1])
+def test_greedy_step_of_large_finite_logits(cuda_device, split, V, dtype):
+    """A token forced with a large logit, and rows with nothing above a large negative one, by the clusters
+    and by the pair kernel: finite rows, whatever the rounding of a logit times log2e."""
+    largest = torch.finfo(dtype).max
+    values = (5000.0, 1e6, 1e9, 2e9, 1e10, 1e12, 1e20, 1e30, 1e38, largest, -5000.0, -1e9, -1e10, -1e20, -9e29)
+    wide = _matrix(2 * len(values), V, dtype, V)
+    x = wide[:, 3:3 + V]
+    for k, v in enumerate(values):
+        x[2 * k + 1] = -largest                    # alone, and behind a masked first half
+        if v > 0:
+            x[2 * k, 11 * k] = x[2 * k + 1, V - 1 - k] = v
+        else:
+            x[2 * k, :] = v
+            x[2 * k + 1, V // 2:] = v
+    want = ref.greedy_step(H.storage_numpy(x.contiguous()), V)
+    got = ssd.ssd_greedy_step(wide.to(cuda_device)[:, 3:3 + V], opts=H.opts(split=split) if split else None)
+    torch.cuda.synchronize()
+    got = {k: got[k].cpu().numpy() for k in ("next_token", "next_logp", "row_lse", "row_status")}
+    assert not got["row_status"].any()
+    np.testing.assert_array_equal(got["next_token"], want["next_token"])
+    # nothing beside a forced token; V or V - V // 2 equal logits (a difference of log-sum-exps of 1e20 does
+    # not show either in 64 bits)
+    likely = [0.0 if v > 0 else -np.log(n) for v in values for n in (V, V - V // 2)]
+    assert np.abs(got["next_logp"] - likely).max() <= H.FLOAT_TOL
+    # the sum and the result are rounded once each
+    assert (np.abs(got["row_lse"] - want["row_lse"]) <= H.FLOAT_TOL + 2.0 ** -23 * np.abs(want["row_lse"])).all()
+    forced = [r for r in range(len(x)) if values[r // 2] > 0]
+    assert (got["next_logp"][forced] == 0).all()
+
+
 # [0, M] as it should be; a gap before, between and after; one utterance's end before its start; one
 # past the matrix; two that overlap
 OFFSETS = {"sound": lambda M: [0, M // 3, M // 3, M], "gaps": lambda M: [M // 5, M // 2, M - 1],
