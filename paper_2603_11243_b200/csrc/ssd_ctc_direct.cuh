@@ -50,6 +50,11 @@ template <int G> __device__ __forceinline__ float group_sum(float v) {
     return v;
 }
 
+// A row's results are good: a sum in range, relative to a finite maximum.
+__device__ __forceinline__ bool row_is_sound(float m, float S) {
+    return S > 0.5f && S < INFINITY && fabsf(m) < INFINITY;      // else NaN / +inf / only -inf
+}
+
 // Log-sum-exp and entropy of a row with maximum m from S, the sum of 2^t, and A, that of t * 2^t, with
 // t = x * log2e - fl(m * log2e).  What rounding left out of fl(m * log2e) every exponent carries: it
 // comes out of the log-sum-exp and cancels in the entropy.
@@ -58,11 +63,13 @@ __device__ __forceinline__ void close_row(float m, float S, float A, RowOut &out
     const float lnS = logf(S);
     out.lse = m + (lnS - ml * kLn2);
     out.H = fmaxf(lnS - kLn2 * (A / S), 0.f);
-    if (!(S > 0.5f) || !(S < INFINITY) || !(fabsf(m) < INFINITY))
-        out.H = __int_as_float(0x7fc00000);       // NaN / +inf / nothing finite: flagged downstream
+    if (!row_is_sound(m, S)) out.H = __int_as_float(0x7fc00000);       // flagged downstream
 }
 
-// A row with a NaN, a +inf or nothing above the floor, element by element.
+// A row with a NaN, a +inf, nothing above the floor, or a maximum so large that an exponent should not
+// carry what rounding leaves out of its product with log2e (kMostExact: up to 1/16; from 1.2e7 up it
+// reaches 1, from 3e9 fp32's exponent range), element by element and by differences.
+constexpr float kMostExact = 1048576.f;
 template <typename T, int G>
 __device__ __noinline__ RowOut row_by_elements(const char *x, int row_bytes, int sub) {
     constexpr int ES = Elem<T>::kBytes;
@@ -76,14 +83,17 @@ __device__ __noinline__ RowOut row_by_elements(const char *x, int row_bytes, int
     RowOut out;
     out.arg = group_min<G>(m == top ? at : INT_MAX);
     if (out.arg == INT_MAX) out.arg = 0;
-    const float nmh = -(top * kLog2e);
     float S = 0.f, A = 0.f;
     for (int e = sub * ES; e < row_bytes; e += G * ES) {
-        const float t = fmaf(fmax_nan(Elem<T>::load(x + e), kFloor), kLog2e, nmh), p = ex2(t);
+        const float t = (Elem<T>::load(x + e) - top) * kLog2e, p = ex2(t);
         S += p;
         A += p > 0.f ? t * p : 0.f;
     }
-    close_row(top, group_sum<G>(S), group_sum<G>(A), out);
+    S = group_sum<G>(S);
+    A = group_sum<G>(A);
+    const float lnS = logf(S);
+    out.lse = top + lnS;
+    out.H = row_is_sound(top, S) ? fmaxf(lnS - kLn2 * (A / S), 0.f) : __int_as_float(0x7fc00000);
     return out;
 }
 
@@ -231,7 +241,7 @@ __device__ __forceinline__ RowOut reduce_row(Row<T, G, U> &row, const char *x, i
     read();
     S = group_sum<G>(S);
     A = group_sum<G>(A);
-    const bool odd = !(m > -1.0e29f) || !(S > 0.5f) || !(S < INFINITY);
+    const bool odd = !(fabsf(m) < kMostExact) || !row_is_sound(m, S);
     if (__any_sync(0xffffffffu, odd)) {
         const RowOut slow = row_by_elements<T, G>(x, row_bytes, sub);
         if (odd) return slow;

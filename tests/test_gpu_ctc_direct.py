@@ -73,3 +73,33 @@ def test_rows_that_are_not_plain(cuda_device, V, dtype):
     d = (a["frame_lse"] - b["frame_lse"])[~odd].abs()
     # a few units in the last place of values up to 30,000
     assert bool((d <= H.FLOAT_TOL + 4 * 2.0 ** -23 * b["frame_lse"][~odd].abs()).all())
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", [9, 300, 1000])
+@pytest.mark.parametrize("times", [1, 4])
+def test_rows_of_large_finite_logits(cuda_device, times, V, dtype):
+    """One large logit, alone and among others; rows with nothing above a large negative one; also columns
+    of a matrix so wide that the bulk-copy tiles do not take it."""
+    largest = torch.finfo(dtype).max
+    values = (1e6, 1.3e7, 2e7, 1e8, 1e10, 1e20, 1e38, largest, -1e6, -2e7, -1e10, -1e20, -1e30, -largest)
+    g = torch.Generator()
+    g.manual_seed(V)
+    x = torch.randn((2 * len(values), V * times), generator=g).to(dtype)[:, :V]
+    for k, v in enumerate(values):
+        x[2 * k + 1] = float("-inf")
+        if v > 0:
+            x[2 * k, k % V] = x[2 * k + 1, V - 1 - k % V] = v
+        else:
+            x[2 * k, :] = v
+            x[2 * k + 1, V // 2:] = v
+    orc = ref.ctc_draft(H.storage_numpy(x.contiguous()), V, np.array([0, len(x)], np.int64), 0, 0)
+    wide = torch.zeros((len(x), V * times), dtype=dtype, device=cuda_device)
+    wide[:, :V] = x.to(cuda_device)
+    out = _statistics(wide[:, :V], cuda_device)
+    np.testing.assert_array_equal(out["frame_argmax"].cpu().numpy(), orc["frame_argmax"])
+    # equal logits or one by itself, whatever they are: 64 bits do not hold this beside 1e20 either
+    entropy = [0.0 if v > 0 else np.log(n) for v in values for n in (V, V - V // 2)]
+    assert np.abs(out["frame_entropy"].cpu().numpy() - entropy).max() <= H.FLOAT_TOL
+    d = np.abs(out["frame_lse"].cpu().numpy().astype(np.float64) - orc["frame_lse"])
+    assert (d <= H.FLOAT_TOL + 2.0 ** -23 * np.abs(orc["frame_lse"])).all()
