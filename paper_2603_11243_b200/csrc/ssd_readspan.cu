@@ -38,7 +38,20 @@ int32_t ssd_ctc_draft_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, 
     const int64_t total = N > 0 ? (N - 1) * row_pitch + row_bytes : 0;
     const uintptr_t base = (uintptr_t)base_addr;
     Span sp;
-    if (plan.kernel == 2) {
+    if (plan.direct) {
+        // a row read into registers: whole units and two ragged ends of less than one each, the units no
+        // more than the lanes that share it have room for
+        for (int64_t row = 0; row < N; ++row) {
+            const uintptr_t g0 = base + (uintptr_t)(row * row_pitch);
+            const ranges::RowUnits r = ranges::row_units(g0, (int)row_bytes);
+            bool ok = r.units == 0 || (g0 + (uintptr_t)r.head) % 32 == 0;
+            ok = ok && r.head >= 0 && r.head < 32 && r.units >= 0 && r.units % 32 == 0;
+            ok = ok && r.row == row_bytes && r.row - r.head - r.units >= 0 && r.row - r.head - r.units < 32;
+            ok = ok && r.units <= 32 * plan.d_lanes * plan.d_units;
+            if (!ok) ++sp.faults;
+            sp.add(g0, g0 + (uintptr_t)r.row);
+        }
+    } else if (plan.kernel == 2) {
         for (int64_t tile = 0; tile < plan.num_tiles; ++tile) {
             const ranges::TileReads t =
                 ranges::tile_reads(base, total, row_pitch, row_bytes, N, plan.rows_per_tile, tile);
@@ -77,22 +90,10 @@ int32_t ssd_ctc_draft_read_span(uint64_t base_addr, ssd_dtype dtype, int32_t V, 
     } else if (N > 0) {
         sp.add(base, base + (uintptr_t)total);   // element-wise loads of the rows' own bytes
     }
-    // a row read into registers: whole units and two ragged ends of less than one each, the units no
-    // more than the lanes that share it have room for
-    for (int64_t row = 0; row < N; ++row) {
-        const uintptr_t g0 = base + (uintptr_t)(row * row_pitch);
-        const ranges::RowUnits r = ranges::row_units(g0, (int)row_bytes);
-        bool ok = r.units == 0 || (g0 + (uintptr_t)r.head) % 32 == 0;
-        ok = ok && r.head >= 0 && r.head < 32 && r.units >= 0 && r.units % 32 == 0;
-        ok = ok && r.row == row_bytes && r.row - r.head - r.units >= 0 && r.row - r.head - r.units < 32;
-        if (plan.direct) ok = ok && r.units <= 32 * plan.d_lanes * plan.d_units;
-        if (!ok) ++sp.faults;
-        sp.add(g0, g0 + (uintptr_t)r.row);
-    }
     out->lo = sp.hi ? sp.lo : base_addr;
     out->hi = sp.hi ? sp.hi : base_addr;
     out->faults = sp.faults;
-    out->kernel = plan.kernel;
+    out->kernel = plan.direct ? 2 : plan.kernel;
     out->direct = plan.direct;
     return SSD_OK;
 }

@@ -54,6 +54,29 @@ def test_ctc_reads_with_forced_shapes():
                 assert r.hi == BASE + mis + _extent(N, V + 1, V, 2)
 
 
+def test_ctc_reads_of_the_kernel_that_runs():
+    """Tiles, which short rows only take where they are asked for, rows read into registers, and rows that
+    are longer than either takes: 2 GB and more for a row's own bytes."""
+    tiles = ssd.LaunchOpts()
+    tiles.kernel = 2
+    reached = {0: 0, 1: 0}
+    for V, pad, N in itertools.product(VS, (0, 1, 3, 8), (1, 2, 33, 1000, 4097)):
+        for dtype, es in ((ssd.F32, 4), (ssd.BF16, 2)):
+            for mis, o in itertools.product((0, es, 16 - es), (None, tiles)):
+                r = ssd.ssd_ctc_draft_read_span(BASE + mis, dtype, V, V + pad, N, o)
+                assert r.faults == 0 and r.kernel == 2 and not (o and r.direct), (V, pad, N, mis)
+                assert r.lo == BASE + mis and r.hi == BASE + mis + _extent(N, V + pad, V, es), (V, pad, N, mis)
+                reached[r.direct] += 1
+    assert min(reached.values()) > 1000
+    # a matrix so much wider than its rows that no tile would hold them: still registers
+    r = ssd.ssd_ctc_draft_read_span(BASE + 2, ssd.BF16, 348, 2000, 500)
+    assert (r.faults, r.kernel, r.direct, r.hi) == (0, 2, 1, BASE + 2 + _extent(500, 2000, 348, 2))
+    for V in ((1 << 29) - 1, 1 << 29, (1 << 29) + 5, (1 << 31) - 1):
+        r = ssd.ssd_ctc_draft_read_span(BASE + 4, ssd.F32, V, V, 3)
+        assert (r.faults, r.kernel, r.direct) == (0, 1, 0), V
+        assert r.lo == BASE + 4 and r.hi == BASE + 4 + _extent(3, V, V, 4), V
+
+
 @pytest.mark.parametrize("dtype,es", [(ssd.F32, 4), (ssd.BF16, 2)])
 def test_verify_reads_stay_inside_each_row(dtype, es):
     checked_bulk = 0
