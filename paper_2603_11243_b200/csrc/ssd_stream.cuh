@@ -268,6 +268,24 @@ __device__ __forceinline__ int count_rows_by_warp(const int64_t *tok_off, const 
     __syncwarp();
     return total;
 }
+// Whether none of the B + 1 offsets is below the one before it.  Called by all lanes of a warp.
+__device__ __forceinline__ int offsets_ordered(const int64_t *off, int B) {
+    constexpr int L = 4;                 // pairs a lane has in flight
+    const int lane = threadIdx.x & 31;
+    bool ok = true;
+    for (int b0 = 0; b0 < B; b0 += 32 * L) {
+        int64_t i0[L], i1[L];
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int b = min(b0 + 32 * j + lane, B - 1);
+            i0[j] = off[b];
+            i1[j] = off[b + 1];
+        }
+#pragma unroll
+        for (int j = 0; j < L; ++j) ok = ok && i0[j] <= i1[j];
+    }
+    return __all_sync(0xffffffffu, ok);
+}
 // The utterance that has row number `at`, below the total: the last one with no more than that many
 // rows before it.
 __device__ __forceinline__ int utterance_of_count(const int32_t *act, int B, int at) {

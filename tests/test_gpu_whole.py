@@ -73,7 +73,12 @@ def test_greedy_step_of_large_finite_logits(cuda_device, split, V, dtype):
 # past the matrix; two that overlap
 OFFSETS = {"sound": lambda M: [0, M // 3, M // 3, M], "gaps": lambda M: [M // 5, M // 2, M - 1],
            "reversed": lambda M: [0, M // 2, M // 4, M], "past": lambda M: [0, M // 2, M + 3],
-           "twice": lambda M: [0, M // 2, M // 4, M // 2, M // 3, M]}
+           "twice": lambda M: [0, M // 2, M // 4, M // 2, M // 3, M],
+           # more utterances than a warp looks at in one go, most of them empty: rows in front of the first and
+           # behind the last one's, and one that ends past the matrix
+           "many": lambda M: [M // 4 + min(b // 8, M // 2) for b in range(700)],
+           "many, past": lambda M: [M // 4 + min(b // 8, M // 2) for b in range(700)] + [M + 1],
+           "many, falling": lambda M: [M // 4 + min(b // 8, M // 2) for b in range(700)] + [M // 8, M // 4]}
 
 
 @pytest.mark.parametrize("offsets", sorted(OFFSETS))
