@@ -246,7 +246,11 @@ __device__ __forceinline__ void stream_spans(const DirectParams &p, const Cut cu
             cur.valid = cur.a < deal.rows;
             const int at = deal.first + cur.a * deal.stride;
             if (cur.valid && at >= b_end) {
-                do b_end = act[++cur.b + 1]; while (b_end <= at);
+                b_end = act[++cur.b + 1];
+                if (b_end <= at) {               // not the next one: short drafts
+                    cur.b = stream::utterance_of_count(act, p.B, at);
+                    b_end = act[cur.b + 1];
+                }
                 cur.shift = (int)p.tok_off[cur.b] - act[cur.b];
             }
             cur.row = at + cur.shift;
