@@ -124,6 +124,35 @@ def test_skipped_utterances(cuda_device, B, split):
     assert diff.numel() == 0 or float(diff.max()) <= H.FLOAT_TOL
 
 
+@pytest.mark.parametrize("kernel", [0, 2])
+@pytest.mark.parametrize("B", [31, 32, 33, 64, 65, 97, 128, 129, 511, 512, 513, 1024, 1025, 1537, 2047])
+def test_count_of_rows_to_read(cuda_device, B, kernel):
+    """As many utterances as a warp, a turn and the block count, one fewer and one more, by the direct loads
+    and by the ring: each utterance's own rows are read, and no others."""
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, 4, size=B)
+    lens[[0, -1]] = 3
+    skip = (rng.random(B) < 0.4).astype(np.uint8)
+    skip[[0, -1]] = 0
+    V, M = 40, int(lens.sum())
+    wide, view, ids = _rows(M, V, 0, B)
+    off = _offsets(lens).to(cuda_device)
+    args = (wide.to(cuda_device)[:, :V], off, ids.to(cuda_device), 0.1)
+    plain = ssd.ssd_verify(*args, opts=H.opts(kernel=1))
+    out = ssd.alloc_verify_outputs(M, B, cuda_device, ssd.ssd_verify_workspace_bytes(B, M, V, ssd.BF16))
+    for k in ("token_logp", "row_lse"):
+        out[k].fill_(7.0)
+    ssd.ssd_verify(*args, skip=torch.from_numpy(skip).to(cuda_device), out=out, opts=H.opts(kernel=kernel))
+    torch.cuda.synchronize()
+    read = torch.from_numpy(np.repeat(skip == 0, lens)).to(cuda_device)
+    for k in ("token_logp", "row_lse"):
+        assert float((out[k][read] - plain[k][read]).abs().max()) <= H.FLOAT_TOL, k
+        assert bool((out[k][~read] == 7.0).all()), k
+    was_read = torch.from_numpy(skip == 0).to(cuda_device)
+    assert torch.equal(out["accepted_len"][was_read], plain["accepted_len"][was_read])
+    assert not out["utt_status"].any()
+
+
 def test_malformed_offsets(cuda_device):
     """Offsets that run backwards: flagged, the sound utterances around them unharmed."""
     wide, view, ids = _rows(30, 900, 0, 3)
