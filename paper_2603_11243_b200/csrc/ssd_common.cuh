@@ -399,6 +399,21 @@ __device__ __forceinline__ int load_now(const int32_t *p) {
     return v;
 }
 
+// The value at p, or 0 without a look at it: a predicated load and no branch around it, so that several in a
+// row are one round trip.
+__device__ __forceinline__ int64_t load_if(bool ok, const int64_t *p) {
+    int64_t v;
+    asm volatile("{ .reg .pred q; setp.ne.b32 q, %2, 0; mov.b64 %0, 0; @q ld.global.s64 %0, [%1]; }"
+                 : "=l"(v) : "l"(p), "r"((int)ok) : "memory");
+    return v;
+}
+__device__ __forceinline__ int load_if(bool ok, const uint8_t *p) {
+    int v;
+    asm volatile("{ .reg .pred q; setp.ne.b32 q, %2, 0; mov.b32 %0, 0; @q ld.global.u8 %0, [%1]; }"
+                 : "=r"(v) : "l"(p), "r"((int)ok) : "memory");
+    return v;
+}
+
 struct bf16_t { uint16_t bits; };
 template <> struct Elem<bf16_t> {
     static constexpr int kBytes = 2;

@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     int rows = (int)p.M;
     Cut cut = p.cut[0];
     if (table) {
-        rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, warp_tot, kWarps);
+        rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, warp_tot, kWarps, nullptr);
 #pragma unroll
         for (int q = 1; q < kCuts; ++q)
             if (rows <= (int)(p.M >> q)) cut = p.cut[q];

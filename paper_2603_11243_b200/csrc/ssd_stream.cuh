@@ -201,7 +201,9 @@ __device__ __forceinline__ float row_logp(float x, float Mx, float lnS) {
 // Rows to read before each utterance, in shared memory, for up to 32 * L utterances from b0 on and in
 // front of utterance `end`: act[b] is `total` and the rows of the ones before b, shift[b] (where asked for)
 // what to add to a count of rows to have the row.  Returns the total with them.  Called by all lanes of a
-// warp.  The loads are one round trip, and the L prefix sums go through the warp side by side.
+// warp.  The loads are one round trip, and the L prefix sums go through the warp side by side.  Loops are
+// kept rolled here and below: a CTA runs this once, and what it costs is fetching the instructions (400 bf16
+// rows of 64 KB behind a gate, 8 utterances: 10.4 us unrolled, 10.0 rolled).
 template <int L>
 __device__ __forceinline__ int count_turn(const int64_t *tok_off, const uint8_t *skip, int end, int64_t M, int b0,
                                           int total, int32_t *act, int32_t *shift) {
@@ -210,17 +212,15 @@ __device__ __forceinline__ int count_turn(const int64_t *tok_off, const uint8_t 
     int skipped[L], mine[L], incl[L];
 #pragma unroll
     for (int j = 0; j < L; ++j) {
-        const int b = min(b0 + 32 * j + lane, end - 1);
-        i0[j] = tok_off[b];
-        i1[j] = tok_off[b + 1];
-        skipped[j] = skip[b];
+        const int b = b0 + 32 * j + lane;
+        i0[j] = load_if(b < end, tok_off + b);
+        i1[j] = load_if(b < end, tok_off + b + 1);
+        skipped[j] = load_if(b < end, skip + b);
     }
 #pragma unroll
-    for (int j = 0; j < L; ++j) {
-        const bool read = b0 + 32 * j + lane < end && !(i0[j] < 0 || i1[j] < i0[j] || i1[j] > M || skipped[j]);
-        incl[j] = mine[j] = read ? (int)(i1[j] - i0[j]) : 0;
-    }
-#pragma unroll
+    for (int j = 0; j < L; ++j)
+        incl[j] = mine[j] = i0[j] < 0 || i1[j] < i0[j] || i1[j] > M || skipped[j] ? 0 : (int)(i1[j] - i0[j]);
+#pragma unroll 1
     for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
         for (int j = 0; j < L; ++j) {
@@ -238,66 +238,41 @@ __device__ __forceinline__ int count_turn(const int64_t *tok_off, const uint8_t 
     }
     return total;
 }
-// Rows to read before each utterance (act[B]: their total, which is returned), in shared memory.  Called
-// by all threads of a block of so many warps, a constant; warp_tot has a word per warp.  (With the warps
-// counted at run time, and a thread's utterances one after another, every call behind a gate took 0.1 to
-// 0.3 us longer: 400 bf16 rows of 64 KB, 2 utterances 10.5 us, 10.3 now; 32 utterances 11.05 and 10.75.)
+// Rows to read before each utterance (act[B]: their total, which is returned), in shared memory, and what
+// to add to such a count to have the row (shift, where asked for).  Called by all threads of a block;
+// warp_tot has a word per warp.
 __device__ __forceinline__ int count_rows(const int64_t *tok_off, const uint8_t *skip, int B, int64_t M,
-                                          int32_t *act, int32_t *warp_tot, const int warps) {
+                                          int32_t *act, int32_t *warp_tot, const int warps, int32_t *shift) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int share = 32 * ((B + 32 * warps - 1) / (32 * warps)), b0 = warp * share, end = min(B, b0 + share);
-    int mine = 0, b = b0;                // rows of this warp's utterances
-    for (; b + 64 < end; b += 128) mine = count_turn<4>(tok_off, skip, end, M, b, mine, act, nullptr);
-    for (; b < end; b += 32) mine = count_turn<1>(tok_off, skip, end, M, b, mine, act, nullptr);
+    int mine = 0;                        // rows of this warp's utterances
+    if (b0 < B) {
+        if (share > 32)
+            for (int b = b0; b < end; b += 128) mine = count_turn<4>(tok_off, skip, end, M, b, mine, act, shift);
+        else
+            mine = count_turn<1>(tok_off, skip, end, M, b0, 0, act, shift);
+    }
     if (lane == 0) warp_tot[warp] = mine;
     __syncthreads();
-    int before = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < warps; ++w) {
-        const int t = warp_tot[w];
-        if (w < warp) before += t;
-        total += t;
+    const int each = lane < warps ? warp_tot[lane] : 0;
+    const int before = __reduce_add_sync(0xffffffffu, lane < warp ? each : 0);
+    const int total = __reduce_add_sync(0xffffffffu, each);
+#pragma unroll 1
+    for (int b = b0 + lane; b < end; b += 32) {
+        act[b] += before;
+        if (shift) shift[b] -= before;
     }
-    for (b = b0 + lane; b < end; b += 32) act[b] += before;
     if (threadIdx.x == 0) act[B] = total;
     __syncthreads();
     return total;
 }
-// The same by one warp, for itself, and what to add to such a count to have the row.
+// The same by one warp, for itself, of up to 128 utterances; with `rehearse` it reads and counts nothing.
 __device__ __forceinline__ int count_rows_by_warp(const int64_t *tok_off, const uint8_t *skip, int B, int64_t M,
-                                                  int32_t *act, int32_t *shift) {
-    constexpr int L = 4;                 // utterances a lane has in flight
-    const int lane = threadIdx.x & 31;
-    int total = 0;
-    for (int b0 = 0; b0 < B; b0 += 32 * L) {
-        int64_t i0[L], i1[L];
-        int skipped[L];
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            const int b = min(b0 + 32 * j + lane, B - 1);
-            i0[j] = tok_off[b];
-            i1[j] = tok_off[b + 1];
-            skipped[j] = skip[b];
-        }
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            const int b = b0 + 32 * j + lane;
-            const bool read = b < B && !skipped[j] && i0[j] >= 0 && i1[j] >= i0[j] && i1[j] <= M;
-            const int mine = read ? (int)(i1[j] - i0[j]) : 0;
-            int incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (b < B) {
-                act[b] = total + incl - mine;
-                shift[b] = (int)i0[j] - (total + incl - mine);
-            }
-            total += __shfl_sync(0xffffffffu, incl, 31);
-        }
-    }
-    if (lane == 0) act[B] = total;
+                                                  int32_t *act, int32_t *shift, bool rehearse) {
+    const int end = rehearse ? 0 : B;
+    const int total = B > 32 ? count_turn<4>(tok_off, skip, end, M, 0, 0, act, shift)
+                             : count_turn<1>(tok_off, skip, end, M, 0, 0, act, shift);
+    if ((threadIdx.x & 31) == 0) act[B] = total;
     __syncwarp();
     return total;
 }

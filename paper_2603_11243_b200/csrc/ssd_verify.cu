@@ -56,6 +56,12 @@ struct VerifyParams {
     unsigned long long epoch;
 };
 
+// Up to so many utterances the ring's producing warp counts by itself, after a rehearsal while the kernel
+// before still runs; beyond, all warps do (one warp's 128 at a time were a round trip each: 2,000 rows of 98
+// KB, none skipped, of 500 utterances 44.3 us, of 2,000 67.5; 43.1 and 58.9 now; of 56 38.3 and 37.8).
+// All warps through a rehearsal: 0.5 us less where rows are read, but 2 us more where all are skipped.
+constexpr int kCountedByWarp = 128;
+
 template <typename T, int kF, bool kArg>
 __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -84,20 +90,31 @@ __global__ void __launch_bounds__(544, 1) verify_rows_tma(const VerifyParams p) 
         mbar_init_fence();
     }
     __syncthreads();             // the barriers are there
-    pdl_wait();
-    if (!kArg) pdl_launch_dependents();
+    int to_read = 0;
+    if (table && p.B <= kCountedByWarp && warp == 0) {
+#pragma unroll 1
+        for (int real = 0; real < 2; ++real) {
+            if (real) {
+                pdl_wait();
+                if (!kArg) pdl_launch_dependents();
+            }
+            to_read = count_rows_by_warp(p.tok_off, p.skip, p.B, p.M, act, shift, !real);
+        }
+    } else {
+        pdl_wait();
+        if (!kArg) pdl_launch_dependents();
+        if (table && p.B > kCountedByWarp)     // (the stages are empty yet: the warps' counts pass through the first)
+            to_read = count_rows(p.tok_off, p.skip, p.B, p.M, act, reinterpret_cast<int32_t *>(stage0_ptr),
+                                 blockDim.x >> 5, shift);
+    }
 
     const int64_t row_bytes = (int64_t)p.V * ES;
-
     if (warp == 0) {
         // =============================== producer ===============================
         // With skip flags only rows that are read are dealt out (with more utterances or rows than
         // the table takes, skipped ones are passed over instead): a batch of which nothing is read
-        // costs a CTA its look at the flags, by this warp alone.  (56 utterances, 20,000 rows of 98
-        // KB, none read: the call 5.8 us with every row looked up, 3.5 with a count by the whole
-        // block; but 50 rows of 128 KB 6.4 and 7.2.)
-        int64_t num_items = p.num_items;
-        if (table) num_items = (int64_t)count_rows_by_warp(p.tok_off, p.skip, p.B, p.M, act, shift) * p.split;
+        // costs a CTA its look at the flags.
+        const int64_t num_items = table ? (int64_t)to_read * p.split : p.num_items;
         int s = 0;                  // stage to fill next, and the phase of its barriers
         uint32_t ph = 0;
         bool failed = false;
