@@ -422,6 +422,10 @@ inline bool table_fits(int B, int64_t M) {
 // three blocks' worth of instructions of its own (reference, merge, the next span's addresses).
 // (A finer cut of the rows that do not fill a round, so that every warp gets the same bytes, was
 // slower throughout: 22.4 against 21.1 us on 250 rows of 304 KB, 95 against 93.5 on 5,568 of 98.)
+// Spans that all begin at one offset of 64 KB keep the warps, which go through them in step, on the same
+// few memory channels: they count an eighth more (fp32 behind a gate, us, by spans of 64 KB, of 32 and by the
+// ring: 1,500 rows of 192 KB 56.5, 48.2, 49.6; 750 of 384 KB 56.4, 48.3, 51.8; 1,500 of 195 KB do not
+// mind: 49.6, 49.7, 50.6).
 inline Cut plan_spans(int64_t M, int64_t row_bytes, int warps, int most) {
     const int64_t nb = row_blocks(row_bytes);
     int64_t best = 0;
@@ -431,27 +435,29 @@ inline Cut plan_spans(int64_t M, int64_t row_bytes, int warps, int most) {
         ns = ns < 1 ? 1 : ns > most ? most : ns;
         const int64_t bps = (nb + ns - 1) / ns;
         ns = (nb + bps - 1) / bps;
-        const int64_t cost = (M * ns + warps - 1) / warps * (bps + 3);
+        int64_t cost = (M * ns + warps - 1) / warps * (bps + 3);
+        if (bps % 64 == 0 && row_bytes % 65536 == 0) cost += cost / 8;
         if (best == 0 || cost < best) { best = cost; cut = Cut{(int)ns, (int)bps}; }
         if (M > 0 && (int64_t)rounds * warps / M >= most) break;
     }
     return cut;
 }
 
-// With `skip` only the kernel knows how many rows are read, and the cut for all of a large batch's rows
-// leaves most warps without one where few are.  So such a batch (a row per warp and more) has a cut
-// for every halving of its rows, of up to eight spans, and the kernel takes the one for what its table
-// counted.  One cut, cuts, and the ring for comparison, us: 43,000 rows of 200 KB of which 330 are
-// read 58.5, 21.1, 22.4; 46,000 of 304 KB, 990: 117, 66.7, 72.0; 30,000 of 98 KB, 2,800: 62.4, 50.4,
-// 53.0; all 43,000: 1,276, 1,270, 1,361.  (pairs > spans of a cut only here: at most sixteen, a lane
-// each.)
-constexpr int kMostSpansSkipping = 8;
+// With `skip` only the kernel knows how many rows are read, and the cut for all of a batch's rows leaves
+// most warps without a span where few are.  So such a batch has a cut for every halving of its rows, and
+// the kernel takes the one for what its table counted.  One cut, cuts, and the ring for comparison,
+// us: bf16, 43,000 rows of 200 KB of which 330 are read 58.5, 21.1, 22.4; 46,000 of 304 KB, 990: 117, 66.7,
+// 72.0; 30,000 of 98 KB, 2,800: 62.4, 50.4, 53.0; all 43,000: 1,276, 1,270, 1,361; fp32, 500 of 608 KB, 50:
+// 24.9, 15.0, 20.0; 590 of 400 KB, 60: 19.0, 10.6, 14.5.  The finer cuts have up to eight spans, which the
+// closing kernel takes in a lane or two; calls of few rows, whose cut for all of them has more, up to 32.
+// (pairs > spans of a cut only here.)
 inline void plan_cuts(int64_t M, int64_t row_bytes, int warps, int most, bool may_skip, Cut *cut, int *pairs) {
     cut[0] = plan_spans(M, row_bytes, warps, most);
     *pairs = cut[0].spans;
-    const int fine = most < kMostSpansSkipping ? most : kMostSpansSkipping;
+    const int finest = 8 * M < warps ? 32 : 8, fine = most < finest ? most : finest;
     for (int k = 1; k < kCuts; ++k) {
-        cut[k] = may_skip && M >= warps ? plan_spans(M >> k, row_bytes, warps, fine) : cut[0];
+        cut[k] = may_skip ? plan_spans(M >> k, row_bytes, warps, fine) : cut[0];
+        if (M < warps && cut[k].spans < cut[k - 1].spans) cut[k] = cut[k - 1];     // fewer by `fine` alone
         if (cut[k].spans > *pairs) *pairs = cut[k].spans;
     }
 }

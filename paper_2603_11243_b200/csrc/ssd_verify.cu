@@ -869,13 +869,14 @@ unsigned long long next_epoch();
 //     98 KB: 31.9 / 33.7; 8,000: 136 / 141), direct beyond (12,000: 200 / 200; 16,000: 265 / 245;
 //     22,000 of 200 KB: 708 / 664): it spends a fifth fewer instructions on a logit.  With `skip`
 //     half of the rows are taken to be read (a batch of 1.3 GB, partly gated: 199 / 206).
-//   fp32, up to 400 MB: direct (50 rows of 240 KB 11.7 / 9.0, 100 15.3 / 11.6; 250 of 128 KB 13.8 / 11.7,
-//     600 19.8 / 18.0, 1,500 35.9 / 35.1; 600 of 608 KB 63.6 / 58.6; 3,000 of 128 KB 63.1 / 62.1): the ring
-//     cuts few rows into spans of 32 KB and hands each over.  Beyond: the ring (6,000 of 128 KB 117.0 /
-//     118.3, 6,000 of 240 KB 208.8 / 213.0, 16,000 of 192 KB 437 / 455), which has more bytes in flight and
-//     half the logits per byte.  That is with skip flags, as behind a gate; without, the ring throughout,
-//     which is what ssd_verify_read_span replays for fp32.  The greedy step on few rows: direct (200 of
-//     196 KB: 14.0 / 12.3; 300 of 608 KB: 36.4 / 35.8; 500 of 196 KB: 21.9 / 23.3)
+//   fp32 with skip flags, as behind a gate, up to 400 MB: direct, all rows read, half and a tenth of them (50
+//     of 304 KB 10.1 / 8.3, 8.1, 6.0; 300 of 192 KB 16.7 / 14.5, 13.4 / 12.0, 9.9 / 8.7; 590 of 608 KB 57.6 /
+//     57.7, 39.8 / 37.6, 20.6 / 15.9; 2,000 of 128 KB 45.2 / 44.2, 29.1 / 28.1, 12.9 / 11.6): the ring cuts few
+//     rows into spans of 32 KB and hands each over.  Of 64 sizes from 120 to 400 MB the ring is 4 % slower
+//     in the mean, and the better one on some (all of 2,300 of 125 KB 50.3 / 51.6 to 53.5).
+//   fp32 without skip flags: the ring (6,000 of 128 KB 117.0 / 118.3, 6,000 of 240 KB 208.8 / 213.0, 16,000 of
+//     192 KB 437 / 455), which has more bytes in flight and half the logits per byte; the greedy step
+//     on few rows: direct (200 of 196 KB: 14.0 / 12.3; 300 of 608 KB: 36.4 / 35.8; 500 of 196 KB: 21.9 / 23.3)
 // The greedy step on bf16 rows: direct (1,024 of 304 KB: 59.5 / 55.1; 24 of 98 KB: 14.0 / 12.6).
 static int use_direct(int64_t M, int64_t row_bytes, ssd_dtype dtype, int kernel, int sms,
                       const ssd_launch_opts *o, const RowsAt &at) {

@@ -236,3 +236,40 @@ def test_shares_of_a_large_batch(cuda_device, B, V, col0):
         was_read = torch.from_numpy(skip == 0).to(dev)
         assert torch.equal(out["accepted_len"][was_read], plain["accepted_len"][was_read]), target
         assert not out["utt_status"].any()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("M,V", [(33, 40003), (300, 40003), (591, 20011), (593, 20011), (1500, 16384), (5000, 700)])
+def test_shares_of_a_small_batch(cuda_device, M, V, dtype):
+    """Fewer rows than warps (and, at the end, a few more) of both types, all to none of them read, at the counts
+    where the kernel changes its cut: more spans a row than the cut for all rows has."""
+    dev, B = cuda_device, min(M, 120)
+    code = ssd.F32 if dtype == torch.float32 else ssd.BF16
+    g = torch.Generator(device=dev).manual_seed(M)
+    wide = torch.randn((M, V + 3), generator=g, device=dev).to(dtype)
+    x = wide[:, 1:1 + V]
+    ids = torch.randint(0, V, (M,), generator=g, device=dev, dtype=torch.int32)
+    rng = np.random.default_rng(M)
+    cuts = np.sort(rng.choice(np.arange(1, M), size=B - 1, replace=False)) if B < M else np.arange(1, M)
+    off = torch.tensor(np.concatenate([[0], cuts, [M]]), dtype=torch.int64)
+    lens = np.diff(off.numpy())
+    plain = ssd.ssd_verify(x, off.to(dev), ids, 0.1, opts=H.opts(kernel=1))
+    for target in sorted({M} | {(M >> k) + d for k in range(1, 7) for d in (0, 1)}):
+        skip, left = np.ones(B, np.uint8), target
+        for b in rng.permutation(B):
+            if lens[b] <= left:
+                skip[b], left = 0, left - lens[b]
+        out = ssd.alloc_verify_outputs(M, B, dev, ssd.ssd_verify_workspace_bytes(B, M, V, code))
+        for t in (out["token_logp"], out["row_lse"]):
+            t.fill_(7.0)
+        out["workspace"].fill_(0xff)                     # pairs that nobody writes would be NaN
+        ssd.ssd_verify(x, off.to(dev), ids, 0.1, skip=torch.from_numpy(skip).to(dev), out=out)
+        torch.cuda.synchronize()
+        read = torch.from_numpy(np.repeat(skip == 0, lens)).to(dev)
+        for k in ("token_logp", "row_lse"):
+            d = (out[k][read] - plain[k][read]).abs()
+            assert d.numel() == 0 or float(d.max()) <= H.FLOAT_TOL, (k, target)
+            assert bool((out[k][~read] == 7.0).all()), (k, target)
+        was_read = torch.from_numpy(skip == 0).to(dev)
+        assert torch.equal(out["accepted_len"][was_read], plain["accepted_len"][was_read]), target
+        assert not out["utt_status"].any()
