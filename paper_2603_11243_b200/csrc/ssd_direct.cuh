@@ -354,9 +354,7 @@ __device__ __forceinline__ void stream_spans(const DirectParams &p, const Cut cu
             add(u, last);
             Sw = warp_sum(total + ((Sa.x + Sa.y) + (Sb.x + Sb.y) + ex2(fmaf(my_edge, kLog2e, ref.nmh))));
             fast = Sw < kSpanSumLimit;
-            // every exponent carried m*log2e + nmh; with the arg max the reference's own is then exactly 1
-            const float carried = fmaf(ref.m, kLog2e, ref.nmh);
-            if (kArg) Sw /= ex2(carried); else Sw *= ex2(-carried);
+            Sw *= ex2(-fmaf(ref.m, kLog2e, ref.nmh));   // every exponent carried m*log2e + nmh
         }
         SpanResult out;
         if (fast) {
@@ -386,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
     extern __shared__ int32_t act[];
     __shared__ int32_t warp_tot[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool table = p.table != 0;
+    const bool table = !kArg && p.table != 0;      // a greedy step reads all rows
     pdl_wait();
     pdl_launch_dependents();
     int rows = (int)p.M;
@@ -398,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) verify_rows_direct(const
             if (rows <= (int)(p.M >> q)) cut = p.cut[q];
     }
     // counted so that neighbours go to different CTAs
-    const Deal deal{blockIdx.x + gridDim.x * warp, gridDim.x * kWarps, rows, 0, 1, table, p.skip == nullptr};
+    const Deal deal{blockIdx.x + gridDim.x * warp, gridDim.x * kWarps, rows, 0, 1, table, kArg || p.skip == nullptr};
     stream_spans<T, kF, kArg, 0>(p, cut, deal, act, [] {}, [&](int row, int, int sp, const SpanResult &out) {
         if (kArg) {
             if (lane == 0) reinterpret_cast<float4 *>(p.partials)[(int64_t)row * p.pairs + sp] =

@@ -344,16 +344,18 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
     vm = warp_max(vm);
     // Sums are taken relative to the largest logit, and its own exponential is taken out of the one partial
     // that holds it: what is left beside it is all that the logarithm of a confident row is about.  It is
-    // taken in the form that the partial has it, with one rounding: 1 where the logit is the partial's
-    // reference, a quotient that both carry what rounding left out of x * log2e above a reference of the
-    // fast pass (below 4,096), and a power of the difference elsewhere (1e10 * log2e is rounded by 440:
-    // neither part of the quotient is in fp32's range).
+    // taken in the form that the partial has it: below 4,096 the exponents of both carry what rounding left
+    // out of the reference's product with log2e, which the direct loads (kUnit) take out by a product and
+    // the ring by a quotient; from there on the direct loads hold differences, and in the ring's quotient the
+    // reference itself is 1 (1e10 * log2e is rounded by 440: no such factor is in fp32's range).
     const bool plain = vm > kNegInit;
     const float base = plain ? vm : Mx;
     int vi = INT_MAX;
+    float ref = 0.f;                  // of the first partial of this lane that has the largest logit
     each([&](const float4 &v) {
-        if (v.z == vm) vi = min(vi, __float_as_int(v.w));
+        if (v.z == vm && __float_as_int(v.w) < vi) { vi = __float_as_int(v.w); ref = v.x; }
     });
+    const int mine = vi;
     vi = __reduce_min_sync(0xffffffffu, vi);
     const int found = vi;
     float beside = -INFINITY;
@@ -361,15 +363,17 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
         const int64_t e = (int64_t)vi + lane;
         if (lane < 32 / Elem<T>::kBytes && e < V) beside = Elem<T>::load(row + e * Elem<T>::kBytes);
     }
+    float own = 0.f;                  // in one lane, each partial having its own indexes; once, not for each held
+    if (plain && mine == found) {
+        const float nmh = -(ref * kLog2e), up = ex2(fmaf(vm, kLog2e, nmh)), carried = fmaf(ref, kLog2e, nmh);
+        if (!(fabsf(ref) < 4096.f)) own = ex2((vm - ref) * kLog2e);
+        else if (kUnit) own = up * ex2(-carried);
+        else own = up / ex2(carried);
+    }
     float S = 0.f;
     each([&](const float4 &v) {
-        float sum = v.y;
-        if (plain && v.z == vm && __float_as_int(v.w) == found) {     // one partial: each has its own indexes
-            const float nmh = -(v.x * kLog2e);
-            sum -= fabsf(v.x) < 4096.f ? ex2(fmaf(vm, kLog2e, nmh)) / ex2(fmaf(v.x, kLog2e, nmh))
-                                       : ex2((vm - v.x) * kLog2e);
-        }
-        S += sum * ex2((v.x - base) * kLog2e);
+        const bool holds = v.z == vm && __float_as_int(v.w) == found;
+        S += (v.y - (holds ? own : 0.f)) * ex2((v.x - base) * kLog2e);
     });
     S = warp_sum(S);
     if (kUnit) {

@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kThreads, direct::kCtasPerSm) rows_whole(const
     // A malformed list of offsets may name rows more than once, more of them than this CTA's shared
     // memory is laid out for: then every row is read once and asked for its owner (look_up).
     int rows = (int)p.M;
-    if (p.table) rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, warp_tot, kWarps, nullptr);
-    const bool table = p.table && rows <= (int)p.M;
+    if (!kArg && p.table) rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, warp_tot, kWarps, nullptr);
+    const bool table = !kArg && p.table && rows <= (int)p.M;
     if (!table) rows = (int)p.M;
     const int here = cl < rows ? (rows - cl + nc - 1) / nc : 0;
     cluster_wait();          // all CTAs of the cluster run: their shared memory may be written
