@@ -332,6 +332,7 @@ __device__ __forceinline__ GreedyRow greedy_row(Get get, int P, const char *row,
 #pragma unroll
             for (int j = 0; j < L; ++j) look(held[j]);
         } else {
+#pragma unroll 1
             for (int q = lane; q < P; q += 32) look(get(q));
         }
     };
