@@ -889,13 +889,24 @@ static int64_t lanes_for(ssd_dtype dtype, int V, int64_t rows, int64_t warps, in
 //     and the tiles' few lanes per row spend fewer of them on what is done once per row
 //   fp32, half the logits per byte: 9,600 rows of 4 KB 15.4 / 11.3, 130,000 of 516 bytes (66 MB) 24.7 /
 //     19.0, 30,000 of 4 KB (122 MB) 25.6 / 24.9, 50,000 37.3 / 37.2, 130,000 81.8 / 84.5
+// bf16 rows of which the warps need a second round (by more than a tenth) stay with the tiles where those come
+// in one, nine tenths full at most: 24,000 rows of 400 bytes 10.1 / 11.3, 13,000 of 1.2 KB 10.8 / 11.4,
+// 12,000 of 2 KB 13.0 / 13.7, 7,500 of 2.7 KB 11.1 / 11.7, 7,500 of 3.3 KB 12.2 / 13.6, 5,500 of 4 KB 11.8 /
+// 12.8; not rows of one unit a lane, or of three of which eight ninths are there (22,000 of 256 bytes 11.0 /
+// 9.8; 11,500 of 1.4 KB 11.9 / 11.2; 5,300 of 3 KB 11.2 / 10.8).
 static void plan_direct(ssd_dtype dtype, int V, int64_t N, const ssd_launch_opts *o, CtcPlan *pl) {
     if (o && (o->kernel || o->split || o->stages || o->stage_bytes || o->fma_exp)) return;
     const int es = dtype == SSD_F32 ? 4 : 2;
     const int64_t sms = device_sm_count(), row_bytes = (int64_t)V * es;
     if (sms <= 0 || N < 1 || row_bytes / 32 > 32 * ctc::kMostUnits) return;
     if (N > (dtype == SSD_F32 ? 200ll << 20 : 40ll << 20) / row_bytes) return;
-    pl->direct = lanes_for(dtype, V, N, sms * direct::kCtasPerSm * direct::kWarps, &pl->d_lanes, &pl->d_units) != 0;
+    const int64_t warps = sms * direct::kCtasPerSm * direct::kWarps;
+    if (lanes_for(dtype, V, N, warps, &pl->d_lanes, &pl->d_units) == 0) return;
+    const int64_t passes = (N * pl->d_lanes + 31) / 32, last = passes % warps;
+    const bool second_round = passes > warps && last * 10 > warps;
+    const bool one_of_tiles = pl->kernel == 2 && pl->num_tiles * 10 <= pl->warps * sms * 9;
+    const bool spare = pl->d_units == 3 ? row_bytes / 32 * 9 < pl->d_lanes * 3 * 8 : pl->d_units > 1;
+    pl->direct = !(dtype == SSD_BF16 && second_round && one_of_tiles && spare);
 }
 
 // Kernel and launch shape of the frame-statistics pass for these sizes.

@@ -103,3 +103,20 @@ def test_rows_of_large_finite_logits(cuda_device, times, V, dtype):
     assert np.abs(out["frame_entropy"].cpu().numpy() - entropy).max() <= H.FLOAT_TOL
     d = np.abs(out["frame_lse"].cpu().numpy().astype(np.float64) - orc["frame_lse"])
     assert (d <= H.FLOAT_TOL + 2.0 ** -23 * np.abs(orc["frame_lse"])).all()
+
+
+@pytest.mark.parametrize("N,V,direct", [(4736, 2047, 1), (5500, 2047, 0), (24000, 200, 0), (44000, 128, 1),
+                                        (11500, 700, 1), (13000, 600, 0), (15000, 1025, 1)])
+def test_rounds_of_either_kernel(cuda_device, N, V, direct):
+    """bf16 rows that registers would need a second round for and tiles would not, and sizes beside them: the
+    kernel that is meant runs, and agrees with the plain loads."""
+    direct = direct if torch.cuda.get_device_properties(0).multi_processor_count == 148 else None
+    x = torch.randn((N, V), generator=torch.Generator(device=cuda_device).manual_seed(N), device=cuda_device).bfloat16()
+    off = torch.tensor([0, N // 3, N], device=cuda_device)
+    span = ssd.ssd_ctc_draft_read_span(x.data_ptr(), ssd.BF16, V, V, N)
+    assert span.faults == 0 and direct in (None, span.direct)
+    a, b = ssd.ssd_ctc_draft(x, off, 0, 50), ssd.ssd_ctc_draft(x, off, 0, 50, opts=H.opts(kernel=1))
+    torch.cuda.synchronize()
+    assert torch.equal(a["frame_argmax"], b["frame_argmax"]) and torch.equal(a["draft_len"], b["draft_len"])
+    for k in ("frame_entropy", "frame_lse"):
+        assert float((a[k] - b[k]).abs().max()) <= H.FLOAT_TOL, k
