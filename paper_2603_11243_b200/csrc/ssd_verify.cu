@@ -891,35 +891,40 @@ static int use_direct(int64_t M, int64_t row_bytes, ssd_dtype dtype, int kernel,
 // How rows are dealt to clusters that close them (rows_whole): column spans, cluster size and number
 // of clusters with the fewest block steps of a warp, counted as plan_spans counts them; that number,
 // or 0 where a CTA's pairs do not fit.
+// (Every call searches: in 32 bits, since rows and row_bytes are below 2^30, and no further than more rounds
+// cut finer.  With 64-bit divisions throughout, 1.1 us of host time a call; now 0.2 to 0.6.)
 static int64_t plan_whole(int64_t M, int64_t row_bytes, int sms, const RowsAt &at, int B, VerifyPlan *pl) {
     constexpr size_t kMostSmem = 12 * 1024;      // little enough for the L1-heavy split
-    const int64_t nb = direct::row_blocks(row_bytes);
+    constexpr uint32_t kMostSpans = 128;
+    const uint32_t nb = (uint32_t)direct::row_blocks(row_bytes), rows = (uint32_t)M;
     const size_t pair = at.greedy ? sizeof(float4) : sizeof(float2), draft = at.greedy ? 0 : sizeof(float2);
-    int64_t best = 0;
+    uint64_t best = 0;
     for (int clog = 0; clog <= 3; ++clog) {
-        const int C = 1 << clog, W = C * direct::kWarps;
+        const uint32_t C = 1u << clog, W = C * direct::kWarps;
         // clusters of four and eight CTAs do not fill the GPU's clusters of SMs: 71 of 74 and 33 of 37
         // run at a time, and one more waits for the longest of those (300 rows of 98 KB on 35 clusters
         // of eight: 13.9 us; on 32, 10.0)
-        const int64_t most = (int64_t)direct::kCtasPerSm * sms / C * (clog == 3 ? 22 : clog == 2 ? 24 : 25) / 25;
-        const int64_t nc = M < most ? M : most > 0 ? most : 1;
-        const int64_t q = (M + nc - 1) / nc;
-        for (int rounds = 1; rounds <= 16; ++rounds) {
-            int64_t ns = (int64_t)rounds * W / q;
-            ns = ns < 1 ? 1 : ns > 128 ? 128 : ns;
-            const int64_t bps = (nb + ns - 1) / ns;
+        const uint32_t most = (uint32_t)direct::kCtasPerSm * sms / C * (clog == 3 ? 22 : clog == 2 ? 24 : 25) / 25;
+        const uint32_t nc = rows < most ? rows : most > 0 ? most : 1;
+        const uint32_t q = (rows + nc - 1) / nc;
+        for (uint32_t rounds = 1; rounds <= 16; ++rounds) {
+            const uint32_t share = rounds * W / q;
+            uint32_t ns = share < 1 ? 1 : share > kMostSpans ? kMostSpans : share;
+            const uint32_t bps = (nb + ns - 1) / ns;
             ns = (nb + bps - 1) / bps;
             const size_t smem = (size_t)((q + C - 1) / C) * (ns * pair + draft) + (at.skip ? (size_t)(B + 1) * 4 : 0);
-            const int64_t cost = (q * ns + W - 1) / W * (bps + 3);
-            if (smem > kMostSmem || (best != 0 && cost >= best)) continue;
-            best = cost;
-            pl->whole_cut = direct::Cut{(int)ns, (int)bps};
-            pl->whole_cluster_log2 = clog;
-            pl->whole_clusters = (int)nc;
-            pl->whole_smem_bytes = smem;
+            const uint64_t cost = ((uint64_t)q * ns + W - 1) / W * (bps + 3);
+            if (smem <= kMostSmem && (best == 0 || cost < best)) {
+                best = cost;
+                pl->whole_cut = direct::Cut{(int)ns, (int)bps};
+                pl->whole_cluster_log2 = clog;
+                pl->whole_clusters = (int)nc;
+                pl->whole_smem_bytes = smem;
+            }
+            if (share >= kMostSpans || bps == 1) break;
         }
     }
-    return best;
+    return (int64_t)best;
 }
 
 // Whether the rows of a greedy step or a shard are closed by the clusters that read them.  Measured,
