@@ -363,6 +363,14 @@ def test_frame_statistics_kernels_agree_under_random_options(cuda_device, seed):
 
 
 @pytest.mark.parametrize("seed", range(40))
+def test_frame_statistics_kernels_agree_under_random_options_through_the_tiles(cuda_device, seed, monkeypatch):
+    """The same by bulk-copy tiles, which short rows take only where they are asked for."""
+    make = H.opts
+    monkeypatch.setattr(H, "opts", lambda **kw: make(**{"kernel": 2, **kw}))
+    test_frame_statistics_kernels_agree_under_random_options(cuda_device, seed)
+
+
+@pytest.mark.parametrize("seed", range(40))
 def test_verify_kernels_agree_under_random_options(cuda_device, seed):
     """ssd_verify's bulk-copy kernel under random launch options (grid, warps, column spans, ring
     shape, exponential split, where rows are finished) against the plain-load kernel, on new

@@ -365,6 +365,15 @@ def test_workspace_left_dirty_by_anything(cuda_device):
             assert n > 0
 
 
+def test_tile_counter_left_dirty_by_anything(cuda_device, monkeypatch):
+    """The same by the bulk-copy tiles, which claim from the counter: short rows are read into registers
+    unless the tiles are asked for."""
+    make, call = H.opts, ssd.ssd_ctc_draft
+    monkeypatch.setattr(H, "opts", lambda **kw: make(**{"kernel": 2, **kw}))
+    monkeypatch.setattr(ssd, "ssd_ctc_draft", lambda *a, **kw: call(*a, **{"opts": H.opts(), **kw}))
+    test_workspace_left_dirty_by_anything(cuda_device)
+
+
 def test_internal_error_marks_never_pass_the_gate(cuda_device):
     """The value a kernel leaves in a frame's entropy when one of its bounded waits ran out
     (a NaN with a fixed payload) makes the gate refuse the utterance and report
