@@ -870,7 +870,7 @@ unsigned long long next_epoch();
 //     22,000 of 200 KB: 708 / 664): it spends a fifth fewer instructions on a logit.  With `skip`
 //     half of the rows are taken to be read (a batch of 1.3 GB, partly gated: 199 / 206).
 //   fp32 with skip flags, as behind a gate, up to 400 MB: direct, all rows read, half and a tenth of them (50
-//     of 304 KB 10.1 / 8.3, 8.1, 6.0; 300 of 192 KB 16.7 / 14.5, 13.4 / 12.0, 9.9 / 8.7; 590 of 608 KB 57.6 /
+//     of 392 KB, all, 11.7 / 8.8; 300 of 192 KB 16.7 / 14.5, 13.4 / 12.0, 9.9 / 8.7; 590 of 608 KB 57.6 /
 //     57.7, 39.8 / 37.6, 20.6 / 15.9; 2,000 of 128 KB 45.2 / 44.2, 29.1 / 28.1, 12.9 / 11.6): the ring cuts few
 //     rows into spans of 32 KB and hands each over.  Of 64 sizes from 120 to 400 MB the ring is 4 % slower
 //     in the mean, and the better one on some (all of 2,300 of 125 KB 50.3 / 51.6 to 53.5).
@@ -940,9 +940,12 @@ static int64_t plan_whole(int64_t M, int64_t row_bytes, int sms, const RowsAt &a
 //     KB 23.5 / 20.5; 12,000 of 152 KB 260 / 268: long rows of long batches stay with the ring, as
 //     in use_direct, where rows start on 16-byte boundaries (12,000 of 64,004 bytes 138 / 113)
 // Whole rows do not always come out even over the clusters.  Where that takes clusters of four and
-// more in more than a few rows each, or a third more steps, the pair kernel's finer deal is better
-// (600 rows of 32 KB 7.7 / 8.7; the greedy step on 74 of 304 KB 9.3 / 9.9).  With skip flags on a
-// row per warp and more only the kernel knows how many are read, and plan_cuts has cuts for that.
+// more in more than a few rows each, or a third more steps, the pair kernel's finer deal is better (600
+// rows of 32 KB 7.7 / 8.7; the greedy step on 74 of 304 KB 9.3 / 9.9); for the greedy step also where the
+// steps are more than the second launch is worth (1,500 rows of 98 KB 27.6 / 28.7 and of 304 KB 73.1 / 75.0, 1,800
+// of 304 KB 86.1 / 87.7; but a shard's 3,000 rows of 24 KB 16.6 / 15.8).
+// With skip flags on a row per warp and more only the kernel knows how many are read, and plan_cuts has
+// cuts for that.
 static int use_whole(int B, int64_t M, int64_t row_bytes, ssd_dtype dtype, int sms, const ssd_launch_opts *o,
                      const RowsAt &at, VerifyPlan *pl) {
     if (!(at.greedy || at.shard) || M == 0 || pl->kernel != 2 || row_bytes >= (1ll << 30) || M >= (1ll << 30)) return 0;
@@ -959,7 +962,8 @@ static int use_whole(int B, int64_t M, int64_t row_bytes, ssd_dtype dtype, int s
     if (dtype == SSD_F32) return 1;
     const direct::Cut c = direct::plan_spans(M, row_bytes, warps, 64);
     const int64_t pairs = (M * c.spans + warps - 1) / warps * (c.blocks + 3);
-    return pl->whole_cluster_log2 >= 2 ? cost <= pairs + 1 && M <= 8ll * pl->whole_clusters : 3 * cost <= 4 * pairs + 3;
+    if (pl->whole_cluster_log2 >= 2) return cost <= pairs + 1 && M <= 8ll * pl->whole_clusters;
+    return 3 * cost <= 4 * pairs + 3 && (at.shard || cost <= pairs + 6);
 }
 
 // Workspace: [0,256) header (error word, finished-CTA counter), two words per utterance, then
