@@ -1114,8 +1114,11 @@ static int launch_whole(const void *logits, ssd_dtype dtype, int V, int64_t ld, 
     e.cluster_log2 = plan.whole_cluster_log2;
     e.V = V;
     constexpr int kF = kEnd == whole::kGreedy ? 0 : 1;       // as in launch_direct
-    void (*kern)(const direct::DirectParams, const whole::EndParams) = whole::rows_whole<bf16_t, kF, kEnd>;
-    if (dtype == SSD_F32) kern = whole::rows_whole<float, 0, kEnd>;
+    void (*kern)(const direct::DirectParams, const whole::EndParams) = whole::rows_whole<bf16_t, kF, kEnd, false>;
+    if (dtype == SSD_F32) kern = whole::rows_whole<float, 0, kEnd, false>;
+    if constexpr (kEnd == whole::kShard) {
+        if (skip) kern = dtype == SSD_F32 ? whole::rows_whole<float, 0, kEnd, true> : whole::rows_whole<bf16_t, kF, kEnd, true>;
+    }
     const unsigned cluster = 1u << plan.whole_cluster_log2;
     cudaError_t err = cudaSuccess;
     if (o && o->ev_begin) err = cudaEventRecord(static_cast<cudaEvent_t>(o->ev_begin), L.stream);

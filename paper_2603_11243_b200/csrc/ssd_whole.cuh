@@ -43,9 +43,26 @@ struct EndParams {
     float *stats;
 };
 
+__device__ __forceinline__ bool owns(const int64_t *tok_off, const uint8_t *skip, int64_t M, int b, int row) {
+    const int64_t i0 = tok_off[b], i1 = tok_off[b + 1];
+    return ranges::rows_sound(i0, i1, M) && i0 <= row && row < i1 && !(skip && skip[b]);
+}
+// Whether an utterance that the search does not find has the row.  Asking every utterance for each row that
+// none has -- behind the last one's rows, or in front of the first one's -- took 174 us for 4,000 rows of 8 KB
+// of which 2,000 utterances have half (15 now; 20 with a closing kernel): only where the offsets fall
+// somewhere.  Called by all lanes of a warp; out of line, away from what every row needs.
+template <typename T, bool kSkip>
+__device__ __noinline__ bool owned_elsewhere(const int64_t *tok_off, const uint8_t *skip, int B, int64_t M, int row) {
+    bool owned = false;
+    if (!stream::offsets_ordered(tok_off, B))
+        for (int b = 0; !owned && b < B; ++b) owned = owns(tok_off, skip, M, b, row);
+    return owned;
+}
+
 // Shared memory: the pairs of the rows this CTA closes, their drafts, and (with skip flags) the rows
 // to read before each utterance.
-template <typename T, int kF, int kEnd>
+// (kSkip: a call with skip flags.  Without, the code for them in the same kernel cost a shard 1 % and more.)
+template <typename T, int kF, int kEnd, bool kSkip>
 __global__ void __launch_bounds__(kThreads, direct::kCtasPerSm) rows_whole(const DirectParams p, const EndParams e) {
     constexpr bool kArg = kEnd == kGreedy;
     constexpr int ES = Elem<T>::kBytes;
@@ -66,8 +83,8 @@ __global__ void __launch_bounds__(kThreads, direct::kCtasPerSm) rows_whole(const
     // A malformed list of offsets may name rows more than once, more of them than this CTA's shared
     // memory is laid out for: then every row is read once and asked for its owner (look_up).
     int rows = (int)p.M;
-    if (!kArg && p.table) rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, warp_tot, kWarps, nullptr);
-    const bool table = !kArg && p.table && rows <= (int)p.M;
+    if (kSkip && p.table) rows = stream::count_rows(p.tok_off, p.skip, p.B, p.M, act, warp_tot, kWarps, nullptr);
+    const bool table = kSkip && p.table && rows <= (int)p.M;
     if (!table) rows = (int)p.M;
     const int here = cl < rows ? (rows - cl + nc - 1) / nc : 0;
     cluster_wait();          // all CTAs of the cluster run: their shared memory may be written
@@ -84,7 +101,6 @@ __global__ void __launch_bounds__(kThreads, direct::kCtasPerSm) rows_whole(const
     // way: where spans do not fill the last round it has the fewest.
     auto look_up = [&]() {
         if (warp != kWarps - 1) return;
-        int ordered = -1;        // 1: the offsets never fall, so that a row's owner is where the search looks
         for (int k0 = 0; (k0 << clog) + rank < here; k0 += 32) {
             const bool mine = ((k0 + lane) << clog) + rank < here;
             const int k = mine ? k0 + lane : k0;
@@ -93,24 +109,13 @@ __global__ void __launch_bounds__(kThreads, direct::kCtasPerSm) rows_whole(const
             float x = -INFINITY;
             if (id >= 0 && id < e.V) x = Elem<T>::load(p.logits + (int64_t)row * p.row_pitch + id * ES);
             // rows of no sound utterance that is read are left alone; those of the table all have one
-            const int at = table ? 0 : utterance_of_row(p.tok_off, p.B, row);
-            auto owns = [&](int b) {
-                const int64_t i0 = p.tok_off[b], i1 = p.tok_off[b + 1];
-                return ranges::rows_sound(i0, i1, p.M) && i0 <= row && row < i1 && !(p.skip && p.skip[b]);
-            };
-            bool wanted = table || owns(at);
-            // Asking every utterance for each row that none has -- behind the last one's rows, or in front of
-            // the first one's -- took 174 us for 4,000 rows of 8 KB of which 2,000 utterances have half (15
-            // now; 20 with a closing kernel): only where the offsets fall somewhere.
-            if (ordered != 1 && __any_sync(0xffffffffu, !wanted)) {
-                if (ordered < 0) ordered = stream::offsets_ordered(p.tok_off, p.B);
-                for (int b = 0; !ordered && !wanted && b < p.B; ++b) wanted = owns(b);
-            }
+            bool wanted = table || owns(p.tok_off, p.skip, p.M, utterance_of_row(p.tok_off, p.B, row), row);
+            if (__any_sync(0xffffffffu, !wanted)) wanted |= owned_elsewhere<T, kSkip>(p.tok_off, p.skip, p.B, p.M, row);
             if (mine) drafts[k] = make_float2(x, wanted ? 1.f : 0.f);
         }
     };
     const int first = (warp << clog) + rank;
-    direct::stream_spans<T, kF, kArg, 1 + kEnd>(
+    direct::stream_spans<T, kF, kArg, 1 + kEnd + 2 * kSkip>(
         p, cut, Deal{(unsigned)first, (unsigned)(kWarps << clog), here, cl, nc, table, true}, act,
         [&] { if (!kArg) look_up(); },
         [&](int, int a, int sp, const SpanResult &out) {
